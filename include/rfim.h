@@ -318,7 +318,7 @@ int rfim_profile_read(rfim_ctx *ctx, double *sweep_ms, int64_t *sweep_launches, 
 /* Launch-shape tuner for the bit layout.  Times every instantiated launch shape (cluster size S
    = z slabs per replica group, replicas G per cluster, replicas GT per thread, threads per CTA;
    S = 0 is the grid-wide cooperative plan with one CTA per SM, G replicas per (group, z plane)
-   unit) on a scratch realization with this L, R and field kind (20-50 exchange intervals of 10
+   unit; the shapes ending in "r" or "m" are the resident plan's, see rfim_get_plan) on a scratch realization with this L, R and field kind (20-50 exchange intervals of 10
    sweeps each, CUDA-event timing) and remembers the fastest: later rfim_create calls in this
    process with the same L, R_capacity and field kind use it.  plan_out (optional, plan_cap chars)
    receives "S,G,GT,threads"; *attempts_per_ns (optional) the best rate.  Synchronous; allocates
@@ -326,8 +326,10 @@ int rfim_profile_read(rfim_ctx *ctx, double *sweep_ms, int64_t *sweep_launches, 
 int rfim_tune(int32_t L, int32_t R, int32_t field_kind, char *plan_out, int32_t plan_cap, double *attempts_per_ns);
 
 /* Launch shape of this context's sweep kernel, in the format rfim_tune reports: "S,G,GT,threads"
-   with ",4" appended when every word is split over four warps (S = 0: the grid-wide plan), and
-   ",int8" appended when the int8 layout is staged as bits; "" when the context runs the int8
+   with ",4" appended when every word is split over four warps (S = 0: the grid-wide plan), or
+   "S,G,NB,threads,r" for the resident plan of small realizations (a cluster of S slabs holds G replicas
+   for up to 512 exchange intervals per launch, NB Philox blocks of a word per thread item; "m" instead
+   of "r" when a thread runs several items), and ",int8" appended when the int8 layout is staged as bits; "" when the context runs the int8
    kernels (L outside 8, 16, 32, 64).  plan_out receives at most plan_cap chars (NUL included).
    Errors: RFIM_EINVAL (NULL ctx or plan_out, plan_cap < 1). */
 int rfim_get_plan(const rfim_ctx *ctx, char *plan_out, int32_t plan_cap);

@@ -116,6 +116,10 @@ GridFn grid_kernel_for(int L, int G, int GT, int threads, bool bim, bool i8) {
   return nullptr;
 }
 
+// L = 64: largest replica capacity that can take the resident plan by default (36 clusters of four
+// slabs fit at one CTA per SM, two replicas each; three are slower than the grid-wide plan).
+constexpr int32_t kResidentMaxR64 = 72;
+
 constexpr size_t kGridMinSmem = 116 * 1024;  // more than half an SM's shared memory: one CTA per SM
 
 // Partition of the current R over the CTAs of a grid-wide launch.
@@ -225,7 +229,7 @@ MultiHit make_multihit(int32_t L, int32_t mh, int32_t tile) {
 }
 
 cudaError_t prepare_multihit(const BitsPlan &plan, bool bimodal) {
-  if (plan.S == 0) return cudaErrorInvalidConfiguration;
+  if (plan.S == 0 || plan.resident()) return cudaErrorInvalidConfiguration;
   for (int T : {8, 16, 32}) {
     if (!multihit_tile_ok(plan.L, T)) continue;
     MhFn fn = mh_kernel_for(plan.L, plan.S, plan.GT, plan.threads, bimodal, T);
@@ -251,14 +255,33 @@ void remember_tuned_plan(int32_t L, int32_t R, bool bimodal, const std::string &
   g_tuned[{L, R, bimodal}] = plan;
 }
 
-std::vector<std::string> plan_candidates(int32_t L) {
+std::string plan_name(const BitsPlan &p) {
+  char buf[64];
+  if (p.resident())
+    snprintf(buf, sizeof buf, "%d,%d,%d,%d,%c%s", p.res.S, p.res.G, p.res.NB, p.res.threads, p.res.one ? 'r' : 'm',
+             p.i8 ? ",int8" : "");
+  else
+    snprintf(buf, sizeof buf, "%d,%d,%d,%d%s%s", p.S, p.G, p.GT, p.threads, p.NS == 4 ? ",4" : "", p.i8 ? ",int8" : "");
+  return buf;
+}
+
+std::vector<std::string> plan_candidates(int32_t L, int32_t R, bool bimodal) {
+  std::vector<std::string> c;
   if (L == 64)
-    return {"4,4,4,512", "0,4,4,512", "0,4,1,512", "4,4,2,512", "2,2,2,512", "4,4,4,1024", "1,1,1,1024"};
-  if (L == 32)
-    return {"2,1,1,256", "4,1,1,128", "1,1,1,512", "1,2,2,512", "2,1,1,512", "0,4,4,512", "0,4,1,512",
-            "2,1,1,1024,4", "2,1,1,512,4", "4,1,1,512,4"};
-  if (L == 16) return {"1,8,1,512", "1,4,1,512", "1,16,1,512", "1,8,1,1024,4", "1,4,1,512,4", "1,8,1,512,4"};
-  return {"1,16,1,128", "1,16,1,512", "1,8,1,128", "1,16,1,512,4", "1,8,1,256,4"};
+    c = {"4,4,4,512", "0,4,4,512", "0,4,1,512", "4,4,2,512", "2,2,2,512", "4,4,4,1024", "1,1,1,1024"};
+  else if (L == 32)
+    c = {"2,1,1,256", "4,1,1,128", "1,1,1,512", "1,2,2,512", "2,1,1,512", "0,4,4,512", "0,4,1,512",
+         "2,1,1,1024,4", "2,1,1,512,4", "4,1,1,512,4"};
+  else if (L == 16)
+    c = {"1,8,1,512", "1,4,1,512", "1,16,1,512", "1,8,1,1024,4", "1,4,1,512,4", "1,8,1,512,4"};
+  else
+    c = {"1,16,1,128", "1,16,1,512", "1,8,1,128", "1,16,1,512,4", "1,8,1,256,4"};
+  for (const ResidentShape &s : resident_shapes(L, R, bimodal)) {
+    BitsPlan p;
+    p.res = s;
+    c.push_back(plan_name(p));
+  }
+  return c;
 }
 
 int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::string *err, bool i8) {
@@ -316,6 +339,19 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
   } else {
     p.S = 1; p.G = 4; p.GT = 1; p.threads = 512; p.NS = 4;  // C1: 3.1 against 1.5
   }
+  // the resident plan where all its CTAs fit at once; at L = 64 where its estimate beats the grid-wide
+  // plan's half-sweep of about 5.2 us + 0.76 us per unit of the fullest CTA (measured, Gaussian field,
+  // half-sweep resident / grid: R = 4 1.2 / -, 12 2.8 / 7.6, 16 5.2 / 8.5, 36 5.2 / 8.4, 48 10.1 / 10.0,
+  // 64 10.1 / 11.7, 70 10.1 / 11.5, 80 15.0 / 13.0 us), and not for the staged int8 layout
+  ResidentShape rs;
+  bool resident = false;
+  double cycles = 0.0;
+  if (L < 64) {
+    resident = resident_shape(L, Rcap, bimodal, &rs, &cycles);
+  } else if (!i8 && sms_dev > 0 && Rcap <= kResidentMaxR64) {
+    const int units = ((Rcap + 3) / 4 * L + sms_dev - 1) / sms_dev;
+    resident = resident_shape(L, Rcap, bimodal, &rs, &cycles) && cycles < 2070.0 * (5.2 + 0.76 * std::max(units, 3));
+  }
   // "S,G,GT,threads": the tuner's current candidate, else a tuned shape for this (L, R, field),
   // else the RFIM_BITS_PLAN environment override, else the defaults above
   std::string tuned;
@@ -327,28 +363,43 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
   const char *o = t_plan_override ? t_plan_override : (!tuned.empty() ? tuned.c_str() : getenv("RFIM_BITS_PLAN"));
   if (o) {
     int s, g, gt, th, ns = 1;
-    // "S,G,GT,threads[,NS]" (NS = 4: every word split over four warps); an override that names no
+    ResidentShape named_rs;
+    char suffix = 0;
+    const bool is_res = sscanf(o, "%d,%d,%d,%d,%c", &named_rs.S, &named_rs.G, &named_rs.NB, &named_rs.threads, &suffix) == 5 &&
+                        (suffix == 'r' || suffix == 'm');
+    named_rs.one = suffix == 'r';
+    // "S,G,NB,threads,r" (or m: several items per thread): a resident shape; "S,G,GT,threads[,NS]" (NS = 4: every word split over four warps); an override that names no
     // instance for this L (e.g. an L=64 shape while building L=16) is ignored and the defaults stand
-    const int nf = sscanf(o, "%d,%d,%d,%d,%d", &s, &g, &gt, &th, &ns);
+    const int nf = is_res ? 0 : sscanf(o, "%d,%d,%d,%d,%d", &s, &g, &gt, &th, &ns);
     const bool named = nf == 4 || nf == 5;
+    if (is_res && resident_fits(L, Rcap, bimodal, &named_rs)) {
+      rs = named_rs;
+      resident = true;
+    }
     if (nf == 4) ns = 1;
     const bool exists = named && (s == 0 ? (ns == 1 && th >= 256 && th <= 1024 && th % 32 == 0 &&
                                             grid_kernel_for(L, g, gt, th, bimodal, i8))
                                          : kernel_for(L, s, gt, th, bimodal, i8, ns) != nullptr);
     if (exists) {
       p.S = s; p.G = g; p.GT = gt; p.threads = th; p.NS = ns;
+      resident = false;
     }
   }
-  if (p.S != 0) {
+  if (resident) {
+    p.S = rs.S; p.G = rs.G; p.GT = 1; p.threads = rs.threads; p.NS = 1;
+    p.res = rs;
+    p.smem = rs.smem;
+  }
+  if (p.S != 0 && !resident) {
     if (p.G > Rcap) p.G = Rcap;
     if (p.GT > p.G) p.GT = 1;
     if (p.G % p.GT) p.G = (p.G / p.GT) * p.GT;
   }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-  KernelFn fn = p.S == 0 ? nullptr : kernel_for(L, p.S, p.GT, p.threads, bimodal, i8, p.NS);
+  KernelFn fn = p.S == 0 || resident ? nullptr : kernel_for(L, p.S, p.GT, p.threads, bimodal, i8, p.NS);
   GridFn gfn = p.S == 0 && p.threads >= 256 && p.threads <= 1024 ? grid_kernel_for(L, p.G, p.GT, p.threads, bimodal, i8) : nullptr;
-  if (!fn && !gfn) {
+  if (!fn && !gfn && !resident) {
     if (err) *err = "no bit-layout kernel instance for this plan";
     return -1;  // RFIM_EINVAL
   }
@@ -366,15 +417,15 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
     }
     p.smem = grid_smem(L, p.G, maxu, Rcap);
   }
-  if (!gfn)
+  if (fn)
     p.smem = (size_t)p.G * 2 * words_per_cta(L, p.S) * 4 + tab_bytes(p.G);
   if (p.smem > 227 * 1024) {
     if (err) *err = "bit-layout plan exceeds shared memory";
     return -1;
   }
   const void *fptr = gfn ? (const void *)gfn : (const void *)fn;
-  cudaError_t e = raise_smem_limit(fptr, p.smem);
-  if (e == cudaSuccess && p.S > 1)
+  cudaError_t e = fptr ? raise_smem_limit(fptr, p.smem) : cudaSuccess;  // resident_fits has raised its own
+  if (e == cudaSuccess && fn && p.S > 1)
     e = cudaFuncSetAttribute(fptr, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) {
     if (err) *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e);
@@ -413,6 +464,9 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
     // int8 layout: the published end planes (halos) in the bit layout
     if (!rc && i8) rc = grab((void **)&p.gbits, (size_t)Rcap * 2 * ((size_t)L * L * L / 64) * 4, "halo words");
   }
+  const size_t rec_bytes = resident ? 2 * parts * sizeof(uint4) : 0;
+  if (!rc && resident) rc = grab((void **)&p.rec, rec_bytes, "energy records");
+  if (!rc && p.rec && cudaMemset(p.rec, 0, rec_bytes) != cudaSuccess) rc = -3;
   if (!rc && cudaMemset(p.counter, 0, 16) != cudaSuccess) rc = -3;
   if (!rc && p.prog && cudaMemset(p.prog, 0, (size_t)std::max(sms, 1) * 4) != cudaSuccess) rc = -3;
   if (rc) {
@@ -427,7 +481,7 @@ bool bits_plan_fits(const BitsPlan &plan, int32_t R) { return R <= plan.Rcap; }
 
 void free_bits_plan(BitsPlan &plan) {
   void *ptrs[] = {plan.field4, plan.flimb, plan.fquant, plan.partB, plan.partM, plan.partFi, plan.partF,
-                  plan.counter, plan.gpartB, plan.gpartM, plan.gpartFi, plan.gpartF, plan.prog, plan.gbits};
+                  plan.counter, plan.gpartB, plan.gpartM, plan.gpartFi, plan.gpartF, plan.prog, plan.gbits, plan.rec};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   plan.field4 = nullptr;
@@ -440,6 +494,22 @@ void free_bits_plan(BitsPlan &plan) {
   plan.gpartF = nullptr;
   plan.prog = nullptr;
   plan.gbits = nullptr;
+  plan.rec = nullptr;
+}
+
+cudaError_t reset_bits_plan(const BitsPlan &plan, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  if (plan.prog) {
+    e = cudaMemsetAsync(plan.prog, 0, (size_t)std::max(plan.sms, 1) * 4, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(plan.counter + 2, 0, 4, st);
+    plan.prog_base = 0;
+    plan.arrive_base = 0;
+  }
+  if (e == cudaSuccess && plan.rec) {
+    e = cudaMemsetAsync(plan.rec, 0, 2 * (size_t)plan.Rcap * plan.S * sizeof(uint4), st);
+    plan.epoch = 0;
+  }
+  return e;
 }
 
 cudaError_t build_field4(const RealView &v, BitsPlan &plan, cudaStream_t st) {
@@ -474,6 +544,23 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
   xa.err = plan.counter + 1;
   xa.flimb = plan.flimb;
   xa.fquant = plan.fquant;
+  if (plan.resident()) {
+    if ((mh && mh->mh > 0) || n_intervals < 1 || (!exchange && n_intervals != 1)) return cudaErrorInvalidValue;
+    if (exchange && plan.epoch >= kRecordEpochs - 1 - (uint32_t)n_intervals) {  // numbers would wrap: start again
+      const cudaError_t e = reset_bits_plan(plan, st);
+      if (e != cudaSuccess) return e;
+    }
+    ResidentArgs ra{};
+    ra.G = plan.res.G;
+    ra.rcap = plan.Rcap;
+    ra.n_iv = n_intervals;
+    ra.epoch0 = plan.epoch + 1;
+    ra.rec = plan.rec;
+    ra.i8 = plan.i8;
+    const cudaError_t e = launch_resident(v, plan.res, ra, sweep0, n_sweeps, plan.field4, xa, st);
+    if (e == cudaSuccess && exchange) plan.epoch += (uint32_t)n_intervals;
+    return e;
+  }
   if (plan.S == 0) {
     GridFn gfn = grid_kernel_for(plan.L, plan.G, plan.GT, plan.threads, v.kind == kBimodal, plan.i8);
     if (!gfn || (plan.i8 && !plan.gbits)) return cudaErrorInvalidConfiguration;

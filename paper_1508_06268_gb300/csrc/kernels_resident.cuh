@@ -1,0 +1,491 @@
+// Resident sweep of small realizations: every lattice stays in shared memory for many exchange
+// intervals of one launch.
+//
+// Bound: latency.  A half-sweep of a small realization (L = 8, R = 16: 1024 Philox blocks; L = 32,
+// R = 70: 286720) is a few hundred cycles of work per SM, so what counts is the chain from one
+// half-sweep to the next and the exchange step, not the rate of the decisions.  Therefore
+//   - a cluster of S CTAs (z slabs) holds G replicas, with S and G chosen so that all CTAs are
+//     resident at once and spread over the SMs (resident_shape); a launch runs up to
+//     kResidentIntervals intervals;
+//   - an item is NB of the 8 Philox blocks of a 32-site word of one replica; the NP = 8 / NB items of a
+//     word xor their flips into it.  ONE: every thread has one item for the whole launch, and all
+//     that depends on it alone (neighbour addresses, field values, the products of the first two
+//     Philox rounds that hold the block index) is formed once and stays in registers;
+//   - the random words do not depend on the spins: S = 1 forms those of the next half-sweep in the
+//     same straight-line code as the decisions of this one, so that the two dependent chains fill
+//     each other's latencies; S > 1 forms them while the halos are on their way;
+//   - slabs push their end planes into the neighbours' halo planes with st.async, which counts the
+//     bytes into the neighbour's mbarrier: the data is its own signal.  (A cluster barrier with
+//     release semantics per half-sweep instead stalls on the memory barrier it implies: a fifth of
+//     the issue slots at L = 32, R = 70.)
+//   - the exchange step gathers the energies as records (exchange_records.cuh) instead of one
+//     launch per interval with an arrival counter and a last CTA that takes the step alone, and
+//     the measurement of temperature k is added by CTA k mod P.
+#pragma once
+#include <cstdint>
+
+#include "exchange_records.cuh"
+#include "kernels_bits.cuh"
+
+namespace rfim {
+
+// Round keys of the realization's Philox streams (operands from the constant bank: no key adds).
+struct PhiloxKeys {
+  uint32_t k0[10], k1[10];
+};
+
+struct ResidentArgs {
+  PhiloxKeys keys;
+  int32_t G;        // replicas per cluster
+  int32_t rcap;     // replica capacity
+  int32_t n_iv;     // exchange intervals in this launch
+  uint32_t epoch0;  // interval number of this launch's first interval
+  uint4 *rec;       // [2][rcap * S] energy records
+  int32_t i8;       // the realization is stored as bytes (v.spins8) and staged as bits
+  int32_t lw;       // log2 of the words whose items of one part are neighbouring threads (ONE; else 5)
+};
+
+// Copy of the exchange state each CTA keeps, one entry per replica or temperature.
+struct ResidentState {
+  double *E, *beta;
+  int32_t *M, *t2r, *r2t;
+  uint8_t *swapped;
+};
+
+__host__ __device__ constexpr size_t resident_state_bytes(int rcap) { return (size_t)rcap * 29 + 32; }
+
+// Planes of a slab in shared memory: with S > 1 a halo plane before and after the slab's own.
+template <int L, int S>
+__host__ __device__ constexpr int resident_planes() { return L / S + (S > 1 ? 2 : 0); }
+
+// 32-word chunks (L = 8: 16-word ones, a replica) the energy reduction of a slab is cut into.
+template <int L, int S>
+__host__ __device__ constexpr int resident_chunks() {
+  return 2 * (L / S) * (L * L / 64) >= 32 ? 2 * (L / S) * (L * L / 64) / 32 : 1;
+}
+
+constexpr unsigned kMbarSpinLimit = 1u << 20;
+
+struct alignas(16) ChunkSum {
+  int B, M;
+  long long F;
+};
+
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// Bounded wait for the phase of parity `par` of an mbarrier of this CTA.
+__device__ __forceinline__ void mbar_wait(uint32_t mbar, uint32_t par, unsigned *err) {
+  for (unsigned it = 0; it < kMbarSpinLimit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(mbar), "r"(par)
+        : "memory");
+    if (done) return;
+    if ((it & 63u) == 63u && *(volatile unsigned *)err) return;
+  }
+  atomicOr(err, 2u);
+}
+
+// What the words of Philox blocks of one thread need besides the replica and the sweep: the products
+// of the first two rounds that hold only the block index and the colour.
+template <int NB>
+struct BlockParts {
+  uint32_t lo[NB];      // low half of M0 * block
+  uint64_t q[2][NB];    // per colour: M1 * (high half of M0 * block ^ tag ^ k1[0])
+};
+
+// Words of the NB blocks for sweep and colour c: rounds 0 and 1 from the parts, then eight rounds.
+template <int NB>
+__device__ __forceinline__ void philox_words(const PhiloxKeys &k, const BlockParts<NB> &bp, int c, uint32_t r, uint32_t sweep,
+                                             Words4 (&w)[NB]) {
+  const uint64_t s = (uint64_t)kPhiloxM1 * sweep;
+  const uint64_t p = (uint64_t)kPhiloxM0 * ((uint32_t)(s >> 32) ^ r ^ k.k0[0]);
+#pragma unroll
+  for (int j = 0; j < NB; ++j) {
+    uint32_t c0 = (uint32_t)(bp.q[c][j] >> 32) ^ (uint32_t)s ^ k.k0[1], c1 = (uint32_t)bp.q[c][j];
+    uint32_t c2 = (uint32_t)(p >> 32) ^ bp.lo[j] ^ k.k1[1], c3 = (uint32_t)p;
+#pragma unroll
+    for (int i = 2; i < 10; ++i) {
+      const uint64_t p0 = (uint64_t)kPhiloxM0 * c0, p1 = (uint64_t)kPhiloxM1 * c2;
+      c0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.k0[i];
+      c2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.k1[i];
+      c1 = (uint32_t)p1;
+      c3 = (uint32_t)p0;
+    }
+    w[j].w[0] = c0;
+    w[j].w[1] = c1;
+    w[j].w[2] = c2;
+    w[j].w[3] = c3;
+  }
+}
+
+template <int NB>
+__device__ __forceinline__ BlockParts<NB> block_parts(const PhiloxKeys &k, uint32_t stage, uint32_t block0) {
+  BlockParts<NB> bp;
+#pragma unroll
+  for (int j = 0; j < NB; ++j) {
+    const uint64_t p = (uint64_t)kPhiloxM0 * (block0 + (uint32_t)j);
+    bp.lo[j] = (uint32_t)p;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      bp.q[c][j] = (uint64_t)kPhiloxM1 * ((uint32_t)(p >> 32) ^ tag_word(kTagMetro, stage, (uint32_t)c) ^ k.k1[0]);
+  }
+  return bp;
+}
+
+// One item: word iw of plane zl of replica g of the slab, blocks sh .. sh + NB - 1 of it.
+template <int NB>
+struct ResidentItem {
+  int g, z, sh;
+  int64_t wq;                     // word within its colour
+  int same, next, prev, up, down; // word indices in the replica's colour-0 planes
+  uint32_t p0;                    // row-parity mask of colour 0 (colour 1: its complement)
+};
+
+template <int L, int S, int NB, bool BIM, int NT, bool ONE>
+__global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_constant__ ResidentArgs ra, uint32_t sweep0,
+                                                 int32_t nsw, const float4 *__restrict__ field4, const ExchArgs xa) {
+  using Gm = BitsGeom<L>;
+  constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P, NP = 8 / NB;
+  constexpr int CW = resident_planes<L, S>() * P;  // words of one colour of one replica, halos included
+  constexpr int Z1 = S > 1 ? 1 : 0;                // the slab's first own plane
+  constexpr int64_t WPAD = (W + 31) / 32 * 32;
+  constexpr int SEG = 2 * WC < 32 ? 2 * WC : 32, NCH = resident_chunks<L, S>();
+  static_assert(2 * WC >= 16, "a slab of one replica fills at least half a warp");
+  static_assert(S == 1 || P % 4 == 0, "halo planes are pushed 16 bytes at a time");
+  extern __shared__ __align__(16) uint32_t sm[];
+  __shared__ __align__(8) uint64_t mbar[2];  // halos pushed after even / odd half-sweeps
+  const int rank = S > 1 ? (int)cluster_rank() : 0;
+  const int z0 = rank * PZ, r0 = (int)(blockIdx.x / S) * ra.G, gact = min(ra.G, v.R - r0);
+  const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  const int R = v.R;
+
+  uint32_t *sp = sm;                            // [G][2][CW]
+  uint32_t *tab = sm + (size_t)ra.G * 2 * CW;   // G decision-table slots
+  const uint32_t slot0 = tab_slot0(tab);
+  ChunkSum *red = reinterpret_cast<ChunkSum *>(reinterpret_cast<char *>(tab) + tab_bytes(ra.G));  // [G][NCH]
+  ResidentState xs;
+  xs.E = reinterpret_cast<double *>(red + (size_t)ra.G * NCH);
+  xs.beta = xs.E + ra.rcap;
+  xs.M = reinterpret_cast<int32_t *>(xs.beta + ra.rcap);
+  xs.t2r = xs.M + ra.rcap;
+  xs.r2t = xs.t2r + ra.rcap;
+  xs.swapped = reinterpret_cast<uint8_t *>(xs.r2t + ra.rcap);
+
+  // debug build: the replica range, the shared-memory plan and the cluster must be the launch's
+  const bool ok = RFIM_DCHECK(xa.err, gact >= 1 && gact <= ra.G && r0 + gact <= R && R <= ra.rcap, kDbgGlobal) &&
+                  RFIM_DCHECK(xa.err, (uint32_t)__cvta_generic_to_shared(xs.swapped + ra.rcap) <=
+                                          (uint32_t)__cvta_generic_to_shared(sm) + dyn_smem_bytes(),
+                              kDbgTable) &&
+                  RFIM_DCHECK(xa.err, S == 1 || cluster_ctas() == (uint32_t)S, kDbgRank);
+  // the slab with its halo planes (the halos of colour 0 are pushed before they are needed)
+  for (int t = tid; ok && t < gact * 2 * CW; t += nt) {
+    const int g = t / (2 * CW), rem = t % (2 * CW), c = rem / CW, pl = rem % CW / P, iw = rem % P;
+    const int z = (z0 + pl - Z1 + L) % L;
+    const int64_t gw = ((int64_t)(r0 + g) * 2 + c) * W + (int64_t)z * P + iw;
+    sp[t] = ra.i8 ? pack_int8_word(v.spins8 + 32 * gw) : v.bits[gw];
+  }
+  if (ok) tab_fill<BIM>(v, tab, slot0, gact, [&](int g) { return r0 + g; });
+  if (xa.enabled && ok)
+    for (int r = tid; r < R; r += nt) {
+      xs.t2r[r] = v.t2r[r];
+      xs.r2t[r] = v.r2t[r];
+      xs.beta[r] = v.beta_d[r];
+    }
+  const bool limbs = !BIM && xa.flimb != nullptr;
+  const double fscale = limbs ? ldexp(1.0, xa.fquant->qe) : 1.0;
+  const long long Htot = limbs ? xa.fquant->Htot : 0;
+  const uint32_t mbar0 = (uint32_t)__cvta_generic_to_shared(mbar);
+  if (S > 1) {
+    if (tid == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;" ::"r"(mbar0),
+                   "r"(mbar0 + 8)
+                   : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    sync_slabs<S>();  // every CTA's mbarriers are ready before the first push
+  } else {
+    __syncthreads();
+  }
+
+  const int words = ok ? gact * WC : 0;
+  auto decode = [&](int item, int lw, bool *valid) {
+    ResidentItem<NB> it;
+    const int fw = ((item >> lw) / NP << lw) + (item & ((1 << lw) - 1));
+    *valid = fw < words;
+    const int f = *valid ? fw : 0;  // a thread without an item repeats the first one and drops its flips
+    it.sh = (item >> lw) % NP * NB;
+    it.g = f / WC;
+    const int wl = f % WC, zl = wl / P, iw = wl % P;
+    it.z = z0 + zl;
+    it.wq = (int64_t)it.z * P + iw;
+    const int base = it.g * 2 * CW, pl = base + (zl + Z1) * P;
+    it.same = pl + iw;
+    it.next = pl + (iw + 1) % P;
+    it.prev = pl + (iw + P - 1) % P;
+    it.up = S > 1 ? it.same + P : base + (zl + 1) % L * P + iw;
+    it.down = S > 1 ? it.same - P : base + (zl + L - 1) % L * P + iw;
+    it.p0 = parity0_mask<L>(0, it.z, iw);
+    return it;
+  };
+  auto field_of = [&](const ResidentItem<NB> &it, int c, float4 (&h)[NB]) {
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+      h[j] = BIM ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(field4 + field4_index(c, it.wq, it.sh + j, WPAD));
+  };
+  auto field_bits = [&](const ResidentItem<NB> &it, int c) { return BIM ? v.hbits[(int64_t)c * W + it.wq] >> it.sh : 0u; };
+  // decisions of one item of colour c from its random words, xored into its word
+  auto update = [&](const ResidentItem<NB> &it, int c, const Words4 (&w)[NB], const float4 (&h)[NB], uint32_t fb, bool valid) {
+    const uint32_t *O = sp + (c ^ 1) * CW;
+    uint32_t A, B, C, D, c0, c1, c2;
+    nb_xy<L>(O[it.same], O[it.next], O[it.prev], c ? ~it.p0 : it.p0, A, B, C, D);
+    count6(A, B, C, D, O[it.up], O[it.down], c0, c1, c2);
+    uint32_t *self = sp + c * CW + it.same;
+    const PairSlices ps = make_pairs(c0 >> it.sh, c1 >> it.sh, c2 >> it.sh, *self >> it.sh, fb);
+    const uint32_t slot = slot0 + (uint32_t)it.g * kTabSlot;
+    uint32_t flip = 0u, fk[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int j = NB - 1; j >= 0; --j) decide_block<BIM>(w[j], ps, j, slot, h[j], flip, fk);
+    if (!BIM) flip = fk[0] | (fk[1] << 8) | (fk[2] << 16) | (fk[3] << 24);
+    if (valid) atomicXor(self, flip << it.sh);
+  };
+  // After half-sweep number h of this launch (all of the CTA's updates of colour c done): the slab's
+  // first and last planes into the halo planes of the slabs below and above.  Two mbarriers in turn:
+  // a neighbour can push half-sweep h + 2 only after it has this slab's push of h + 1, which
+  // follows this slab's wait for h.
+  auto push_halos = [&](int c, uint32_t h) {
+    const uint32_t bar = mbar0 + 8 * (h & 1u);
+    constexpr int VEC = P >= 4 ? P / 4 : 1;
+    if (tid == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)(gact * 2 * P * 4))
+                   : "memory");
+    for (int t = tid; t < gact * 2 * VEC; t += nt) {
+      const int g = t / (2 * VEC), side = t / VEC & 1, q = t % VEC * 4;
+      const uint32_t peer = (uint32_t)(rank + (side ? 1 : S - 1)) % S;
+      const int from = (g * 2 + c) * CW + (side ? PZ : 1) * P + q, to = (g * 2 + c) * CW + (side ? 0 : PZ + 1) * P + q;
+      const uint4 x = *reinterpret_cast<const uint4 *>(sp + from);
+      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                       mapa_shared((uint32_t)__cvta_generic_to_shared(sp + to), peer)),
+                   "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(mapa_shared(bar, peer))
+                   : "memory");
+    }
+  };
+  auto wait_halos = [&](uint32_t h) { mbar_wait(mbar0 + 8 * (h & 1u), (h >> 1) & 1u, xa.err); };
+
+  bool valid;
+  const ResidentItem<NB> own = decode(tid, ONE ? ra.lw : 5, &valid);
+  BlockParts<NB> bp;
+  float4 hown[2][NB];
+  uint32_t fbown[2] = {0u, 0u};
+  Words4 w[NB];
+  if (ONE) {
+    bp = block_parts<NB>(ra.keys, v.stage, (uint32_t)(8 * own.wq + own.sh));
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (NB <= 2) field_of(own, c, hown[c]);
+      fbown[c] = field_bits(own, c);
+    }
+    if (S == 1) philox_words<NB>(ra.keys, bp, 0, (uint32_t)(r0 + own.g), sweep0, w);
+  }
+
+  const int n_iv = xa.enabled ? ra.n_iv : 1;
+  uint32_t h = 0, sweep = sweep0;  // half-sweeps done in this launch; current sweep
+  for (int iv = 0; iv < n_iv; ++iv) {
+#pragma unroll 1
+    for (int s = 0; s < nsw; ++s, ++sweep) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        if (ONE && S == 1) {
+          if (NB > 2) field_of(own, c, hown[c]);
+          Words4 next[NB];
+          philox_words<NB>(ra.keys, bp, c ^ 1, (uint32_t)(r0 + own.g), sweep + (uint32_t)c, next);
+          update(own, c, w, hown[c], fbown[c], valid);
+#pragma unroll
+          for (int j = 0; j < NB; ++j) w[j] = next[j];
+          __syncthreads();
+        } else if (ONE) {
+          if (NB > 2) field_of(own, c, hown[c]);
+          philox_words<NB>(ra.keys, bp, c, (uint32_t)(r0 + own.g), sweep, w);
+          if (h > 0) wait_halos(h - 1);
+          update(own, c, w, hown[c], fbown[c], valid);
+          __syncthreads();
+          push_halos(c, h);
+        } else {
+          for (int item = tid; item < (words + 31) / 32 * 32 * NP; item += nt) {
+            bool in;
+            const ResidentItem<NB> it = decode(item, 5, &in);
+            float4 hf[NB];
+            field_of(it, c, hf);
+            const uint32_t fb = field_bits(it, c);
+            bp = block_parts<NB>(ra.keys, v.stage, (uint32_t)(8 * it.wq + it.sh));
+            philox_words<NB>(ra.keys, bp, c, (uint32_t)(r0 + it.g), sweep, w);
+            if (S > 1 && item == tid && h > 0) wait_halos(h - 1);
+            update(it, c, w, hf, fb, in);
+          }
+          __syncthreads();
+          if (S > 1) push_halos(c, h);
+        }
+        ++h;
+      }
+    }
+    if (S > 1 && h > 0) wait_halos(h - 1);
+    if (!xa.enabled) break;
+
+    // ---- energies (Eq. 1) of this slab's replicas, one ChunkSum per SEG words --------------------
+    for (int e = tid; e < (gact * 2 * WC + 31) / 32 * 32; e += nt) {
+      int b = 0, m = 0;
+      unsigned hu[4] = {0u, 0u, 0u, 0u};
+      int hsum = 0;
+      if (ok && e < gact * 2 * WC) {
+        const int g = e / (2 * WC), c = e / WC & 1, wl = e % WC, zl = wl / P, iw = wl % P, z = z0 + zl;
+        const int64_t wq = (int64_t)z * P + iw;
+        const uint32_t *O = sp + (g * 2 + 1) * CW + Z1 * P;  // colour 1, the slab's own planes
+        const uint32_t self = sp[(g * 2 + c) * CW + Z1 * P + wl];
+        m = 2 * __popc(self) - 32;
+        if (c == 0) {
+          uint32_t A, B, C, D;
+          nb_xy<L>(O[wl], O[zl * P + (iw + 1) % P], O[zl * P + (iw + P - 1) % P], parity0_mask<L>(0, z, iw), A, B, C, D);
+          const uint32_t U = S > 1 ? O[wl + P] : O[(zl + 1) % L * P + iw];
+          const uint32_t V = S > 1 ? O[wl - P] : O[(zl + L - 1) % L * P + iw];
+          b = 192 - 2 * (__popc(self ^ A) + __popc(self ^ B) + __popc(self ^ C) + __popc(self ^ D) + __popc(self ^ U) +
+                         __popc(self ^ V));
+        }
+        if (BIM) {
+          hsum = 32 - 2 * __popc(self ^ v.hbits[(int64_t)c * W + wq]);
+        } else {
+          const uint4 top0 = __ldg(xa.flimb + flimb_index(c, wq, 8, WPAD));
+          const uint4 top1 = __ldg(xa.flimb + flimb_index(c, wq, 9, WPAD));
+          const uint32_t top[8] = {top0.x, top0.y, top0.z, top0.w, top1.x, top1.y, top1.z, top1.w};
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint4 lo = __ldg(xa.flimb + flimb_index(c, wq, j, WPAD));
+            const uint32_t up = (self >> j) & 0x01010101u;
+            hu[0] = __dp4a(up, lo.x, hu[0]);
+            hu[1] = __dp4a(up, lo.y, hu[1]);
+            hu[2] = __dp4a(up, lo.z, hu[2]);
+            hu[3] = __dp4a(up, lo.w, hu[3]);
+            hsum = __dp4a((int)up, (int)top[j], hsum);
+          }
+        }
+      }
+      ChunkSum s;
+      if (SEG == 32) {
+        s.B = __reduce_add_sync(0xffffffffu, b);
+        s.M = __reduce_add_sync(0xffffffffu, m);
+        s.F = __reduce_add_sync(0xffffffffu, hsum);
+        if (!BIM) {
+          s.F <<= 32;
+#pragma unroll
+          for (int l = 0; l < 4; ++l) s.F += (long long)__reduce_add_sync(0xffffffffu, hu[l]) << (8 * l);
+        }
+      } else {
+        s.B = b;
+        s.M = m;
+        s.F = hsum;
+        if (!BIM)
+          s.F = (s.F << 32) + hu[0] + ((long long)hu[1] << 8) + ((long long)hu[2] << 16) + ((long long)hu[3] << 24);
+#pragma unroll
+        for (int o = SEG / 2; o > 0; o >>= 1) {
+          s.B += __shfl_xor_sync(0xffffffffu, s.B, o);
+          s.M += __shfl_xor_sync(0xffffffffu, s.M, o);
+          s.F += __shfl_xor_sync(0xffffffffu, s.F, o);
+        }
+      }
+      if (lane % SEG == 0 && e < gact * 2 * WC) red[e / SEG] = s;
+    }
+    __syncthreads();
+    const uint32_t epoch = ra.epoch0 + (uint32_t)iv;
+    uint4 *rec = ra.rec + (size_t)(epoch & 1u) * ra.rcap * S;
+    for (int g = NCH > 4 ? wid : tid; ok && g < gact; g += NCH > 4 ? nw : nt) {
+      ChunkSum s{0, 0, 0};
+      if (NCH > 4) {  // a warp adds the chunks of a replica
+        for (int q = lane; q < NCH; q += 32) {
+          const ChunkSum p = red[g * NCH + q];
+          s.B += p.B;
+          s.M += p.M;
+          s.F += p.F;
+        }
+        s.B = __reduce_add_sync(0xffffffffu, s.B);
+        s.M = __reduce_add_sync(0xffffffffu, s.M);
+        s.F = warp_reduce_sum(s.F);
+      } else {
+        for (int q = 0; q < NCH; ++q) {
+          const ChunkSum p = red[g * NCH + q];
+          s.B += p.B;
+          s.M += p.M;
+          s.F += p.F;
+        }
+      }
+      if (NCH <= 4 || lane == 0) record_store(rec + (size_t)(r0 + g) * S + rank, epoch, s.B, s.M, s.F);
+    }
+
+    // ---- exchange step j (Eq. 2, Sec. 3.3), taken by every CTA on its own copy -------------------
+    const uint32_t j = xa.j + (uint32_t)iv;
+    const int p0 = (int)(j & 1u) + 2 * tid;  // this thread's first pair
+    // the random number of this thread's first pair does not depend on the energies
+    const uint32_t u0 = p0 + 1 < R ? philox10(v.seed, v.realization, (uint32_t)p0, 0u, j, tag_word(kTagExch, v.stage, 0)).w[0] : 0u;
+    for (int r = tid; ok && r < R; r += nt) {
+      int B, M;
+      long long F;
+      records_sum(rec + (size_t)r * S, S, epoch, xa.err, &B, &M, &F);
+      const double Fd = BIM ? xa.h * (double)F : (double)(2 * F - Htot) * fscale;
+      xs.E[r] = -xa.J * (double)B - Fd;
+      xs.M[r] = M;
+    }
+    __syncthreads();
+    for (int k = p0; ok && k + 1 < R; k += 2 * nt) {
+      const int a = xs.t2r[k], b = xs.t2r[k + 1];
+      const uint32_t u = k == p0 ? u0 : philox10(v.seed, v.realization, (uint32_t)k, 0u, j, tag_word(kTagExch, v.stage, 0)).w[0];
+      const bool acc = accept_delta((xs.beta[k] - xs.beta[k + 1]) * (xs.E[a] - xs.E[b]), (double)u * 0x1p-32);
+      xs.swapped[k] = acc;
+      if (acc) {
+        xs.t2r[k] = b;
+        xs.t2r[k + 1] = a;
+        xs.r2t[b] = k;
+        xs.r2t[a] = k + 1;
+      }
+    }
+    __syncthreads();
+    // counts and measurement of the temperatures this CTA keeps, then the new tables
+    if (ok) {
+      const bool measure = (int64_t)j >= xa.measure_from;
+      for (int k = (int)blockIdx.x + (nt - 1 - tid) * (int)gridDim.x; k < R; k += nt * (int)gridDim.x) {
+        if (((uint32_t)k & 1u) == (j & 1u) && k + 1 < R) {
+          atomicAdd(reinterpret_cast<unsigned long long *>(v.att) + k, 1ull);
+          if (xs.swapped[k]) atomicAdd(reinterpret_cast<unsigned long long *>(v.acc) + k, 1ull);
+        }
+        const int a = xs.t2r[k];
+        if (measure) measure_red(v.obs + (int64_t)k * 5, xs.E[a], xs.M[a], (double)v.N, 1.0 / (double)v.N);
+        if (k == 0 && measure) atomicAdd(reinterpret_cast<unsigned long long *>(v.n_meas), 1ull);
+      }
+      if (iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
+    }
+    __syncthreads();
+  }
+  if (S > 1) sync_slabs<S>();  // a CTA stays until its neighbours' pushes have landed
+
+  for (int t = tid; ok && t < gact * 2 * WC; t += nt) {
+    const int g = t / (2 * WC), rem = t % (2 * WC), c = rem / WC, wl = rem % WC;
+    const int64_t gw = ((int64_t)(r0 + g) * 2 + c) * W + (int64_t)z0 * P + wl;
+    const uint32_t word = sp[(g * 2 + c) * CW + Z1 * P + wl];
+    if (ra.i8)
+      unpack_int8_word(word, v.spins8 + 32 * gw);
+    else
+      v.bits[gw] = word;
+  }
+  if (xa.enabled && ok && blockIdx.x == 0)
+    for (int r = tid; r < R; r += nt) {
+      v.t2r[r] = xs.t2r[r];
+      v.r2t[r] = xs.r2t[r];
+      v.E[r] = xs.E[r];
+      v.M[r] = xs.M[r];
+    }
+}
+
+}  // namespace rfim

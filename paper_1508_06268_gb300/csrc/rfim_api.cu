@@ -207,12 +207,7 @@ int check_device_error(rfim_ctx *c) {
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
   if (!word) return RFIM_OK;
   CUDA_OR_FAIL(c, cudaMemsetAsync(c->plan.counter + 1, 0, 4, c->stream));
-  if (c->plan.prog) {  // an expired wait can leave the grid-wide kernel's progress words uneven
-    CUDA_OR_FAIL(c, cudaMemsetAsync(c->plan.prog, 0, (size_t)std::max(c->plan.sms, 1) * 4, c->stream));
-    CUDA_OR_FAIL(c, cudaMemsetAsync(c->plan.counter + 2, 0, 4, c->stream));
-    c->plan.prog_base = 0;
-    c->plan.arrive_base = 0;
-  }
+  CUDA_OR_FAIL(c, reset_bits_plan(c->plan, c->stream));
   if (word & kDbgMask)
     return fail(c, RFIM_EBOUNDS, "a bounds check of the debug build failed (error word 0x%x); the checked accesses were skipped", word);
   return fail(c, RFIM_ETIMEOUT, "a bounded device wait expired (error word %u); results of that launch are invalid", word);
@@ -249,8 +244,8 @@ int measure_xi_after(rfim_ctx *c, int64_t j, int64_t measure_from) {
   return RFIM_OK;
 }
 
-// Bit layout: n sweeps and the exchange step in one launch (fused tail); with the grid-wide plan,
-// k such intervals in one launch.
+// Bit layout: n sweeps and the exchange step in one launch (fused tail); with the grid-wide and
+// resident plans, k such intervals in one launch.
 int do_sweeps_exchange_bits(rfim_ctx *c, int64_t n, int64_t measure_from, int32_t k = 1) {
   RealView v = view_of(c);
   cudaEvent_t stop;
@@ -263,9 +258,6 @@ int do_sweeps_exchange_bits(rfim_ctx *c, int64_t n, int64_t measure_from, int32_
   c->xstep += k;
   return measure_xi_after(c, c->xstep - 1, measure_from);
 }
-
-// Exchange intervals one grid-wide launch takes at most (the host regains control between them).
-constexpr int64_t kMaxIntervalsPerLaunch = 64;
 
 int do_exchange(rfim_ctx *c, int64_t measure_from) {
   if (c->plan.counter) return do_sweeps_exchange_bits(c, 0, measure_from);
@@ -291,11 +283,11 @@ int do_run(rfim_ctx *c, int64_t n_sweeps, int32_t ex, int64_t measure_from) {
     }
     const bool ends_interval = ex > 0 && (c->sweep + chunk) % ex == 0;
     int rc;
-    // whole intervals on the grid-wide plan: several per launch (not with the structure factor,
-    // which a separate kernel measures after every exchange step, nor with multi-hit)
-    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && c->plan.counter && c->plan.S == 0 &&
+    // whole intervals on the grid-wide and resident plans: several per launch (not with the
+    // structure factor, which a separate kernel measures after every exchange step, nor with multi-hit)
+    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && c->plan.counter && c->plan.max_intervals() > 1 &&
         !c->xi_on && c->mh.mh == 0) {
-      const int64_t k = std::min(left / ex, kMaxIntervalsPerLaunch);
+      const int64_t k = std::min(left / ex, c->plan.max_intervals());
       rc = do_sweeps_exchange_bits(c, ex, measure_from, (int32_t)k);
       if (rc) return rc;
       left -= k * ex;
@@ -599,7 +591,7 @@ int rfim_set_multihit(rfim_ctx *ctx, int32_t mh, int32_t tile) {
     // the current launch shape has no multi-hit instance (e.g. the grid-wide plan): switch to the
     // default cluster / single-CTA shape of this L
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
-    const char *shape = c->L == 64 ? "4,4,4,512" : c->L == 32 ? "2,1,1,256" : "1,8,1,512";
+    const char *shape = c->L == 64 ? "4,4,4,512" : c->L == 32 ? "2,1,1,256" : "1,4,1,512";
     BitsPlan np;
     set_plan_override(shape);
     const int rc = make_bits_plan(c->L, c->Rcap, bim, &np, &c->err);
@@ -751,8 +743,7 @@ int rfim_get_plan(const rfim_ctx *ctx, char *plan_out, int32_t plan_cap) {
     plan_out[0] = '\0';
     return RFIM_OK;
   }
-  snprintf(plan_out, (size_t)plan_cap, "%d,%d,%d,%d%s%s", p.S, p.G, p.GT, p.threads, p.NS == 4 ? ",4" : "",
-           p.i8 ? ",int8" : "");
+  snprintf(plan_out, (size_t)plan_cap, "%s", plan_name(p).c_str());
   return RFIM_OK;
 }
 
@@ -782,7 +773,7 @@ int rfim_tune(int32_t L, int32_t R, int32_t field_kind, char *plan_out, int32_t 
   const int64_t intervals = L >= 32 ? 20 : 50, ex = 10;
   std::string best;
   double best_rate = 0.0;
-  for (const std::string &cand : plan_candidates(L)) {
+  for (const std::string &cand : plan_candidates(L, R, bim)) {
     set_plan_override(cand.c_str());
     rfim_ctx *c = nullptr;
     const int rc = rfim_create(&cfg, &c);

@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "resident.h"
 
 namespace rfim {
 
@@ -40,6 +41,14 @@ struct BitsPlan {
   int32_t sms = 0;
   bool i8 = false;  // the realization is stored in the int8 layout and staged as bits (cluster shapes)
   int32_t NS = 1;   // 4: every word split over four warps, one block pair each (small lattices)
+  // resident plan (kernels_resident.cuh): its shape (threads > 0 when it is the plan), the energy
+  // records and the number of the last exchange interval that has been launched
+  ResidentShape res;
+  uint4 *rec = nullptr;
+  mutable uint32_t epoch = 0;
+  bool resident() const { return res.threads > 0; }
+  // exchange intervals one launch takes at most
+  int64_t max_intervals() const { return resident() ? kResidentIntervals : S == 0 ? 64 : 1; }
 };
 
 // Multi-hit double 3D checkerboard (Sec. 3.2, kernels_mh.cuh): mh local passes per tile visit
@@ -59,7 +68,7 @@ bool bits_supported(int32_t L);
 // remembered best shape per (L, R, field kind), and the candidates instantiated for each L.
 void set_plan_override(const char *plan);
 void remember_tuned_plan(int32_t L, int32_t R, bool bimodal, const std::string &plan);
-std::vector<std::string> plan_candidates(int32_t L);
+std::vector<std::string> plan_candidates(int32_t L, int32_t R, bool bimodal);
 int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::string *err, bool i8 = false);
 // The int8-layout staging instance for a cluster shape (kernels_bits_i8.cu), or null.
 void *kernel_for_i8(int L, int S, int GT, int NT, bool bim);
@@ -68,11 +77,16 @@ void *kernel_for_split(int L, int S, int GT, int NT, bool bim);
 bool bits_plan_fits(const BitsPlan &plan, int32_t R);
 cudaError_t build_field4(const RealView &v, BitsPlan &plan, cudaStream_t st);
 void free_bits_plan(BitsPlan &plan);
+// Zeroes the words and records that launches of the plan count on across launches (after an expired
+// wait they can be uneven).
+cudaError_t reset_bits_plan(const BitsPlan &plan, cudaStream_t st);
+// The shape in the format of rfim_get_plan.
+std::string plan_name(const BitsPlan &plan);
 // n_sweeps sweeps; when exchange is true the launch ends with exchange step j (energies, swap
 // decisions, permutation, measurement when j >= measure_from).
 // With mh set (mh->mh > 0) the sweeps are multi-hit double-checkerboard sweeps.
-// n_intervals > 1 (grid-wide plan with the exchange only): that many exchange intervals of n_sweeps
-// sweeps each in one launch, exchange steps j, j + 1, ...
+// n_intervals > 1 (grid-wide and resident plans with the exchange only): that many exchange intervals
+// of n_sweeps sweeps each in one launch, exchange steps j, j + 1, ...
 cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t sweep0, int32_t n_sweeps,
                                bool exchange, uint32_t j, int64_t measure_from, double J, double h,
                                cudaStream_t st, const MultiHit *mh = nullptr, int32_t n_intervals = 1);

@@ -1,0 +1,72 @@
+"""The resident sweep kernel (small realizations, many exchange intervals per launch): every launch
+shape it is instantiated for, partial replica groups included, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1508_06268_gb300 as rf
+from paper_1508_06268_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # L, R, "S,G,NB,threads,r" (m: several items per thread)
+    (8, 2, "1,1,1,64,r"), (8, 7, "1,3,1,256,r"), (8, 19, "1,4,2,128,r"), (8, 37, "1,5,4,256,r"),
+    (16, 2, "1,1,1,512,r"), (16, 5, "1,2,2,512,r"), (16, 13, "1,3,4,384,r"), (16, 3, "2,1,1,256,r"), (16, 5, "2,2,2,256,r"),
+    (32, 3, "2,1,4,512,r"), (32, 2, "4,1,4,256,r"), (32, 3, "8,1,2,256,r"), (32, 3, "1,2,4,512,m"), (32, 5, "2,3,4,512,m"),
+    (64, 2, "16,1,4,512,r"), (64, 3, "8,2,4,512,m"), (64, 3, "4,2,4,512,m"),
+]
+
+
+def make(monkeypatch, L, R, plan, **kw):
+    monkeypatch.setenv("RFIM_BITS_PLAN", plan)
+    g = rf.Realization(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
+    monkeypatch.delenv("RFIM_BITS_PLAN")
+    if plan[-1] in "rm":
+        assert g.plan().replace(",int8", "") == plan
+    else:  # a cluster plan: its group is clipped to R
+        assert g.plan()[-1] not in "rm"
+    return g
+
+
+@pytest.mark.parametrize("L,R,plan", SHAPES)
+@pytest.mark.parametrize("layout", [rf.LAYOUT_BITPACK, rf.LAYOUT_INT8])
+def test_resident_shapes_bit_exact(L, R, plan, layout, monkeypatch):
+    """Bimodal field: spins, permutation, exchange counts and sums equal the oracle's after several
+    launches of several intervals, with an odd number of half-sweep pairs between exchanges."""
+    if layout == rf.LAYOUT_INT8 and L == 64:
+        pytest.skip("one layout is enough at the largest size")
+    g = make(monkeypatch, L, R, plan, h=1.5, field_kind=rf.FIELD_BIMODAL, field_seed=3, seed=42, layout=layout)
+    o = oracle.Oracle(L, inputs.geometric_temps(1.0, 5.0, R), h=1.5, field_kind=oracle.FIELD_BIMODAL, field_seed=3, seed=42)
+    n0 = g.launch_count
+    g.run(9, 3, 1)
+    assert g.launch_count - n0 == 1
+    g.sweep(1)
+    g.exchange(0)
+    g.run(7, 2, 0)
+    o.run(9, 3, 1)
+    o.sweep(1)
+    o.exchange(0)
+    o.run(7, 2, 0)
+    st = g.get_state()
+    np.testing.assert_array_equal(st["spins"], o.spins())
+    np.testing.assert_array_equal(st["t2r"], o.perm()[0])
+    np.testing.assert_array_equal(g.observables()["sums"], o.observables())
+
+
+@pytest.mark.parametrize("L,R,plan,ref", [(8, 6, "1,1,1,64,r", "1,16,1,128"), (16, 5, "1,1,2,256,r", "1,8,1,512"),
+                                           (32, 4, "2,1,4,512,r", "2,1,1,256"), (64, 5, "8,1,4,512,m", "4,4,4,512")])
+def test_resident_gaussian_equals_cluster_plan(L, R, plan, ref, monkeypatch):
+    """Float field: the decisions are those of the one-launch-per-interval kernel (the same float
+    operations on the same words), and the fixed-point energies are the same sums."""
+    kw = dict(field_kind=rf.FIELD_EXPLICIT, field=inputs.gaussian_field(L, 77), seed=5)
+    a = make(monkeypatch, L, R, plan, **kw)
+    b = make(monkeypatch, L, R, ref, **kw)
+    for g in (a, b):
+        g.run(60, 3, 4)
+    x, y = a.get_state(), b.get_state()
+    np.testing.assert_array_equal(x["spins"], y["spins"])
+    np.testing.assert_array_equal(x["t2r"], y["t2r"])
+    p, q = a.observables(), b.observables()
+    assert p["n_meas"] == q["n_meas"] == 16
+    for k in ("sums", "att", "acc"):
+        np.testing.assert_array_equal(p[k], q[k])
