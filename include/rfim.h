@@ -329,8 +329,10 @@ int rfim_tune(int32_t L, int32_t R, int32_t field_kind, char *plan_out, int32_t 
    with ",4" appended when every word is split over four warps (S = 0: the grid-wide plan), or
    "S,G,NB,threads,r" for the resident plan of small realizations (a cluster of S slabs holds G replicas
    for up to 512 exchange intervals per launch, NB Philox blocks of a word per thread item; "m" instead
-   of "r" when a thread runs several items), and ",int8" appended when the int8 layout is staged as bits; "" when the context runs the int8
-   kernels (L outside 8, 16, 32, 64).  plan_out receives at most plan_cap chars (NUL included).
+   of "r" when a thread runs several items), with ",int8" appended when the int8 layout is staged as
+   bits; "S,G,4,threads,b" for the resident plan on bytes (int8 layout, L outside 8, 16, 32, 64), and ""
+   when every half-sweep is a launch of its own (larger int8 realizations).  plan_out receives at most
+   plan_cap chars (NUL included).
    Errors: RFIM_EINVAL (NULL ctx or plan_out, plan_cap < 1). */
 int rfim_get_plan(const rfim_ctx *ctx, char *plan_out, int32_t plan_cap);
 

@@ -16,6 +16,43 @@
 
 namespace rfim {
 
+// Copy of the exchange state each CTA keeps, one entry per replica or temperature.
+struct ResidentState {
+  double *E, *beta;
+  int32_t *M, *t2r, *r2t;
+  uint8_t *swapped;
+};
+
+__host__ __device__ constexpr size_t resident_state_bytes(int rcap) { return (size_t)rcap * 29 + 32; }
+
+struct alignas(16) ChunkSum {
+  int B, M;
+  long long F;
+};
+
+constexpr unsigned kMbarSpinLimit = 1u << 20;
+
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// Bounded wait for the phase of parity `par` of an mbarrier of this CTA.
+__device__ __forceinline__ void mbar_wait(uint32_t mbar, uint32_t par, unsigned *err) {
+  for (unsigned it = 0; it < kMbarSpinLimit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(mbar), "r"(par)
+        : "memory");
+    if (done) return;
+    if ((it & 63u) == 63u && *(volatile unsigned *)err) return;
+  }
+  atomicOr(err, 2u);
+}
+
 constexpr unsigned kRecordSpinLimit = 1u << 22;
 constexpr uint32_t kRecordEpochs = 1u << 22;  // interval numbers 1 .. kRecordEpochs - 1; 0: never written
 
@@ -39,11 +76,14 @@ __device__ __forceinline__ int record_spin(unsigned long long hi) { return (int)
 
 // Sums of n consecutive records of interval `epoch`, polled at most kRecordSpinLimit times; false
 // when they did not all arrive (recorded in *err) or an earlier wait of this launch expired.
+// REAL: the 64-bit field sums are doubles, added in record order.
+template <bool REAL>
 __device__ __forceinline__ bool records_sum(const uint4 *rec, int n, uint32_t epoch, unsigned *err, int *B, int *M,
                                             long long *F) {
   for (unsigned it = 0; it < kRecordSpinLimit; ++it) {
     int b = 0, m = 0;
     long long f = 0;
+    double fd = 0.0;
     bool all = true;
 #pragma unroll 4
     for (int q = 0; q < n; ++q) {
@@ -53,12 +93,15 @@ __device__ __forceinline__ bool records_sum(const uint4 *rec, int n, uint32_t ep
       all = all && (uint32_t)(hi >> 42) == epoch;
       b += record_bonds(hi);
       m += record_spin(hi);
-      f += fq;
+      if (REAL)
+        fd = __dadd_rn(fd, __longlong_as_double(fq));
+      else
+        f += fq;
     }
     if (all) {
       *B = b;
       *M = m;
-      *F = f;
+      *F = REAL ? __double_as_longlong(fd) : f;
       return true;
     }
     if ((it & 63u) == 63u && *(volatile unsigned *)err) break;
@@ -89,16 +132,65 @@ __device__ __forceinline__ bool accept_delta(double delta, double u) {
 
 // measure_add with each sum added in memory: the adds of one temperature come from one thread in
 // interval order, each rounded to nearest as measure_add rounds it, and nothing waits for them.
-// inv_N: 1 / N when N is a power of two (the products below are then the quotients), else 0.
-__device__ __forceinline__ void measure_red(double *acc, double E, long long M, double Nd, double inv_N) {
-  const double e = inv_N != 0.0 ? E * inv_N : E / Nd;
-  const double m = inv_N != 0.0 ? (double)M * inv_N : (double)M / Nd;
+// POW2: N is a power of two, so that the products with 1 / N are the quotients.
+template <bool POW2>
+__device__ __forceinline__ void measure_red(double *acc, double E, long long M, double Nd) {
+  const double e = POW2 ? E * (1.0 / Nd) : E / Nd;
+  const double m = POW2 ? (double)M * (1.0 / Nd) : (double)M / Nd;
   const double m2 = __dmul_rn(m, m);
   atomicAdd(acc + 0, e);
   atomicAdd(acc + 1, __dmul_rn(e, e));
   atomicAdd(acc + 2, fabs(m));
   atomicAdd(acc + 3, m2);
   atomicAdd(acc + 4, __dmul_rn(__dmul_rn(m2, m), m));
+}
+
+// Exchange step j over the records of interval `epoch` (slabs per replica: S), taken by every CTA of
+// the launch on its own copy xs of the temperature assignment: energies E = energy_of(bonds, field
+// sum), the swap decisions of the disjoint pairs (Eq. 2, Sec. 3.3), and, for the temperatures
+// k = CTA mod number of CTAs, the pair counts and the measurement (Sec. 7).  All threads of the CTA
+// call it; the assignment is complete when it returns.
+template <bool REAL, bool POW2 = !REAL, class F>
+__device__ __forceinline__ void exchange_from_records(const RealView &v, const ExchArgs &xa, const ResidentState &xs,
+                                                      const uint4 *rec, int S, uint32_t epoch, uint32_t j, F energy_of) {
+  const int nt = blockDim.x, tid = threadIdx.x, R = v.R;
+  const int p0 = (int)(j & 1u) + 2 * tid;  // this thread's first pair
+  auto random_of = [&](int k) {
+    return philox10(v.seed, v.realization, (uint32_t)k, 0u, j, tag_word(kTagExch, v.stage, 0)).w[0];
+  };
+  // the random number of the first pair does not depend on the energies
+  const uint32_t u0 = p0 + 1 < R ? random_of(p0) : 0u;
+  for (int r = tid; r < R; r += nt) {
+    int B, M;
+    long long Fs;
+    records_sum<REAL>(rec + (size_t)r * S, S, epoch, xa.err, &B, &M, &Fs);
+    xs.E[r] = energy_of(B, Fs);
+    xs.M[r] = M;
+  }
+  __syncthreads();
+  for (int k = p0; k + 1 < R; k += 2 * nt) {
+    const int a = xs.t2r[k], b = xs.t2r[k + 1];
+    const uint32_t u = k == p0 ? u0 : random_of(k);
+    const bool acc = accept_delta((xs.beta[k] - xs.beta[k + 1]) * (xs.E[a] - xs.E[b]), (double)u * 0x1p-32);
+    xs.swapped[k] = acc;
+    if (acc) {
+      xs.t2r[k] = b;
+      xs.t2r[k + 1] = a;
+      xs.r2t[b] = k;
+      xs.r2t[a] = k + 1;
+    }
+  }
+  __syncthreads();
+  const bool measure = (int64_t)j >= xa.measure_from;
+  for (int k = (int)blockIdx.x + (nt - 1 - tid) * (int)gridDim.x; k < R; k += nt * (int)gridDim.x) {
+    if (((uint32_t)k & 1u) == (j & 1u) && k + 1 < R) {
+      atomicAdd(reinterpret_cast<unsigned long long *>(v.att) + k, 1ull);
+      if (xs.swapped[k]) atomicAdd(reinterpret_cast<unsigned long long *>(v.acc) + k, 1ull);
+    }
+    const int a = xs.t2r[k];
+    if (measure) measure_red<POW2>(v.obs + (int64_t)k * 5, xs.E[a], xs.M[a], (double)v.N);
+    if (k == 0 && measure) atomicAdd(reinterpret_cast<unsigned long long *>(v.n_meas), 1ull);
+  }
 }
 
 }  // namespace rfim

@@ -257,7 +257,9 @@ void remember_tuned_plan(int32_t L, int32_t R, bool bimodal, const std::string &
 
 std::string plan_name(const BitsPlan &p) {
   char buf[64];
-  if (p.resident())
+  if (p.resident() && !p.res.NB)
+    snprintf(buf, sizeof buf, "%d,%d,4,%d,b", p.res.S, p.res.G, p.res.threads);
+  else if (p.resident())
     snprintf(buf, sizeof buf, "%d,%d,%d,%d,%c%s", p.res.S, p.res.G, p.res.NB, p.res.threads, p.res.one ? 'r' : 'm',
              p.i8 ? ",int8" : "");
   else
@@ -557,7 +559,8 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
     ra.epoch0 = plan.epoch + 1;
     ra.rec = plan.rec;
     ra.i8 = plan.i8;
-    const cudaError_t e = launch_resident(v, plan.res, ra, sweep0, n_sweeps, plan.field4, xa, st);
+    const cudaError_t e = plan.res.NB ? launch_resident(v, plan.res, ra, sweep0, n_sweeps, plan.field4, xa, st)
+                                      : launch_resident_bytes(v, plan.res, ra, sweep0, n_sweeps, xa, st);
     if (e == cudaSuccess && exchange) plan.epoch += (uint32_t)n_intervals;
     return e;
   }

@@ -13,6 +13,7 @@
 #include <cstdint>
 
 #include "decide.cuh"
+#include "decide_bytes.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 #include "philox.cuh"
@@ -65,45 +66,6 @@ __global__ void __launch_bounds__(256) k_halfsweep_int8(RealView v, int colour, 
 
 
 __device__ __forceinline__ uint32_t ld_u32(const uint8_t *p) { return *reinterpret_cast<const uint32_t *>(p); }
-
-// prmt.b32 in its default mode: a selector nibble with bit 3 set gives the sign of the selected
-// byte replicated over the result byte.
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-  return d;
-}
-
-// Decisions of the four sites of one Philox block: 0/1 spin bytes `cur`, up-count bytes `up`,
-// field bits `hb` (bimodal) or values `h4` (float), table slot `slot`.  Returns 0x01 in the byte
-// of every accepted site.
-template <bool kBimodalField>
-__device__ __forceinline__ uint32_t decide4(const Words4 &w, uint32_t cur, uint32_t up, uint32_t hb, const float4 &h4,
-                                            uint32_t slot) {
-  if (kBimodalField) {
-    const uint32_t offs = ((hb << 4) | (cur << 3) | up) << 2;  // per byte: table index x 4
-    uint32_t flips = 0u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      uint32_t t;
-      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t) : "r"(__byte_perm(offs, slot, 0x7650u | (uint32_t)j)));
-      if (accept_table(w.w[j], t)) flips |= 1u << (8 * j);
-    }
-    return flips;
-  }
-  const float hk[4] = {h4.x, h4.y, h4.z, h4.w};
-  const uint32_t offs = ((cur << 3) | up) << 3;  // per byte: table index x 8
-  uint32_t sg[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float2 e;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(e.x), "=f"(e.y) : "r"(__byte_perm(offs, slot, 0x7650u | (uint32_t)j)));
-    sg[j] = accept_float_sign(w.w[j], e.x, hk[j], e.y);
-  }
-  // byte j = 0xFF where site j is accepted (sign of the top byte of sg[j]), then one bit per byte
-  const uint32_t m01 = prmt(sg[0], sg[1], 0x00FBu), m23 = prmt(sg[2], sg[3], 0xFB00u);
-  return ((m01 & 0x0000FFFFu) | (m23 & 0xFFFF0000u)) & 0x01010101u;
-}
 
 // Per-replica decision tables of the CTA's GT replicas (64 words each: bimodal 32 x (thr - 1),
 // float field 16 x (b J n, +-b)), filled by all threads.

@@ -9,6 +9,47 @@
 
 namespace rfim {
 
+int resident_ctas(const void *fn, int S, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void *, int, int, size_t>, int> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const auto key = std::make_tuple(dev, fn, S, threads, smem);
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+  }
+  int n = 0;
+  if (raise_smem_limit(fn, smem) == cudaSuccess &&
+      (S <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
+    if (S == 1) {
+      int per_sm = 0, sms = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) == cudaSuccess &&
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        n = per_sm * sms;
+    } else {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)S);
+      cfg.blockDim = dim3((unsigned)threads);
+      cfg.dynamicSmemBytes = smem;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)S;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int clusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess) n = clusters * S;
+    }
+  }
+  cudaGetLastError();
+  std::lock_guard<std::mutex> lk(mu);
+  known[key] = n;
+  return n;
+}
+
 namespace {
 
 using ResidentFn = void (*)(RealView, ResidentArgs, uint32_t, int32_t, const float4 *, ExchArgs);
@@ -60,55 +101,11 @@ int warp_items(const Instance &i, int32_t G) {
   return ((groups * (8 / i.NB) << lw) + 31) / 32;
 }
 
-// CTAs of (fn, S, threads, smem) resident at once on the current device, 0 on error.
-int resident_ctas(const void *fn, int S, int threads, size_t smem) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, const void *, int, size_t>, int> known;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const auto key = std::make_tuple(dev, fn, threads, smem);
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    const auto it = known.find(key);
-    if (it != known.end()) return it->second;
-  }
-  int n = 0;
-  if (raise_smem_limit(fn, smem) == cudaSuccess &&
-      (S <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)) {
-    if (S == 1) {
-      int per_sm = 0, sms = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) == cudaSuccess &&
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-        n = per_sm * sms;
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)S);
-      cfg.blockDim = dim3((unsigned)threads);
-      cfg.dynamicSmemBytes = smem;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = (unsigned)S;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess) n = clusters * S;
-    }
-  }
-  cudaGetLastError();
-  std::lock_guard<std::mutex> lk(mu);
-  known[key] = n;
-  return n;
-}
-
 // Threads of a CTA: one item each up to the instance's limit, and enough to poll the records.
 int cta_threads(const Instance &i, int32_t G, int32_t R) {
   const int want = std::max(32 * warp_items(i, G), std::min((R + 31) / 32 * 32, 256));
   return std::min(want, i.NT);
 }
-
-constexpr size_t kOneCtaSmem = 116 * 1024;  // more than half an SM's shared memory: one CTA per SM
 
 // Estimated cycles of a half-sweep (measured at L = 8 to 64, 2.07 GHz): warp instructions of the
 // fullest SM (15 per attempt and 50 per item, 137 where items are decoded every time) at 2.4 per
@@ -183,35 +180,34 @@ std::vector<ResidentShape> resident_shapes(int32_t L, int32_t R, bool bimodal) {
   return all;
 }
 
-cudaError_t launch_resident(const RealView &v, const ResidentShape &s, const ResidentArgs &args, uint32_t sweep0,
-                            int32_t n_sweeps, const float4 *field4, const ExchArgs &xa, cudaStream_t st) {
-  const Instance *i = find(v.L, s);
-  if (!i) return cudaErrorInvalidConfiguration;
-  ResidentArgs ra = args;
-  for (uint32_t q = 0; q < 10; ++q) {
-    ra.keys.k0[q] = v.seed + q * kPhiloxW0;
-    ra.keys.k1[q] = v.realization + q * kPhiloxW1;
-  }
-  ra.lw = lane_words(*i, s.G);
-  const int clusters = (v.R + s.G - 1) / s.G;
-  cudaLaunchConfig_t cfg = {};
+ResidentLaunch::ResidentLaunch(int clusters, const ResidentShape &s, bool exchange, cudaStream_t st) {
   cfg.gridDim = dim3((unsigned)(clusters * s.S));
   cfg.blockDim = dim3((unsigned)s.threads);
   cfg.dynamicSmemBytes = s.smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[2];
   if (s.S > 1) {
     at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
     at[cfg.numAttrs].val.clusterDim.x = (unsigned)s.S;
     at[cfg.numAttrs].val.clusterDim.y = 1;
     at[cfg.numAttrs++].val.clusterDim.z = 1;
   }
-  if (xa.enabled && clusters > 1) {  // the exchange step waits for every CTA: all must be resident
+  if (exchange && clusters > 1) {
     at[cfg.numAttrs].id = cudaLaunchAttributeCooperative;
     at[cfg.numAttrs++].val.cooperative = 1;
   }
   cfg.attrs = at;
-  return cudaLaunchKernelEx(&cfg, v.kind == kBimodal ? i->bim : i->flt, v, ra, sweep0, n_sweeps, field4, xa);
+}
+
+cudaError_t launch_resident(const RealView &v, const ResidentShape &s, const ResidentArgs &args, uint32_t sweep0,
+                            int32_t n_sweeps, const float4 *field4, const ExchArgs &xa, cudaStream_t st) {
+  const Instance *i = find(v.L, s);
+  if (!i) return cudaErrorInvalidConfiguration;
+  ResidentArgs ra = args;
+  ra.keys = philox_keys(v.seed, v.realization);
+  ra.lw = lane_words(*i, s.G);
+  const int clusters = (v.R + s.G - 1) / s.G;
+  ResidentLaunch l(clusters, s, xa.enabled, st);
+  return cudaLaunchKernelEx(&l.cfg, v.kind == kBimodal ? i->bim : i->flt, v, ra, sweep0, n_sweeps, field4, xa);
 }
 
 }  // namespace rfim

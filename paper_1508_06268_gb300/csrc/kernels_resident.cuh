@@ -26,13 +26,9 @@
 
 #include "exchange_records.cuh"
 #include "kernels_bits.cuh"
+#include "philox_parts.cuh"
 
 namespace rfim {
-
-// Round keys of the realization's Philox streams (operands from the constant bank: no key adds).
-struct PhiloxKeys {
-  uint32_t k0[10], k1[10];
-};
 
 struct ResidentArgs {
   PhiloxKeys keys;
@@ -45,15 +41,6 @@ struct ResidentArgs {
   int32_t lw;       // log2 of the words whose items of one part are neighbouring threads (ONE; else 5)
 };
 
-// Copy of the exchange state each CTA keeps, one entry per replica or temperature.
-struct ResidentState {
-  double *E, *beta;
-  int32_t *M, *t2r, *r2t;
-  uint8_t *swapped;
-};
-
-__host__ __device__ constexpr size_t resident_state_bytes(int rcap) { return (size_t)rcap * 29 + 32; }
-
 // Planes of a slab in shared memory: with S > 1 a halo plane before and after the slab's own.
 template <int L, int S>
 __host__ __device__ constexpr int resident_planes() { return L / S + (S > 1 ? 2 : 0); }
@@ -62,81 +49,6 @@ __host__ __device__ constexpr int resident_planes() { return L / S + (S > 1 ? 2 
 template <int L, int S>
 __host__ __device__ constexpr int resident_chunks() {
   return 2 * (L / S) * (L * L / 64) >= 32 ? 2 * (L / S) * (L * L / 64) / 32 : 1;
-}
-
-constexpr unsigned kMbarSpinLimit = 1u << 20;
-
-struct alignas(16) ChunkSum {
-  int B, M;
-  long long F;
-};
-
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-
-// Bounded wait for the phase of parity `par` of an mbarrier of this CTA.
-__device__ __forceinline__ void mbar_wait(uint32_t mbar, uint32_t par, unsigned *err) {
-  for (unsigned it = 0; it < kMbarSpinLimit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(mbar), "r"(par)
-        : "memory");
-    if (done) return;
-    if ((it & 63u) == 63u && *(volatile unsigned *)err) return;
-  }
-  atomicOr(err, 2u);
-}
-
-// What the words of Philox blocks of one thread need besides the replica and the sweep: the products
-// of the first two rounds that hold only the block index and the colour.
-template <int NB>
-struct BlockParts {
-  uint32_t lo[NB];      // low half of M0 * block
-  uint64_t q[2][NB];    // per colour: M1 * (high half of M0 * block ^ tag ^ k1[0])
-};
-
-// Words of the NB blocks for sweep and colour c: rounds 0 and 1 from the parts, then eight rounds.
-template <int NB>
-__device__ __forceinline__ void philox_words(const PhiloxKeys &k, const BlockParts<NB> &bp, int c, uint32_t r, uint32_t sweep,
-                                             Words4 (&w)[NB]) {
-  const uint64_t s = (uint64_t)kPhiloxM1 * sweep;
-  const uint64_t p = (uint64_t)kPhiloxM0 * ((uint32_t)(s >> 32) ^ r ^ k.k0[0]);
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    uint32_t c0 = (uint32_t)(bp.q[c][j] >> 32) ^ (uint32_t)s ^ k.k0[1], c1 = (uint32_t)bp.q[c][j];
-    uint32_t c2 = (uint32_t)(p >> 32) ^ bp.lo[j] ^ k.k1[1], c3 = (uint32_t)p;
-#pragma unroll
-    for (int i = 2; i < 10; ++i) {
-      const uint64_t p0 = (uint64_t)kPhiloxM0 * c0, p1 = (uint64_t)kPhiloxM1 * c2;
-      c0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.k0[i];
-      c2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.k1[i];
-      c1 = (uint32_t)p1;
-      c3 = (uint32_t)p0;
-    }
-    w[j].w[0] = c0;
-    w[j].w[1] = c1;
-    w[j].w[2] = c2;
-    w[j].w[3] = c3;
-  }
-}
-
-template <int NB>
-__device__ __forceinline__ BlockParts<NB> block_parts(const PhiloxKeys &k, uint32_t stage, uint32_t block0) {
-  BlockParts<NB> bp;
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    const uint64_t p = (uint64_t)kPhiloxM0 * (block0 + (uint32_t)j);
-    bp.lo[j] = (uint32_t)p;
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-      bp.q[c][j] = (uint64_t)kPhiloxM1 * ((uint32_t)(p >> 32) ^ tag_word(kTagMetro, stage, (uint32_t)c) ^ k.k1[0]);
-  }
-  return bp;
 }
 
 // One item: word iw of plane zl of replica g of the slab, blocks sh .. sh + NB - 1 of it.
@@ -425,47 +337,13 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
       if (NCH <= 4 || lane == 0) record_store(rec + (size_t)(r0 + g) * S + rank, epoch, s.B, s.M, s.F);
     }
 
-    // ---- exchange step j (Eq. 2, Sec. 3.3), taken by every CTA on its own copy -------------------
-    const uint32_t j = xa.j + (uint32_t)iv;
-    const int p0 = (int)(j & 1u) + 2 * tid;  // this thread's first pair
-    // the random number of this thread's first pair does not depend on the energies
-    const uint32_t u0 = p0 + 1 < R ? philox10(v.seed, v.realization, (uint32_t)p0, 0u, j, tag_word(kTagExch, v.stage, 0)).w[0] : 0u;
-    for (int r = tid; ok && r < R; r += nt) {
-      int B, M;
-      long long F;
-      records_sum(rec + (size_t)r * S, S, epoch, xa.err, &B, &M, &F);
+    // ---- exchange step, then the tables of the temperatures it assigned ------------------------------
+    auto energy_of = [&](int B, long long F) {
       const double Fd = BIM ? xa.h * (double)F : (double)(2 * F - Htot) * fscale;
-      xs.E[r] = -xa.J * (double)B - Fd;
-      xs.M[r] = M;
-    }
-    __syncthreads();
-    for (int k = p0; ok && k + 1 < R; k += 2 * nt) {
-      const int a = xs.t2r[k], b = xs.t2r[k + 1];
-      const uint32_t u = k == p0 ? u0 : philox10(v.seed, v.realization, (uint32_t)k, 0u, j, tag_word(kTagExch, v.stage, 0)).w[0];
-      const bool acc = accept_delta((xs.beta[k] - xs.beta[k + 1]) * (xs.E[a] - xs.E[b]), (double)u * 0x1p-32);
-      xs.swapped[k] = acc;
-      if (acc) {
-        xs.t2r[k] = b;
-        xs.t2r[k + 1] = a;
-        xs.r2t[b] = k;
-        xs.r2t[a] = k + 1;
-      }
-    }
-    __syncthreads();
-    // counts and measurement of the temperatures this CTA keeps, then the new tables
-    if (ok) {
-      const bool measure = (int64_t)j >= xa.measure_from;
-      for (int k = (int)blockIdx.x + (nt - 1 - tid) * (int)gridDim.x; k < R; k += nt * (int)gridDim.x) {
-        if (((uint32_t)k & 1u) == (j & 1u) && k + 1 < R) {
-          atomicAdd(reinterpret_cast<unsigned long long *>(v.att) + k, 1ull);
-          if (xs.swapped[k]) atomicAdd(reinterpret_cast<unsigned long long *>(v.acc) + k, 1ull);
-        }
-        const int a = xs.t2r[k];
-        if (measure) measure_red(v.obs + (int64_t)k * 5, xs.E[a], xs.M[a], (double)v.N, 1.0 / (double)v.N);
-        if (k == 0 && measure) atomicAdd(reinterpret_cast<unsigned long long *>(v.n_meas), 1ull);
-      }
-      if (iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
-    }
+      return -xa.J * (double)B - Fd;
+    };
+    if (ok) exchange_from_records<false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, energy_of);
+    if (ok && iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
   if (S > 1) sync_slabs<S>();  // a CTA stays until its neighbours' pushes have landed

@@ -15,7 +15,8 @@ namespace rfim {
 constexpr int64_t kResidentIntervals = 512;
 
 struct ResidentShape {
-  int32_t S = 0, G = 0, NB = 0, threads = 0;  // slabs, replicas per cluster, Philox blocks per item, threads per CTA
+  // slabs, replicas per cluster, Philox blocks per item (0: the kernel on bytes), threads per CTA
+  int32_t S = 0, G = 0, NB = 0, threads = 0;
   bool one = true;  // one item per thread (else a thread may run several)
   size_t smem = 0;
 };
@@ -27,6 +28,23 @@ bool resident_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, doub
 std::vector<ResidentShape> resident_shapes(int32_t L, int32_t R, bool bimodal);
 // Whether the instance exists and all CTAs of R replicas are resident at once; fills s->smem.
 bool resident_fits(int32_t L, int32_t R, bool bimodal, ResidentShape *s);
+// CTAs of (kernel, clusters of S, threads, shared memory) resident at once on the current device.
+int resident_ctas(const void *fn, int S, int threads, size_t smem);
+constexpr size_t kOneCtaSmem = 116 * 1024;  // more than half an SM's shared memory: one CTA per SM
+
+// Launch configuration of `clusters` clusters of shape s; cooperative when the CTAs wait for one
+// another (the exchange step of more than one cluster).
+struct ResidentLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  ResidentLaunch(int clusters, const ResidentShape &s, bool exchange, cudaStream_t st);
+  ResidentLaunch(const ResidentLaunch &) = delete;
+};
+
+// The same on bytes (kernels_bytes.cuh): realizations of the int8 layout at other even L.
+bool bytes_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles);
+cudaError_t launch_resident_bytes(const RealView &v, const ResidentShape &s, const ResidentArgs &args, uint32_t sweep0,
+                                  int32_t n_sweeps, const ExchArgs &xa, cudaStream_t st);
 cudaError_t launch_resident(const RealView &v, const ResidentShape &s, const ResidentArgs &args, uint32_t sweep0,
                             int32_t n_sweeps, const float4 *field4, const ExchArgs &xa, cudaStream_t st);
 

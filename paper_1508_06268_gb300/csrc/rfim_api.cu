@@ -201,7 +201,7 @@ int reset_state(rfim_ctx *c, uint32_t stage) {
 // checks of the debug build as RFIM_EBOUNDS; the word is cleared once reported.  Synchronises the
 // stream.
 int check_device_error(rfim_ctx *c) {
-  if (!c->plan.counter) return RFIM_OK;  // no bit-layout plan (int8 kernels of other L)
+  if (!c->plan.counter) return RFIM_OK;  // no plan (one int8 launch per half-sweep)
   unsigned int word = 0;
   CUDA_OR_FAIL(c, cudaMemcpyAsync(&word, c->plan.counter + 1, 4, cudaMemcpyDeviceToHost, c->stream));
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
@@ -218,7 +218,7 @@ int do_sweeps(rfim_ctx *c, int64_t n) {
   RealView v = view_of(c);
   cudaEvent_t stop;
   CUDA_OR_FAIL(c, prof_begin(c, 0, &stop));
-  if (c->plan.counter) {  // bit layout, or the int8 layout staged as bits
+  if (c->plan.counter) {  // bit layout, or the int8 layout staged as bits or resident as bytes
     CUDA_OR_FAIL(c, launch_sweeps_bits(v, c->plan, (uint32_t)c->sweep, (int32_t)n, false, 0u, 0, (double)c->J,
                                        (double)c->h, c->stream, &c->mh));
     c->launches += 1;
@@ -380,7 +380,8 @@ int rfim_create(const rfim_config *cfg, rfim_ctx **out) {
     return code;
   };
   // int8 layout with L in {8, 16, 32, 64}: stored as bytes, swept by the bit-layout kernels that
-  // stage each slab as bits in shared memory (kernels_bits_i8.cu)
+  // stage each slab as bits in shared memory; other L: resident in shared memory as bytes where the
+  // lattice fits (kernels_bytes.cuh), else one launch per half-sweep (kernels_int8.cu)
   const bool staged_i8 = cfg->layout == RFIM_LAYOUT_INT8 && bits_supported(L);
   if (c->layout == RFIM_LAYOUT_BITPACK) {
     if ((rc = dalloc(c, &c->bits, (size_t)Rcap * N / 32))) return bail(rc);
@@ -416,6 +417,8 @@ int rfim_create(const rfim_config *cfg, rfim_ctx **out) {
   (void)half;
   if (c->layout == RFIM_LAYOUT_BITPACK || staged_i8) {
     if ((rc = make_bits_plan(L, Rcap, c->kind == kBimodal, &c->plan, &c->err, staged_i8))) return bail(rc);
+  } else if ((rc = make_bytes_plan(L, Rcap, c->kind == kBimodal, &c->plan, &c->err))) {
+    return bail(rc);
   }
   if (c->kind == RFIM_FIELD_EXPLICIT) {
     cudaError_t e = cudaMemcpyAsync(c->hraw, cfg->field, N * 4, cudaMemcpyHostToDevice, c->stream);

@@ -74,6 +74,9 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
 void *kernel_for_i8(int L, int S, int GT, int NT, bool bim);
 // The split-word instance (NS = 4, kernels_bits_split.cu) for a shape, or null.
 void *kernel_for_split(int L, int S, int GT, int NT, bool bim);
+// The resident plan on bytes for the int8 layout at L without a bit layout; an empty plan (counter
+// null) when the lattice does not fit.
+int make_bytes_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::string *err);
 bool bits_plan_fits(const BitsPlan &plan, int32_t R);
 cudaError_t build_field4(const RealView &v, BitsPlan &plan, cudaStream_t st);
 void free_bits_plan(BitsPlan &plan);

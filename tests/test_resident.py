@@ -21,10 +21,10 @@ def make(monkeypatch, L, R, plan, **kw):
     monkeypatch.setenv("RFIM_BITS_PLAN", plan)
     g = rf.Realization(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
     monkeypatch.delenv("RFIM_BITS_PLAN")
-    if plan[-1] in "rm":
+    if plan[-1] in "rmb":
         assert g.plan().replace(",int8", "") == plan
     else:  # a cluster plan: its group is clipped to R
-        assert g.plan()[-1] not in "rm"
+        assert g.plan()[-1] not in "rmb"
     return g
 
 
@@ -70,3 +70,42 @@ def test_resident_gaussian_equals_cluster_plan(L, R, plan, ref, monkeypatch):
     assert p["n_meas"] == q["n_meas"] == 16
     for k in ("sums", "att", "acc"):
         np.testing.assert_array_equal(p[k], q[k])
+
+
+BYTES = [  # L, R, "S,G,4,threads,b": rows of whole blocks, even rows, odd rows; blocks across slabs
+    (4, 2, "1,1,4,32,b"), (4, 9, "2,4,4,64,b"), (6, 5, "1,3,4,96,b"), (6, 3, "2,2,4,32,b"), (10, 3, "1,1,4,128,b"),
+    (10, 5, "4,2,4,96,b"), (14, 3, "2,2,4,256,b"), (18, 2, "8,1,4,128,b"), (12, 5, "1,2,4,256,b"), (12, 3, "4,2,4,128,b"),
+    (20, 3, "2,1,4,512,b"), (28, 2, "8,1,4,448,b"), (24, 3, "1,1,4,512,b"), (24, 5, "4,2,4,512,b"), (40, 2, "4,1,4,512,b"),
+    (48, 2, "8,1,4,512,b"), (50, 2, "8,1,4,512,b"), (56, 2, "1,1,4,512,b"), (36, 2, "2,1,4,512,b"),
+]
+
+
+@pytest.mark.parametrize("L,R,plan", BYTES)
+@pytest.mark.parametrize("kind", [rf.FIELD_BIMODAL, rf.FIELD_EXPLICIT])
+def test_resident_bytes_match_oracle(L, R, plan, kind, monkeypatch):
+    """Sizes without a bit layout: bimodal spins, permutation and sums equal the oracle's; with a
+    float field one sweep from the same state gives the oracle's spins up to 1e-4 of the sites (the
+    device's acceptance test is within a few 2^-23 of the oracle's) and its energies to 1e-9."""
+    field = inputs.gaussian_field(L, 9) if kind == rf.FIELD_EXPLICIT else None
+    kw = dict(h=1.5, field_kind=kind, field=field, field_seed=3, seed=42)
+    g = make(monkeypatch, L, R, plan, layout=rf.LAYOUT_INT8, **kw)
+    o = oracle.Oracle(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
+    if kind == rf.FIELD_BIMODAL:
+        for x in (g, o):
+            x.run(6, 3, 1)
+            x.sweep(1)
+            x.exchange(0)
+            x.run(4, 2, 0)
+        np.testing.assert_array_equal(g.get_state()["spins"], o.spins())
+        np.testing.assert_array_equal(g.get_state()["t2r"], o.perm()[0])
+        np.testing.assert_array_equal(g.observables()["sums"], o.observables())
+        return
+    for x in (g, o):
+        x.sweep(1)
+    spins = g.get_state()["spins"]
+    assert np.mean(spins != o.spins()) <= 1e-4
+    o.set_spins(spins)
+    for x in (g, o):
+        x.exchange(0)
+    np.testing.assert_array_equal(g.get_state()["t2r"], o.perm()[0])
+    np.testing.assert_allclose(g.observables()["sums"], o.observables(), rtol=1e-9)
