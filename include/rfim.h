@@ -273,7 +273,7 @@ const char *rfim_server_last_error(const rfim_server *s);
    It computes every replica's energy (Eq. 1) from caller-owned buffers and takes exchange step j
    exactly as rfim_exchange does (Eq. 2, Sec. 3.3; measurement of Sec. 7 when j >= measure_from),
    enqueued on `stream`.  It allocates nothing: its scratch (partial sums per replica and z slab,
-   and an arrival counter) is a file-scope device array of 512 KiB that every GPU loading the
+   and an arrival counter) is a file-scope device array of 256 KiB that every GPU loading the
    library holds until exit.  R times the number of z slabs must fit 16384 slots (RFIM_EINVAL
    otherwise, message in rfim_last_error(NULL)).  Every call looks up the array's address on the
    current device (cudaGetSymbolAddress, no stream work); its arrival counter is zero when the
