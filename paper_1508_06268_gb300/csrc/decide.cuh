@@ -36,12 +36,40 @@ __device__ __forceinline__ bool accept_float_l2e(uint32_t word, float bjn, float
   return __uint2float_rz(word) < p32;
 }
 
+// prmt.b32 in its default mode: a selector nibble with bit 3 set gives the sign of the selected
+// byte replicated over the result byte.
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+  return d;
+}
+
+// Rejections of a bimodal test collected as carries: the table holds ~(thr - 1), so that
+// word + ~(thr - 1) carries out exactly when word > thr - 1, and fk becomes 2 fk + carry.  Two
+// additions, which issue at twice the rate of a comparison and a predicated logic operation
+// (5.9 against 5.5 attempts per clock and SM with Philox).
+__device__ __forceinline__ void collect_reject(uint32_t word, uint32_t not_thr, uint32_t &fk) {
+  asm("{\n\t.reg .u32 x;\n\tadd.cc.u32 x, %1, %2;\n\taddc.u32 %0, %0, %0;\n\t}" : "+r"(fk) : "r"(word), "r"(not_thr));
+}
+
 // The same test as a sign bit: bit 31 of the result is 1 iff the move is accepted.  One FMA
 // forms rz(word) - 2^t 2^32 with a single rounding; the product is exact (a power-of-two scaling)
 // so the result is the correctly rounded difference, negative exactly when rz(word) < p32 and
 // +0 when they are equal.
 __device__ __forceinline__ uint32_t accept_float_sign(uint32_t word, float bjn, float hh, float b) {
   return __float_as_uint(__fmaf_rn(ex2_approx(boltzmann_exponent(bjn, hh, b)), -4294967296.0f, __uint2float_rz(word)));
+}
+
+// accept_float_sign of two sites, the two differences by one packed FMA (each rounded on its own):
+// 5.09 against 4.96 attempts per clock and SM with Philox, 5.21 with the signs collected by prmt.
+__device__ __forceinline__ uint2 accept_float_signs(uint32_t w0, uint32_t w1, float2 e0, float2 e1, float h0, float h1) {
+  uint2 r;
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmov.b64 c, {%5, %6};\n\t"
+      "fma.rn.f32x2 a, a, b, c;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "=r"(r.x), "=r"(r.y)
+      : "f"(ex2_approx(boltzmann_exponent(e0.x, h0, e0.y))), "f"(ex2_approx(boltzmann_exponent(e1.x, h1, e1.y))),
+        "f"(-4294967296.0f), "f"(__uint2float_rz(w0)), "f"(__uint2float_rz(w1)));
+  return r;
 }
 
 }  // namespace rfim

@@ -7,14 +7,6 @@
 
 namespace rfim {
 
-// prmt.b32 in its default mode: a selector nibble with bit 3 set gives the sign of the selected
-// byte replicated over the result byte.
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-  return d;
-}
-
 // Decisions of the four sites of one Philox block: 0/1 spin bytes `cur`, up-count bytes `up`,
 // field bits `hb` (bimodal) or values `h4` (float), table slot `slot`.  Returns 0x01 in the byte
 // of every accepted site.
@@ -34,15 +26,16 @@ __device__ __forceinline__ uint32_t decide4(const Words4 &w, uint32_t cur, uint3
   }
   const float hk[4] = {h4.x, h4.y, h4.z, h4.w};
   const uint32_t offs = ((cur << 3) | up) << 3;  // per byte: table index x 8
-  uint32_t sg[4];
+  float2 e[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float2 e;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(e.x), "=f"(e.y) : "r"(__byte_perm(offs, slot, 0x7650u | (uint32_t)j)));
-    sg[j] = accept_float_sign(w.w[j], e.x, hk[j], e.y);
-  }
-  // byte j = 0xFF where site j is accepted (sign of the top byte of sg[j]), then one bit per byte
-  const uint32_t m01 = prmt(sg[0], sg[1], 0x00FBu), m23 = prmt(sg[2], sg[3], 0xFB00u);
+  for (int j = 0; j < 4; ++j)
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];"
+                 : "=f"(e[j].x), "=f"(e[j].y)
+                 : "r"(__byte_perm(offs, slot, 0x7650u | (uint32_t)j)));
+  const uint2 a = accept_float_signs(w.w[0], w.w[1], e[0], e[1], hk[0], hk[1]);
+  const uint2 b = accept_float_signs(w.w[2], w.w[3], e[2], e[3], hk[2], hk[3]);
+  // byte j = 0xFF where site j is accepted (its sign bit), then one bit per byte
+  const uint32_t m01 = prmt(a.x, a.y, 0x00FBu), m23 = prmt(b.x, b.y, 0xFB00u);
   return ((m01 & 0x0000FFFFu) | (m23 & 0xFFFF0000u)) & 0x01010101u;
 }
 

@@ -31,7 +31,7 @@ cudaError_t raise_smem_limit(const void *fn, size_t bytes) {
 
 namespace {
 
-using KernelFn = void (*)(RealView, int32_t, uint32_t, int32_t, const float4 *, ExchArgs);
+using KernelFn = void (*)(RealView, int32_t, uint32_t, int32_t, const float4 *, ExchArgs, PhiloxKeys);
 
 template <int L, int S, int GT, int NT>
 KernelFn pick(bool bim) {
@@ -69,7 +69,7 @@ KernelFn kernel_for(int L, int S, int GT, int NT, bool bim, bool i8 = false, int
   return nullptr;
 }
 
-using MhFn = void (*)(RealView, int32_t, uint32_t, int32_t, const float4 *, ExchArgs, MultiHit);
+using MhFn = void (*)(RealView, int32_t, uint32_t, int32_t, const float4 *, ExchArgs, MultiHit, PhiloxKeys);
 
 template <int L, int S, int GT, int NT, int T>
 MhFn mh_pick(bool bim) {
@@ -89,7 +89,7 @@ MhFn mh_kernel_for(int L, int S, int GT, int NT, bool bim, int T) {
 
 int words_per_cta(int L, int S) { return L <= 0 || S <= 0 ? 0 : (L / S) * (L * L / 64); }
 
-using GridFn = void (*)(RealView, GridArgs, uint32_t, int32_t, const float4 *, ExchArgs);
+using GridFn = void (*)(RealView, GridArgs, uint32_t, int32_t, const float4 *, ExchArgs, PhiloxKeys);
 
 template <int L, int GG, int GTI, int NT, bool I8 = false>
 GridFn grid_pick(bool bim) {
@@ -599,7 +599,8 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, gfn, vg, ga, sweep0, n_sweeps, (const float4 *)plan.field4, xa);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, gfn, vg, ga, sweep0, n_sweeps, (const float4 *)plan.field4, xa,
+                                              philox_keys(v.seed, v.realization));
     if (le != cudaSuccess) {  // nothing ran: the words did not advance
       plan.prog_base -= add;
       plan.arrive_base -= arrivals;
@@ -613,6 +614,7 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
   MhFn mfn = multihit ? mh_kernel_for(plan.L, plan.S, plan.GT, plan.threads, v.kind == kBimodal, mh->tile) : nullptr;
   if (!fn && !mfn) return cudaErrorInvalidConfiguration;
   const int clusters = (v.R + plan.G - 1) / plan.G;
+  const PhiloxKeys keys = philox_keys(v.seed, v.realization);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(clusters * plan.S));
   cfg.blockDim = dim3((unsigned)plan.threads);
@@ -628,8 +630,8 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
     cfg.numAttrs = 1;
   }
   if (mfn)
-    return cudaLaunchKernelEx(&cfg, mfn, v, (int32_t)plan.G, sweep0, n_sweeps, (const float4 *)plan.field4, xa, *mh);
-  return cudaLaunchKernelEx(&cfg, fn, v, (int32_t)plan.G, sweep0, n_sweeps, (const float4 *)plan.field4, xa);
+    return cudaLaunchKernelEx(&cfg, mfn, v, (int32_t)plan.G, sweep0, n_sweeps, (const float4 *)plan.field4, xa, *mh, keys);
+  return cudaLaunchKernelEx(&cfg, fn, v, (int32_t)plan.G, sweep0, n_sweeps, (const float4 *)plan.field4, xa, keys);
 }
 
 }  // namespace rfim

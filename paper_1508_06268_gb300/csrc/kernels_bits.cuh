@@ -22,7 +22,7 @@
 #include "decide.cuh"
 #include "exchange.cuh"
 #include "internal.h"
-#include "philox.cuh"
+#include "philox_parts.cuh"
 
 namespace rfim {
 
@@ -165,8 +165,9 @@ __device__ __forceinline__ uint32_t tab_slot0(const void *p) {
 }
 
 // Fills the tables of n slots, slot g for temperature temp_of(g), with all threads of the CTA.
-// `base` is any generic pointer into dynamic shared memory at or before the slots.
-template <bool BIM, class F>
+// `base` is any generic pointer into dynamic shared memory at or before the slots.  NEG: bimodal
+// thresholds complemented, as collect_reject takes them.
+template <bool BIM, bool NEG = true, class F>
 __device__ __forceinline__ void tab_fill_temps(const RealView &v, void *base, uint32_t slot0, int n, F temp_of) {
   constexpr int E = BIM ? 32 : 16;
   char *gen = reinterpret_cast<char *>(base) + (slot0 - (uint32_t)__cvta_generic_to_shared(base));
@@ -175,7 +176,8 @@ __device__ __forceinline__ void tab_fill_temps(const RealView &v, void *base, ui
     const int k = temp_of(g);
     char *slot = gen + (size_t)g * kTabSlot;
     if (BIM) {
-      reinterpret_cast<uint32_t *>(slot)[i] = v.thr[(int64_t)k * 32 + i];
+      const uint32_t thr = v.thr[(int64_t)k * 32 + i];
+      reinterpret_cast<uint32_t *>(slot)[i] = NEG ? ~thr : thr;
     } else {
       const float b = (i >> 3) ? v.b2l[k] : -v.b2l[k];
       reinterpret_cast<float2 *>(slot)[i] = make_float2(__fmul_rn(b, v.gjn[i & 7]), b);
@@ -184,9 +186,9 @@ __device__ __forceinline__ void tab_fill_temps(const RealView &v, void *base, ui
 }
 
 // The same with slot g for the temperature of replica replica_of(g).
-template <bool BIM, class F>
+template <bool BIM, bool NEG = true, class F>
 __device__ __forceinline__ void tab_fill(const RealView &v, void *base, uint32_t slot0, int n, F replica_of) {
-  tab_fill_temps<BIM>(v, base, slot0, n, [&](int g) { return v.r2t[replica_of(g)]; });
+  tab_fill_temps<BIM, NEG>(v, base, slot0, n, [&](int g) { return v.r2t[replica_of(g)]; });
 }
 
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
@@ -201,24 +203,46 @@ __device__ __forceinline__ float2 lds_f2(uint32_t a) {
   return r;
 }
 
+// Decisions of the Philox blocks of one word of one replica, one bit per site.  Float field: block
+// j's accepted sites set bit 8k + j of f[0]; the signs of two sites go into two bytes with one byte
+// permute, then one masked OR per pair (an accumulator per k, shifted by one per site, needs
+// four registers instead of one and 2 % more time).  Bimodal: rejections shifted into f[k], blocks
+// visited in descending order, so that the last one is at bit 0.
+template <bool BIM>
+struct Flips {
+  uint32_t f[BIM ? 4 : 1];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < (BIM ? 4 : 1); ++k) f[k] = 0u;
+  }
+  // The four collectors as one word, collected block b at bit 8k + b (bimodal only).
+  __device__ __forceinline__ uint32_t rejects() const {
+    return f[0] | (f[BIM ? 1 : 0] << 8) | (f[BIM ? 2 : 0] << 16) | (f[BIM ? 3 : 0] << 24);
+  }
+  // Accepted sites of N blocks decided at j = N - 1 .. 0: block j at bit 8k + j.
+  template <int N>
+  __device__ __forceinline__ uint32_t word() const {
+    return BIM ? ~rejects() & (0x01010101u * ((1u << N) - 1u)) : f[0];
+  }
+};
+
 // Decisions of Philox block j of one word of one replica: sites 4j + k (k = 0..3) at bits 8k + j,
-// table slot `slot`, float field h4 of those sites.  Bimodal: accepted sites set their bit of
-// `flip`; float field: the acceptance sign bits are shifted into fk[k] (blocks visited j = 7..0,
-// so block j ends at bit j of fk[k]).
+// table slot `slot`, float field h4 of those sites.
 template <bool BIM>
 __device__ __forceinline__ void decide_block(const Words4 &w, const PairSlices &ps, int j, uint32_t slot,
-                                             const float4 &h4, uint32_t &flip, uint32_t (&fk)[4]) {
+                                             const float4 &h4, Flips<BIM> &fl) {
   const uint32_t offs = block_offsets<BIM>(ps, j);
+  if constexpr (BIM) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const uint32_t a = __byte_perm(offs, slot, 0x7650u | (uint32_t)k);
-    if (BIM) {
-      if (accept_table(w.w[k], lds_u32(a))) flip |= 1u << (8 * k + j);
-    } else {
-      const float hk = k == 0 ? h4.x : k == 1 ? h4.y : k == 2 ? h4.z : h4.w;
-      const float2 e = lds_f2(a);
-      fk[k] = __funnelshift_l(accept_float_sign(w.w[k], e.x, hk, e.y), fk[k], 1);
-    }
+    for (int k = 0; k < 4; ++k) collect_reject(w.w[k], lds_u32(__byte_perm(offs, slot, 0x7650u | (uint32_t)k)), fl.f[k]);
+  } else {
+    float2 e[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) e[k] = lds_f2(__byte_perm(offs, slot, 0x7650u | (uint32_t)k));
+    const uint2 a = accept_float_signs(w.w[0], w.w[1], e[0], e[1], h4.x, h4.y);
+    const uint2 b = accept_float_signs(w.w[2], w.w[3], e[2], e[3], h4.z, h4.w);
+    fl.f[0] |= prmt(a.x, a.y, 0x00FBu) & (0x00000101u << j);
+    fl.f[0] |= prmt(b.x, b.y, 0xFB00u) & (0x01010000u << j);
   }
 }
 
@@ -558,13 +582,13 @@ __device__ __forceinline__ uint32_t deposit_nibbles(uint32_t x) {
 // replicas of group grp: neighbour counts from the other colour's words, one Philox block per
 // (block j, replica) with counter (8 wq + j, r, ctr2, tag), decisions, and the flipped words
 // written back.  Only the blocks with their bit set in PAT are updated (0xFF: all; otherwise four
-// of them, whose float-field sign bits are collected side by side and then moved to their bytes'
-// bit j).  Replicas past the end of a partial group repeat the last one; only their write is
+// of them, whose bimodal bits are collected side by side and then moved to their bytes' bit j).  Replicas past the end of a partial group repeat the last one; only their write is
 // skipped.
 template <int L, int S, int GT, bool BIM, uint32_t PAT>
 __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int c, int zl, int iw, int z0, int grp,
                                             int gact, int r0, uint32_t ctr2, uint32_t tag, uint32_t slot0,
-                                            const float4 *__restrict__ field4, int up_rank, int dn_rank) {
+                                            const float4 *__restrict__ field4, int up_rank, int dn_rank,
+                                            const PhiloxKeys &keys) {
   static_assert(PAT == 0xFFu || __builtin_popcount(PAT) == 4, "a pass updates all blocks or four of them");
   using Gm = BitsGeom<L>;
   constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P;
@@ -578,7 +602,8 @@ __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int
       if ((PAT >> j) & 1u) hh4[j] = __ldg(field4 + field4_index(c, wq, j, WPAD));
   }
   const uint32_t p0 = parity0_mask<L>(c, z, iw);
-  uint32_t c0[GT], c1[GT], c2[GT], sf[GT], flip[GT];
+  uint32_t c0[GT], c1[GT], c2[GT], sf[GT];
+  Flips<BIM> fl[GT];
 #pragma unroll
   for (int gg = 0; gg < GT; ++gg) {
     const int g = min(grp * GT + gg, gact - 1);
@@ -586,18 +611,12 @@ __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int
     neighbour_words<L, S>(sp + ((size_t)g * 2 + (c ^ 1)) * WC, zl, iw, p0, up_rank, dn_rank, nb);
     count6(nb[0], nb[1], nb[2], nb[3], nb[4], nb[5], c0[gg], c1[gg], c2[gg]);
     sf[gg] = sp[((size_t)g * 2 + c) * WC + wl];
-    flip[gg] = 0u;
+    fl[gg].clear();
   }
   const uint32_t fb = BIM ? v.hbits[(int64_t)c * W + wq] : 0u;
   PairSlices ps[GT];
 #pragma unroll
   for (int gg = 0; gg < GT; ++gg) ps[gg] = make_pairs(c0[gg], c1[gg], c2[gg], sf[gg], fb);
-  // float field: flip = fk[k] << 8k once all blocks are done
-  uint32_t fk[GT][4];
-#pragma unroll
-  for (int gg = 0; gg < GT; ++gg)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) fk[gg][k] = 0u;
 #pragma unroll kBlockUnroll
   for (int jj = 0; jj < 8; ++jj) {
     const int j = 7 - jj;
@@ -605,23 +624,17 @@ __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int
 #pragma unroll
       for (int gg = 0; gg < GT; ++gg) {
         const int g = min(grp * GT + gg, gact - 1);
-        const Words4 w = philox10(v.seed, v.realization, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), ctr2, tag);
-        decide_block<BIM>(w, ps[gg], j, slot0 + (uint32_t)g * kTabSlot, hh4[j], flip[gg], fk[gg]);
+        const Words4 w = philox_keyed(keys, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), ctr2, tag);
+        decide_block<BIM>(w, ps[gg], j, slot0 + (uint32_t)g * kTabSlot, hh4[j], fl[gg]);
       }
-    }
-  }
-  if (!BIM) {
-#pragma unroll
-    for (int gg = 0; gg < GT; ++gg) {
-      flip[gg] = fk[gg][0] | (fk[gg][1] << 8) | (fk[gg][2] << 16) | (fk[gg][3] << 24);
-      if (PAT != 0xFFu) flip[gg] = deposit_nibbles<PAT>(flip[gg]);
     }
   }
 #pragma unroll
   for (int gg = 0; gg < GT; ++gg) {
     const int g = grp * GT + gg;
     if (GT > 1 && g >= gact) continue;
-    sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ flip[gg];
+    const uint32_t flip = BIM && PAT != 0xFFu ? deposit_nibbles<PAT>(~fl[gg].rejects()) : fl[gg].template word<8>();
+    sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ flip;
   }
 }
 
@@ -661,7 +674,7 @@ __device__ __forceinline__ void copy_slab(const RealView &v, uint32_t *sp, int r
 template <int L, int S, bool BIM, int BG>
 __device__ __forceinline__ void split_unit(const RealView &v, uint32_t *sp, int c, int g, int wl, int z0, int r0,
                                            uint32_t sweep, uint32_t tag, uint32_t slot, const float4 *__restrict__ field4,
-                                           int up_rank, int dn_rank) {
+                                           int up_rank, int dn_rank, const PhiloxKeys &keys) {
   using Gm = BitsGeom<L>;
   constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P;
   constexpr int64_t WPAD = (W + 31) / 32 * 32;
@@ -678,15 +691,15 @@ __device__ __forceinline__ void split_unit(const RealView &v, uint32_t *sp, int 
   uint32_t *self = sp + ((size_t)g * 2 + c) * WC + wl;
   const uint32_t fb = BIM ? v.hbits[(int64_t)c * W + wq] : 0u;
   const PairSlices ps = make_pairs(c0, c1, c2, *self, fb);
-  uint32_t flip = 0u, fk[4] = {0u, 0u, 0u, 0u};
+  Flips<BIM> fl;
+  fl.clear();
 #pragma unroll
-  for (int jj = 0; jj < 2; ++jj) {  // block 2 BG + 1, then 2 BG: the sign collectors end with block 2 BG at bit 0
+  for (int jj = 0; jj < 2; ++jj) {  // block 2 BG + 1, then 2 BG
     const int j = 2 * BG + 1 - jj;
-    const Words4 w = philox10(v.seed, v.realization, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), sweep, tag);
-    decide_block<BIM>(w, ps, j, slot, h[1 - jj], flip, fk);
+    const Words4 w = philox_keyed(keys, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), sweep, tag);
+    decide_block<BIM>(w, ps, j, slot, h[1 - jj], fl);
   }
-  if (!BIM) flip = (fk[0] | (fk[1] << 8) | (fk[2] << 16) | (fk[3] << 24)) << (2 * BG);
-  atomicXor(self, flip);
+  atomicXor(self, BIM ? fl.template word<2>() << (2 * BG) : fl.template word<8>());
 }
 
 // One exchange interval of replicas [r0, r0 + gact) of realization v, slab `rank` of S: load into
@@ -699,7 +712,8 @@ __device__ __forceinline__ void split_unit(const RealView &v, uint32_t *sp, int 
 // threads with a quarter of the Philox work each.
 template <int L, int S, int GT, bool BIM, bool XI = false, bool I8 = false, int NS = 1>
 __device__ __forceinline__ void bits_interval(const RealView &v, int G, int r0, int gact, int rank, uint32_t sweep0,
-                                              int nsw, const float4 *__restrict__ field4, const ExchArgs &xa) {
+                                              int nsw, const float4 *__restrict__ field4, const ExchArgs &xa,
+                                              const PhiloxKeys &keys) {
   using Gm = BitsGeom<L>;
   constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P;
   constexpr int64_t WPAD = (W + 31) / 32 * 32;
@@ -747,10 +761,10 @@ __device__ __forceinline__ void bits_interval(const RealView &v, int G, int r0, 
           if (!RFIM_DCHECK(xa.err, g < gact && wl < WC, kDbgLattice)) continue;
           const uint32_t slot = slot0 + (uint32_t)g * kTabSlot;
           switch (bg) {  // warp-uniform
-            case 0: split_unit<L, S, BIM, 0>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank); break;
-            case 1: split_unit<L, S, BIM, 1>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank); break;
-            case 2: split_unit<L, S, BIM, 2>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank); break;
-            default: split_unit<L, S, BIM, 3>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank); break;
+            case 0: split_unit<L, S, BIM, 0>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank, keys); break;
+            case 1: split_unit<L, S, BIM, 1>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank, keys); break;
+            case 2: split_unit<L, S, BIM, 2>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank, keys); break;
+            default: split_unit<L, S, BIM, 3>(v, sp, c, g, wl, z0, r0, sweep, tag, slot, field4, up_rank, dn_rank, keys); break;
           }
         }
         sync_slabs<S>();
@@ -769,7 +783,8 @@ __device__ __forceinline__ void bits_interval(const RealView &v, int G, int r0, 
           for (int j = 0; j < 8; ++j) hh4[j] = __ldg(field4 + field4_index(c, wq, j, WPAD));
         }
         const uint32_t p0 = parity0_mask<L>(c, z, iw);
-        uint32_t c0[GT], c1[GT], c2[GT], sf[GT], flip[GT];
+        uint32_t c0[GT], c1[GT], c2[GT], sf[GT];
+        Flips<BIM> fl[GT];
 #pragma unroll
         for (int gg = 0; gg < GT; ++gg) {
           const int g = min(grp * GT + gg, gact - 1);
@@ -777,38 +792,28 @@ __device__ __forceinline__ void bits_interval(const RealView &v, int G, int r0, 
           neighbour_words<L, S>(sp + ((size_t)g * 2 + (c ^ 1)) * WC, zl, iw, p0, up_rank, dn_rank, nb);
           count6(nb[0], nb[1], nb[2], nb[3], nb[4], nb[5], c0[gg], c1[gg], c2[gg]);
           sf[gg] = sp[((size_t)g * 2 + c) * WC + wl];
-          flip[gg] = 0u;
+          fl[gg].clear();
         }
         const uint32_t fb = BIM ? v.hbits[(int64_t)c * W + wq] : 0u;
         PairSlices ps[GT];
 #pragma unroll
         for (int gg = 0; gg < GT; ++gg) ps[gg] = make_pairs(c0[gg], c1[gg], c2[gg], sf[gg], fb);
-        // replicas past the end of a partial group repeat the last one; only their write is skipped.
-        // Float field: flip = fk[k] << 8k once all blocks are done.
-        uint32_t fk[GT][4];
-#pragma unroll
-        for (int gg = 0; gg < GT; ++gg)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) fk[gg][k] = 0u;
+        // replicas past the end of a partial group repeat the last one; only their write is skipped
 #pragma unroll kBlockUnroll
         for (int jj = 0; jj < 8; ++jj) {
           const int j = 7 - jj;
 #pragma unroll
           for (int gg = 0; gg < GT; ++gg) {
             const int g = min(grp * GT + gg, gact - 1);
-            const Words4 w = philox10(v.seed, v.realization, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), sweep, tag);
-            decide_block<BIM>(w, ps[gg], j, slot0 + (uint32_t)g * kTabSlot, hh4[j], flip[gg], fk[gg]);
+            const Words4 w = philox_keyed(keys, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), sweep, tag);
+            decide_block<BIM>(w, ps[gg], j, slot0 + (uint32_t)g * kTabSlot, hh4[j], fl[gg]);
           }
-        }
-        if (!BIM) {
-#pragma unroll
-          for (int gg = 0; gg < GT; ++gg) flip[gg] = fk[gg][0] | (fk[gg][1] << 8) | (fk[gg][2] << 16) | (fk[gg][3] << 24);
         }
 #pragma unroll
         for (int gg = 0; gg < GT; ++gg) {
           const int g = grp * GT + gg;
           if (GT > 1 && g >= gact) continue;
-          sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ flip[gg];
+          sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ fl[gg].template word<8>();
         }
       }
       sync_slabs<S>();
@@ -828,12 +833,13 @@ __device__ __forceinline__ void bits_interval(const RealView &v, int G, int r0, 
 
 template <int L, int S, int GT, bool BIM, int NT, bool I8 = false, int NS = 1>
 __global__ void __launch_bounds__(NT) k_sweeps_bits(RealView v, int32_t G, uint32_t sweep0, int32_t nsw,
-                                                     const float4 *__restrict__ field4, ExchArgs xa) {
+                                                     const float4 *__restrict__ field4, ExchArgs xa,
+                                                     const __grid_constant__ PhiloxKeys keys) {
   const int rank = S > 1 ? (int)cluster_rank() : 0;
   const int r0 = (int)(blockIdx.x / S) * G;
   const int gact = min(G, v.R - r0);
   xa.expected = gridDim.x;
-  bits_interval<L, S, GT, BIM, false, I8, NS>(v, G, r0, gact, rank, sweep0, nsw, field4, xa);
+  bits_interval<L, S, GT, BIM, false, I8, NS>(v, G, r0, gact, rank, sweep0, nsw, field4, xa, keys);
 }
 
 }  // namespace rfim

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     }
   };
   copy_planes(0, PZ + 2, true);
-  if (ok) tab_fill<BIM>(v, tab, slot0, gact, [&](int g) { return r0 + g; });
+  if (ok) tab_fill<BIM, false>(v, tab, slot0, gact, [&](int g) { return r0 + g; });
   if (xa.enabled && ok)
     for (int r = tid; r < R; r += nt) {
       xs.t2r[r] = v.t2r[r];
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
       return -xa.J * (double)B - (BIM ? xa.h * (double)F : __longlong_as_double(F));
     };
     if (ok) exchange_from_records<!BIM, false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, energy_of);
-    if (ok && iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
+    if (ok && iv + 1 < n_iv) tab_fill_temps<BIM, false>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
   if (S > 1) sync_slabs<2>();  // a CTA stays until its neighbours' pushes have landed

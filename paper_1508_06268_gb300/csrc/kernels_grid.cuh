@@ -68,14 +68,15 @@ __device__ __forceinline__ bool grid_wait(const unsigned *prog, int k, unsigned 
   return false;
 }
 
-// Hot loop of a round range of a half-sweep of the grid-wide kernel, kept out of line so that
-// its register allocation does not carry the kernel's set-up and schedule state.
+// Arguments of the loop over a round range of a half-sweep, in shared memory, so that its register
+// allocation does not carry the kernel's set-up and schedule state.  The loop is inlined: a function
+// of its own could not read the round keys from the constant bank (it formed them in registers).
 struct GridHot {
   uint32_t *lat;
   const float4 *field4;
   uint32_t *bits;
   const uint32_t *hbits;
-  uint32_t seed, realization, slot0;
+  uint32_t slot0;
   int nb_items, np;
   unsigned *err;
   const uint32_t *desc;
@@ -85,7 +86,8 @@ struct GridHot {
 };
 
 template <int L, bool BIM, int GG, int GTI>
-__device__ __noinline__ void grid_process(const GridHot *hot_s, int i0, int i1, int c, uint32_t sweep, uint32_t tag) {
+__device__ __forceinline__ void grid_process(const GridHot *hot_s, int i0, int i1, int c, uint32_t sweep, uint32_t tag,
+                                             const PhiloxKeys &keys) {
   const GridHot hot = *hot_s;  // from shared memory: the caller keeps none of it in registers
   constexpr int PW = L * L / 64, W = L * L * L / 64;
   constexpr int64_t WPAD = (W + 31) / 32 * 32;
@@ -112,7 +114,8 @@ __device__ __noinline__ void grid_process(const GridHot *hot_s, int i0, int i1, 
     }
     const uint32_t p0 = parity0_mask<L>(c, z, w);
     PairSlices ps[GTI];
-    uint32_t sf[GTI], flip[GTI], fk[GTI][4];
+    uint32_t sf[GTI];
+    Flips<BIM> fl[GTI];
     const uint32_t fb = BIM ? hot.hbits[(int64_t)c * W + wq] : 0u;
 #pragma unroll
     for (int gg = 0; gg < GTI; ++gg) {
@@ -125,9 +128,7 @@ __device__ __noinline__ void grid_process(const GridHot *hot_s, int i0, int i1, 
       count6(nbw[0], nbw[1], nbw[2], nbw[3], nbw[4], nbw[5], c0, c1, c2);
       sf[gg] = Pl[(g * 2 + c) * cs + w];
       ps[gg] = make_pairs(c0, c1, c2, sf[gg], fb);
-      flip[gg] = 0u;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) fk[gg][q] = 0u;
+      fl[gg].clear();
     }
     const int r0 = hot.pc[p].g * GG;
 #pragma unroll kBlockUnroll
@@ -136,15 +137,14 @@ __device__ __noinline__ void grid_process(const GridHot *hot_s, int i0, int i1, 
 #pragma unroll
       for (int gg = 0; gg < GTI; ++gg) {
         const int g = min(gb + gg, gact - 1);
-        const Words4 wd = philox10(hot.seed, hot.realization, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), sweep, tag);
-        decide_block<BIM>(wd, ps[gg], j, hot.slot0 + (uint32_t)(p * GG + g) * kTabSlot, hh4[j], flip[gg], fk[gg]);
+        const Words4 wd = philox_keyed(keys, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), sweep, tag);
+        decide_block<BIM>(wd, ps[gg], j, hot.slot0 + (uint32_t)(p * GG + g) * kTabSlot, hh4[j], fl[gg]);
       }
     }
 #pragma unroll
     for (int gg = 0; gg < GTI; ++gg) {
       if (gb + gg >= gact) continue;
-      if (!BIM) flip[gg] = fk[gg][0] | (fk[gg][1] << 8) | (fk[gg][2] << 16) | (fk[gg][3] << 24);
-      const uint32_t nw = sf[gg] ^ flip[gg];
+      const uint32_t nw = sf[gg] ^ fl[gg].template word<8>();
       Pl[((gb + gg) * 2 + c) * cs + w] = nw;
       if (end_plane) hot.bits[((int64_t)(r0 + gb + gg) * 2 + c) * W + wq] = nw;  // publish
     }
@@ -156,7 +156,8 @@ __device__ __noinline__ void grid_process(const GridHot *hot_s, int i0, int i1, 
 // layout that carries only the end planes published during the launch.
 template <int L, bool BIM, int GG, int GTI, int NT, bool I8 = false>
 __global__ void __launch_bounds__(NT, 1) k_sweeps_grid(RealView v, GridArgs ga, uint32_t sweep0, int32_t nsw,
-                                                        const float4 *__restrict__ field4, ExchArgs xa) {
+                                                        const float4 *__restrict__ field4, ExchArgs xa,
+                                                        const __grid_constant__ PhiloxKeys keys) {
   constexpr int PW = L * L / 64, W = L * L * L / 64;
   constexpr int64_t WPAD = (W + 31) / 32 * 32;
   extern __shared__ __align__(16) uint32_t sm[];
@@ -273,8 +274,6 @@ __global__ void __launch_bounds__(NT, 1) k_sweeps_grid(RealView v, GridArgs ga, 
     hot.field4 = field4;
     hot.bits = v.bits;
     hot.hbits = v.hbits;
-    hot.seed = v.seed;
-    hot.realization = v.realization;
     hot.slot0 = slot0;
     hot.nb_items = nb * IPW;
     hot.np = np;
@@ -303,7 +302,7 @@ __global__ void __launch_bounds__(NT, 1) k_sweeps_grid(RealView v, GridArgs ga, 
       const uint32_t sweep = sweep0 + (uint32_t)(iv * nsw + (h >> 1));
       const uint32_t tag = tag_word(kTagMetro, v.stage, (uint32_t)c);
       auto process = [&](int i0, int i1) {
-        grid_process<L, BIM, GG, GTI>(&hot, i0, i1, c, sweep, tag);
+        grid_process<L, BIM, GG, GTI>(&hot, i0, i1, c, sweep, tag, keys);
       };
       // end planes (and the interior items sharing their rounds), then the progress word: the CTA
       // barrier orders every thread's end-plane stores before thread 0's gpu-scope fence and release

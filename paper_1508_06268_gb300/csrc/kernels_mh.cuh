@@ -29,7 +29,7 @@ __host__ __device__ constexpr uint32_t odd_tile_blocks(int L, int T) {
 template <int L, int S, int GT, bool BIM, int T>
 __device__ __forceinline__ void bits_interval_mh(const RealView &v, int G, int r0, int gact, int rank, uint32_t sweep0,
                                                  int nsw, const float4 *__restrict__ field4, const ExchArgs &xa,
-                                                 const MultiHit &mh) {
+                                                 const MultiHit &mh, const PhiloxKeys &keys) {
   using Gm = BitsGeom<L>;
   constexpr int P = Gm::P, PZ = L / S, WC = PZ * P;
   constexpr int RW = 64 / L;  // rows of one colour held by a word
@@ -77,10 +77,10 @@ __device__ __forceinline__ void bits_interval_mh(const RealView &v, int G, int r
             // (uniform over the warp, whose 32 words share the class)
             if ((coarse ^ cls) & 1)
               update_word<L, S, GT, BIM, ODD>(v, sp, c, zl, iw, z0, grp, gact, r0, c2, tag, slot0, field4, up_rank,
-                                              dn_rank);
+                                              dn_rank, keys);
             else
               update_word<L, S, GT, BIM, EVEN>(v, sp, c, zl, iw, z0, grp, gact, r0, c2, tag, slot0, field4, up_rank,
-                                               dn_rank);
+                                               dn_rank, keys);
           }
           sync_slabs<S>();
         }
@@ -94,12 +94,13 @@ __device__ __forceinline__ void bits_interval_mh(const RealView &v, int G, int r
 
 template <int L, int S, int GT, bool BIM, int NT, int T>
 __global__ void __launch_bounds__(NT) k_sweeps_bits_mh(RealView v, int32_t G, uint32_t sweep0, int32_t nsw,
-                                                        const float4 *__restrict__ field4, ExchArgs xa, MultiHit mh) {
+                                                        const float4 *__restrict__ field4, ExchArgs xa, MultiHit mh,
+                                                        const __grid_constant__ PhiloxKeys keys) {
   const int rank = S > 1 ? (int)cluster_rank() : 0;
   const int r0 = (int)(blockIdx.x / S) * G;
   const int gact = min(G, v.R - r0);
   xa.expected = gridDim.x;
-  bits_interval_mh<L, S, GT, BIM, T>(v, G, r0, gact, rank, sweep0, nsw, field4, xa, mh);
+  bits_interval_mh<L, S, GT, BIM, T>(v, G, r0, gact, rank, sweep0, nsw, field4, xa, mh, keys);
 }
 
 }  // namespace rfim

@@ -161,11 +161,11 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     uint32_t *self = sp + c * CW + it.same;
     const PairSlices ps = make_pairs(c0 >> it.sh, c1 >> it.sh, c2 >> it.sh, *self >> it.sh, fb);
     const uint32_t slot = slot0 + (uint32_t)it.g * kTabSlot;
-    uint32_t flip = 0u, fk[4] = {0u, 0u, 0u, 0u};
+    Flips<BIM> fl;
+    fl.clear();
 #pragma unroll
-    for (int j = NB - 1; j >= 0; --j) decide_block<BIM>(w[j], ps, j, slot, h[j], flip, fk);
-    if (!BIM) flip = fk[0] | (fk[1] << 8) | (fk[2] << 16) | (fk[3] << 24);
-    if (valid) atomicXor(self, flip << it.sh);
+    for (int j = NB - 1; j >= 0; --j) decide_block<BIM>(w[j], ps, j, slot, h[j], fl);
+    if (valid) atomicXor(self, fl.template word<NB>() << it.sh);
   };
   // After half-sweep number h of this launch (all of the CTA's updates of colour c done): the slab's
   // first and last planes into the halo planes of the slabs below and above.  Two mbarriers in turn:

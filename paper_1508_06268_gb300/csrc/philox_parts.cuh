@@ -11,8 +11,9 @@ namespace rfim {
 struct PhiloxKeys {
   uint32_t k0[10], k1[10];
 };
-inline PhiloxKeys philox_keys(uint32_t seed, uint32_t realization) {
+__host__ __device__ __forceinline__ PhiloxKeys philox_keys(uint32_t seed, uint32_t realization) {
   PhiloxKeys k;
+#pragma unroll
   for (uint32_t i = 0; i < 10; ++i) {
     k.k0[i] = seed + i * kPhiloxW0;
     k.k1[i] = realization + i * kPhiloxW1;
