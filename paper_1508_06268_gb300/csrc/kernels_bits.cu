@@ -243,6 +243,48 @@ cudaError_t prepare_multihit(const BitsPlan &plan, bool bimodal) {
 }
 
 namespace {
+// "S,G,NB,threads,r" (or m: several items per thread): a resident shape.
+bool named_resident(const char *text, ResidentShape *s) {
+  char suffix = 0;
+  if (!text || sscanf(text, "%d,%d,%d,%d,%c", &s->S, &s->G, &s->NB, &s->threads, &suffix) != 5) return false;
+  s->one = suffix == 'r';
+  return suffix == 'r' || suffix == 'm';
+}
+}  // namespace
+
+// L = 64: a pass of the cluster kernel takes about 9.3 us for up to 36 clusters of four replicas
+// (898 attempts/ns at R = 128), whatever their number; the smaller L are latency-bound at every R
+// that fits.
+cudaError_t prepare_multihit_resident(BitsPlan &plan, bool bimodal, int32_t tile, cudaStream_t st, bool *found) {
+  ResidentShape s;
+  double cycles = 0.0;
+  *found = resident_shape(plan.L, plan.Rcap, bimodal, &s, &cycles, tile) && (plan.L < 64 || cycles < 2070.0 * 9.3);
+  ResidentShape named;
+  named.T = tile;
+  if (named_resident(getenv("RFIM_BITS_PLAN"), &named) && resident_fits(plan.L, plan.Rcap, bimodal, &named)) {
+    s = named;
+    *found = true;
+  }
+  if (!*found) return cudaSuccess;
+  const size_t slots = (size_t)plan.Rcap * s.S;
+  if (slots > plan.rec_slots) {
+    uint4 *rec = nullptr;
+    cudaError_t e = cudaMalloc((void **)&rec, 2 * slots * sizeof(uint4));
+    if (e == cudaSuccess) e = cudaMemsetAsync(rec, 0, 2 * slots * sizeof(uint4), st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // also: no launch reads the former records any more
+    if (e != cudaSuccess) {
+      cudaFree(rec);
+      return e;
+    }
+    cudaFree(plan.rec);
+    plan.rec = rec;
+    plan.rec_slots = slots;
+  }
+  plan.mh_res = s;
+  return cudaSuccess;
+}
+
+namespace {
 thread_local const char *t_plan_override = nullptr;
 std::mutex g_tuned_mu;
 std::map<std::tuple<int, int, bool>, std::string> g_tuned;  // (L, R, bimodal) -> "S,G,GT,threads"
@@ -366,11 +408,8 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
   if (o) {
     int s, g, gt, th, ns = 1;
     ResidentShape named_rs;
-    char suffix = 0;
-    const bool is_res = sscanf(o, "%d,%d,%d,%d,%c", &named_rs.S, &named_rs.G, &named_rs.NB, &named_rs.threads, &suffix) == 5 &&
-                        (suffix == 'r' || suffix == 'm');
-    named_rs.one = suffix == 'r';
-    // "S,G,NB,threads,r" (or m: several items per thread): a resident shape; "S,G,GT,threads[,NS]" (NS = 4: every word split over four warps); an override that names no
+    const bool is_res = named_resident(o, &named_rs);
+    // a resident shape, or "S,G,GT,threads[,NS]" (NS = 4: every word split over four warps); an override that names no
     // instance for this L (e.g. an L=64 shape while building L=16) is ignored and the defaults stand
     const int nf = is_res ? 0 : sscanf(o, "%d,%d,%d,%d,%d", &s, &g, &gt, &th, &ns);
     const bool named = nf == 4 || nf == 5;
@@ -467,6 +506,7 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
     if (!rc && i8) rc = grab((void **)&p.gbits, (size_t)Rcap * 2 * ((size_t)L * L * L / 64) * 4, "halo words");
   }
   const size_t rec_bytes = resident ? 2 * parts * sizeof(uint4) : 0;
+  p.rec_slots = resident ? parts : 0;
   if (!rc && resident) rc = grab((void **)&p.rec, rec_bytes, "energy records");
   if (!rc && p.rec && cudaMemset(p.rec, 0, rec_bytes) != cudaSuccess) rc = -3;
   if (!rc && cudaMemset(p.counter, 0, 16) != cudaSuccess) rc = -3;
@@ -508,7 +548,7 @@ cudaError_t reset_bits_plan(const BitsPlan &plan, cudaStream_t st) {
     plan.arrive_base = 0;
   }
   if (e == cudaSuccess && plan.rec) {
-    e = cudaMemsetAsync(plan.rec, 0, 2 * (size_t)plan.Rcap * plan.S * sizeof(uint4), st);
+    e = cudaMemsetAsync(plan.rec, 0, 2 * plan.rec_slots * sizeof(uint4), st);
     plan.epoch = 0;
   }
   return e;
@@ -546,25 +586,30 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
   xa.err = plan.counter + 1;
   xa.flimb = plan.flimb;
   xa.fquant = plan.fquant;
-  if (plan.resident()) {
-    if ((mh && mh->mh > 0) || n_intervals < 1 || (!exchange && n_intervals != 1)) return cudaErrorInvalidValue;
+  const bool multihit = mh && mh->mh > 0;
+  const ResidentShape &rs = multihit ? plan.mh_res : plan.res;
+  if (rs.threads > 0 && (!multihit || rs.T == mh->tile)) {
+    if (n_intervals < 1 || (!exchange && n_intervals != 1)) return cudaErrorInvalidValue;
     if (exchange && plan.epoch >= kRecordEpochs - 1 - (uint32_t)n_intervals) {  // numbers would wrap: start again
       const cudaError_t e = reset_bits_plan(plan, st);
       if (e != cudaSuccess) return e;
     }
     ResidentArgs ra{};
-    ra.G = plan.res.G;
+    ra.G = rs.G;
+    ra.mh = multihit ? mh->mh : 0;
     ra.rcap = plan.Rcap;
     ra.n_iv = n_intervals;
     ra.epoch0 = plan.epoch + 1;
     ra.rec = plan.rec;
     ra.i8 = plan.i8;
-    const cudaError_t e = plan.res.NB ? launch_resident(v, plan.res, ra, sweep0, n_sweeps, plan.field4, xa, st)
-                                      : launch_resident_bytes(v, plan.res, ra, sweep0, n_sweeps, xa, st);
+    const cudaError_t e = rs.NB ? launch_resident(v, rs, ra, sweep0, n_sweeps, plan.field4, xa, st)
+                                : launch_resident_bytes(v, rs, ra, sweep0, n_sweeps, xa, st);
     if (e == cudaSuccess && exchange) plan.epoch += (uint32_t)n_intervals;
     return e;
   }
+  if (plan.resident()) return cudaErrorInvalidConfiguration;  // multi-hit without a shape of its own
   if (plan.S == 0) {
+    if (multihit) return cudaErrorInvalidConfiguration;
     GridFn gfn = grid_kernel_for(plan.L, plan.G, plan.GT, plan.threads, v.kind == kBimodal, plan.i8);
     if (!gfn || (plan.i8 && !plan.gbits)) return cudaErrorInvalidConfiguration;
     RealView vg = v;
@@ -608,8 +653,6 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
     return le;
   }
   if (n_intervals != 1) return cudaErrorInvalidValue;  // several intervals: grid-wide plan only
-  const bool multihit = mh && mh->mh > 0;
-  if (multihit && plan.S == 0) return cudaErrorInvalidConfiguration;
   KernelFn fn = multihit ? nullptr : kernel_for(plan.L, plan.S, plan.GT, plan.threads, v.kind == kBimodal, plan.i8, plan.NS);
   MhFn mfn = multihit ? mh_kernel_for(plan.L, plan.S, plan.GT, plan.threads, v.kind == kBimodal, mh->tile) : nullptr;
   if (!fn && !mfn) return cudaErrorInvalidConfiguration;

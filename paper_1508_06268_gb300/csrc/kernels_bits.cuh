@@ -562,9 +562,9 @@ __device__ __forceinline__ void interval_tail(const RealView &v, int G, int r0, 
 }
 
 
-// Per byte, bit b of the low nibble moves to the b-th set bit of PAT (four set bits).
+// Per byte, bit b moves to the b-th set bit of PAT; bits past their number are dropped.
 template <uint32_t PAT>
-__device__ __forceinline__ uint32_t deposit_nibbles(uint32_t x) {
+__device__ __forceinline__ uint32_t deposit_bits(uint32_t x) {
   uint32_t out = 0u;
   int b = 0;
 #pragma unroll
@@ -633,7 +633,7 @@ __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int
   for (int gg = 0; gg < GT; ++gg) {
     const int g = grp * GT + gg;
     if (GT > 1 && g >= gact) continue;
-    const uint32_t flip = BIM && PAT != 0xFFu ? deposit_nibbles<PAT>(~fl[gg].rejects()) : fl[gg].template word<8>();
+    const uint32_t flip = BIM && PAT != 0xFFu ? deposit_bits<PAT>(~fl[gg].rejects()) : fl[gg].template word<8>();
     sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ flip;
   }
 }

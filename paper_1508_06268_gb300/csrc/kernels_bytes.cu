@@ -124,7 +124,8 @@ int make_bytes_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::
   p.threads = s.threads;
   p.smem = s.smem;
   p.res = s;
-  const size_t rec_bytes = 2 * (size_t)Rcap * s.S * sizeof(uint4);
+  p.rec_slots = (size_t)Rcap * s.S;
+  const size_t rec_bytes = 2 * p.rec_slots * sizeof(uint4);
   cudaError_t e = cudaMalloc((void **)&p.rec, rec_bytes);
   if (e == cudaSuccess) e = cudaMalloc((void **)&p.counter, 16);
   if (e == cudaSuccess) e = cudaMemset(p.rec, 0, rec_bytes);

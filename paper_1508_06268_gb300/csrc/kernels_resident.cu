@@ -1,5 +1,6 @@
 // Instances, launch shapes and launcher of the resident sweep kernel (kernels_resident.cuh).
 #include <algorithm>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -52,32 +53,28 @@ int resident_ctas(const void *fn, int S, int threads, size_t smem) {
 
 namespace {
 
-using ResidentFn = void (*)(RealView, ResidentArgs, uint32_t, int32_t, const float4 *, ExchArgs);
-
-struct Instance {
-  int32_t L, S, NB, NT;
-  bool one;  // one item per thread
-  ResidentFn bim, flt;
-};
-
-template <int L, int S, int NB, int NT, bool ONE>
-constexpr Instance instance() {
-  return {L, S, NB, NT, ONE, k_resident<L, S, NB, true, NT, ONE>, k_resident<L, S, NB, false, NT, ONE>};
-}
+using Instance = ResidentInstance;
 
 const Instance kInstances[] = {
-    instance<8, 1, 1, 512, true>(),   instance<8, 1, 2, 512, true>(),   instance<8, 1, 4, 512, true>(),
-    instance<16, 1, 1, 512, true>(),  instance<16, 1, 2, 512, true>(),  instance<16, 1, 4, 512, true>(),
-    instance<16, 2, 1, 256, true>(),  instance<16, 2, 2, 256, true>(),  instance<32, 2, 4, 512, true>(),
-    instance<32, 4, 4, 256, true>(),  instance<32, 8, 2, 256, true>(),  instance<32, 1, 4, 512, false>(),
-    instance<32, 2, 4, 512, false>(), instance<64, 16, 4, 512, true>(), instance<64, 8, 4, 512, false>(),
-    instance<64, 4, 4, 512, false>(),
+    resident_instance<8, 1, 1, 512, true>(),   resident_instance<8, 1, 2, 512, true>(),   resident_instance<8, 1, 4, 512, true>(),
+    resident_instance<16, 1, 1, 512, true>(),  resident_instance<16, 1, 2, 512, true>(),  resident_instance<16, 1, 4, 512, true>(),
+    resident_instance<16, 2, 1, 256, true>(),  resident_instance<16, 2, 2, 256, true>(),  resident_instance<32, 2, 4, 512, true>(),
+    resident_instance<32, 4, 4, 256, true>(),  resident_instance<32, 8, 2, 256, true>(),  resident_instance<32, 1, 4, 512, false>(),
+    resident_instance<32, 2, 4, 512, false>(), resident_instance<64, 16, 4, 512, true>(), resident_instance<64, 8, 4, 512, false>(),
+    resident_instance<64, 4, 4, 512, false>(),
 };
 
+// The first instance of tile edge T for which f holds, or null.
+template <class F>
+const Instance *find_if(int32_t T, F f) {
+  const std::vector<Instance> &mh = resident_multihit_instances();
+  const Instance *first = T ? mh.data() : std::begin(kInstances), *last = T ? mh.data() + mh.size() : std::end(kInstances);
+  const Instance *i = std::find_if(first, last, [&](const Instance &x) { return x.T == T && f(x); });
+  return i == last ? nullptr : i;
+}
+
 const Instance *find(int32_t L, const ResidentShape &s) {
-  for (const Instance &i : kInstances)
-    if (i.L == L && i.S == s.S && i.NB == s.NB && i.one == s.one) return &i;
-  return nullptr;
+  return find_if(s.T, [&](const Instance &i) { return i.L == L && i.S == s.S && i.NB == s.NB && i.one == s.one; });
 }
 
 int slab_words(int32_t L, int32_t S) { return L / S * (L * L / 64); }
@@ -98,7 +95,7 @@ int lane_words(const Instance &i, int32_t G) {
 
 int warp_items(const Instance &i, int32_t G) {
   const int lw = lane_words(i, G), groups = (G * slab_words(i.L, i.S) + (1 << lw) - 1) >> lw;
-  return ((groups * (8 / i.NB) << lw) + 31) / 32;
+  return ((groups * ((i.T ? 4 : 8) / i.NB) << lw) + 31) / 32;
 }
 
 // Threads of a CTA: one item each up to the instance's limit, and enough to poll the records.
@@ -115,7 +112,9 @@ int cta_threads(const Instance &i, int32_t G, int32_t R) {
 double half_sweep_cycles(const Instance &i, int32_t G, int32_t R, int spread) {
   const int ctas = (R + G - 1) / G * i.S, per_sm = (ctas + spread - 1) / spread;
   const double instr = (double)per_sm * warp_items(i, G) * (4.0 * 15.0 * i.NB + (i.one ? 50.0 : 137.0));
-  return instr / 2.4 + 200.0 + 30.0 * i.NB + (i.S > 1 ? 300.0 + 400.0 * (per_sm - 1) : 0.0);
+  // (multi-hit slabs of whole tiles exchange halos once per visit, not per pass)
+  const bool halos = i.S > 1 && !(i.T && i.L / i.S % i.T == 0);
+  return instr / 2.4 + 200.0 + 30.0 * i.NB + (halos ? 300.0 + 400.0 * (per_sm - 1) : 0.0);
 }
 
 struct Candidate {
@@ -125,10 +124,10 @@ struct Candidate {
 };
 
 // Every instance with every group size, the fastest by estimate first.
-std::vector<Candidate> candidates(int32_t L, int32_t R, bool bimodal) {
+std::vector<Candidate> candidates(int32_t L, int32_t R, bool bimodal, int32_t T = 0) {
   std::vector<Candidate> all;
-  for (const Instance &i : kInstances) {
-    if (i.L != L) continue;
+  find_if(T, [&](const Instance &i) {
+    if (i.L != L) return false;
     const int spread = resident_ctas((const void *)(bimodal ? i.bim : i.flt), i.S, i.NT, kOneCtaSmem);
     for (int32_t G = 1; spread > 0 && G <= std::min(R, 64); ++G) {
       if (i.one && 32 * warp_items(i, G) > i.NT) break;
@@ -137,10 +136,12 @@ std::vector<Candidate> candidates(int32_t L, int32_t R, bool bimodal) {
       c.shape.G = G;
       c.shape.NB = i.NB;
       c.shape.one = i.one;
+      c.shape.T = i.T;
       c.shape.threads = cta_threads(i, G, R);
       all.push_back(c);
     }
-  }
+    return false;
+  });
   std::stable_sort(all.begin(), all.end(), [](const Candidate &a, const Candidate &b) { return a.cycles < b.cycles; });
   return all;
 }
@@ -157,8 +158,8 @@ bool resident_fits(int32_t L, int32_t R, bool bimodal, ResidentShape *s) {
   return ctas <= resident_ctas((const void *)(bimodal ? i->bim : i->flt), s->S, s->threads, s->smem);
 }
 
-bool resident_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles) {
-  for (const Candidate &c : candidates(L, R, bimodal)) {
+bool resident_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles, int32_t T) {
+  for (const Candidate &c : candidates(L, R, bimodal, T)) {
     ResidentShape s = c.shape;
     if (!resident_fits(L, R, bimodal, &s)) continue;
     *out = s;

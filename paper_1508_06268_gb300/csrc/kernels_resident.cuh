@@ -21,6 +21,14 @@
 //   - the exchange step gathers the energies as records (exchange_records.cuh) instead of one
 //     launch per interval with an arrival counter and a last CTA that takes the step alone, and
 //     the measurement of temperature k is added by CTA k mod P.
+//
+// T > 0: the multi-hit double checkerboard (Sec. 3.2; see kernels_mh.cuh for the order of the passes)
+// with tiles of edge T.  A pass updates half of the blocks of a colour, so it is even shorter, and
+// the four blocks of a word in tiles of even x index and the four in odd ones are updated in turn
+// by the same items: an item is NB of four.  Where slabs are whole tiles the halos a visit reads are
+// frozen, so the slabs exchange both colours once per visit instead of one colour per pass.
+// Per pass, against one launch per interval with a cluster barrier per pass (us): L = 16, R = 32 1.43 -> 0.32,
+// L = 32, R = 40 2.06 -> 0.81 (tiles of 8) and 0.85 (of 16), R = 140 2.38 -> 1.42, L = 64, R = 14 10.0 -> 1.34.
 #pragma once
 #include <cstdint>
 
@@ -39,6 +47,7 @@ struct ResidentArgs {
   uint4 *rec;       // [2][rcap * S] energy records
   int32_t i8;       // the realization is stored as bytes (v.spins8) and staged as bits
   int32_t lw;       // log2 of the words whose items of one part are neighbouring threads (ONE; else 5)
+  int32_t mh;       // passes per tile visit (T > 0)
 };
 
 // Planes of a slab in shared memory: with S > 1 a halo plane before and after the slab's own.
@@ -51,26 +60,46 @@ __host__ __device__ constexpr int resident_chunks() {
   return 2 * (L / S) * (L * L / 64) >= 32 ? 2 * (L / S) * (L * L / 64) / 32 : 1;
 }
 
-// One item: word iw of plane zl of replica g of the slab, blocks sh .. sh + NB - 1 of it.
+// Items of a word: its eight blocks, or the four that one pass of the double checkerboard updates,
+// by NB.
+template <int NB, int T>
+__host__ __device__ constexpr int resident_parts() { return (T ? 4 : 8) / NB; }
+
+// Block j of an item relative to its first one; with tiles of edge T the blocks of every other run of T / 8.
+template <int NB, int T>
+__host__ __device__ constexpr int item_block(int j) { return T == 0 ? j : j / (T / 8) * (T / 4) + j % (T / 8); }
+template <int NB, int T>
+__host__ __device__ constexpr uint32_t item_pattern() {
+  uint32_t m = 0u;
+  for (int j = 0; j < NB; ++j) m |= 1u << item_block<NB, T>(j);
+  return m;
+}
+
+// One item: word iw of plane zl of replica g of the slab, blocks sh + item_block(0 .. NB - 1) of it (T > 0:
+// sh for the tiles of even x index, T / 8 further on for the odd ones).
 template <int NB>
 struct ResidentItem {
   int g, z, sh;
+  int odd;                        // T > 0: parity of y / T + z / T
   int64_t wq;                     // word within its colour
   int same, next, prev, up, down; // word indices in the replica's colour-0 planes
   uint32_t p0;                    // row-parity mask of colour 0 (colour 1: its complement)
 };
 
-template <int L, int S, int NB, bool BIM, int NT, bool ONE>
+template <int L, int S, int NB, bool BIM, int NT, bool ONE, int T = 0>
 __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_constant__ ResidentArgs ra, uint32_t sweep0,
                                                  int32_t nsw, const float4 *__restrict__ field4, const ExchArgs xa) {
   using Gm = BitsGeom<L>;
-  constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P, NP = 8 / NB;
+  constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P, NP = resident_parts<NB, T>();
   constexpr int CW = resident_planes<L, S>() * P;  // words of one colour of one replica, halos included
   constexpr int Z1 = S > 1 ? 1 : 0;                // the slab's first own plane
   constexpr int64_t WPAD = (W + 31) / 32 * 32;
   constexpr int SEG = 2 * WC < 32 ? 2 * WC : 32, NCH = resident_chunks<L, S>();
   static_assert(2 * WC >= 16, "a slab of one replica fills at least half a warp");
+  constexpr bool WHOLE_TILES = T > 0 && PZ % (T ? T : 1) == 0;  // no tile is cut by the slabs
   static_assert(S == 1 || P % 4 == 0, "halo planes are pushed 16 bytes at a time");
+  static_assert(T == 0 || (T % 8 == 0 && L % (2 * T) == 0 && NB <= 4 && (NB >= T / 8 || T / 8 % NB == 0)),
+                "an item's blocks lie in tiles of one x parity");
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ __align__(8) uint64_t mbar[2];  // halos pushed after even / odd half-sweeps
   const int rank = S > 1 ? (int)cluster_rank() : 0;
@@ -132,7 +161,8 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     const int fw = ((item >> lw) / NP << lw) + (item & ((1 << lw) - 1));
     *valid = fw < words;
     const int f = *valid ? fw : 0;  // a thread without an item repeats the first one and drops its flips
-    it.sh = (item >> lw) % NP * NB;
+    const int part = (item >> lw) % NP * NB;  // the item's first block (T > 0: among the four of a pass)
+    it.sh = item_block<1, T>(part);
     it.g = f / WC;
     const int wl = f % WC, zl = wl / P, iw = wl % P;
     it.z = z0 + zl;
@@ -144,41 +174,50 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     it.up = S > 1 ? it.same + P : base + (zl + 1) % L * P + iw;
     it.down = S > 1 ? it.same - P : base + (zl + L - 1) % L * P + iw;
     it.p0 = parity0_mask<L>(0, it.z, iw);
+    it.odd = T ? ((iw * (64 / L)) / (T ? T : 1) + it.z / (T ? T : 1)) & 1 : 0;
     return it;
   };
-  auto field_of = [&](const ResidentItem<NB> &it, int c, float4 (&h)[NB]) {
+  // first block of the item in the tiles of coarse colour `coarse` (T = 0: one set of blocks)
+  auto first_block = [&](const ResidentItem<NB> &it, int coarse) { return it.sh + (T ? ((coarse ^ it.odd) & 1) * (T / 8) : 0); };
+  auto parts_of = [&](const ResidentItem<NB> &it, int coarse) {
+    return block_parts<NB>(ra.keys, v.stage, (uint32_t)(8 * it.wq + first_block(it, coarse)), [](int j) { return item_block<NB, T>(j); });
+  };
+  auto field_of = [&](const ResidentItem<NB> &it, int sh, int c, float4 (&h)[NB]) {
 #pragma unroll
     for (int j = 0; j < NB; ++j)
-      h[j] = BIM ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(field4 + field4_index(c, it.wq, it.sh + j, WPAD));
+      h[j] = BIM ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(field4 + field4_index(c, it.wq, sh + item_block<NB, T>(j), WPAD));
   };
-  auto field_bits = [&](const ResidentItem<NB> &it, int c) { return BIM ? v.hbits[(int64_t)c * W + it.wq] >> it.sh : 0u; };
-  // decisions of one item of colour c from its random words, xored into its word
-  auto update = [&](const ResidentItem<NB> &it, int c, const Words4 (&w)[NB], const float4 (&h)[NB], uint32_t fb, bool valid) {
+  auto field_bits = [&](const ResidentItem<NB> &it, int c) { return BIM ? v.hbits[(int64_t)c * W + it.wq] : 0u; };
+  // decisions of one item of colour c, first block sh, from its random words, xored into its word
+  auto update = [&](const ResidentItem<NB> &it, int sh, int c, const Words4 (&w)[NB], const float4 (&h)[NB], uint32_t fb, bool valid) {
     const uint32_t *O = sp + (c ^ 1) * CW;
     uint32_t A, B, C, D, c0, c1, c2;
     nb_xy<L>(O[it.same], O[it.next], O[it.prev], c ? ~it.p0 : it.p0, A, B, C, D);
     count6(A, B, C, D, O[it.up], O[it.down], c0, c1, c2);
     uint32_t *self = sp + c * CW + it.same;
-    const PairSlices ps = make_pairs(c0 >> it.sh, c1 >> it.sh, c2 >> it.sh, *self >> it.sh, fb);
+    const PairSlices ps = make_pairs(c0 >> sh, c1 >> sh, c2 >> sh, *self >> sh, fb >> sh);
     const uint32_t slot = slot0 + (uint32_t)it.g * kTabSlot;
     Flips<BIM> fl;
     fl.clear();
 #pragma unroll
-    for (int j = NB - 1; j >= 0; --j) decide_block<BIM>(w[j], ps, j, slot, h[j], fl);
-    if (valid) atomicXor(self, fl.template word<NB>() << it.sh);
+    for (int j = NB - 1; j >= 0; --j) decide_block<BIM>(w[j], ps, item_block<NB, T>(j), slot, h[j], fl);
+    uint32_t flip = fl.template word<NB>();
+    if (BIM && T > 0) flip = deposit_bits<item_pattern<NB, T>()>(flip);
+    if (valid) atomicXor(self, flip << sh);
   };
   // After half-sweep number h of this launch (all of the CTA's updates of colour c done): the slab's
   // first and last planes into the halo planes of the slabs below and above.  Two mbarriers in turn:
   // a neighbour can push half-sweep h + 2 only after it has this slab's push of h + 1, which
-  // follows this slab's wait for h.
-  auto push_halos = [&](int c, uint32_t h) {
+  // follows this slab's wait for h.  (WHOLE_TILES: both colours after tile visit number h.)
+  auto push_halos = [&](int colour, uint32_t h) {
+    constexpr int NC = WHOLE_TILES ? 2 : 1;
     const uint32_t bar = mbar0 + 8 * (h & 1u);
     constexpr int VEC = P >= 4 ? P / 4 : 1;
     if (tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)(gact * 2 * P * 4))
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)(gact * 2 * NC * P * 4))
                    : "memory");
-    for (int t = tid; t < gact * 2 * VEC; t += nt) {
-      const int g = t / (2 * VEC), side = t / VEC & 1, q = t % VEC * 4;
+    for (int t = tid; t < gact * 2 * NC * VEC; t += nt) {
+      const int g = t / (2 * NC * VEC), c = NC == 2 ? t / (2 * VEC) & 1 : colour, side = t / VEC & 1, q = t % VEC * 4;
       const uint32_t peer = (uint32_t)(rank + (side ? 1 : S - 1)) % S;
       const int from = (g * 2 + c) * CW + (side ? PZ : 1) * P + q, to = (g * 2 + c) * CW + (side ? 0 : PZ + 1) * P + q;
       const uint4 x = *reinterpret_cast<const uint4 *>(sp + from);
@@ -192,18 +231,22 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
 
   bool valid;
   const ResidentItem<NB> own = decode(tid, ONE ? ra.lw : 5, &valid);
-  BlockParts<NB> bp;
-  float4 hown[2][NB];
+  constexpr int SETS = T ? 2 : 1;  // sets of blocks: one per coarse colour
+  BlockParts<NB> bp[SETS];
+  float4 hown[SETS][2][NB];
   uint32_t fbown[2] = {0u, 0u};
   Words4 w[NB];
   if (ONE) {
-    bp = block_parts<NB>(ra.keys, v.stage, (uint32_t)(8 * own.wq + own.sh));
+#pragma unroll
+    for (int k = 0; k < SETS; ++k) bp[k] = parts_of(own, k);
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      if (NB <= 2) field_of(own, c, hown[c]);
+#pragma unroll
+      for (int k = 0; k < SETS; ++k)
+        if (NB <= 2) field_of(own, first_block(own, k), c, hown[k][c]);
       fbown[c] = field_bits(own, c);
     }
-    if (S == 1) philox_words<NB>(ra.keys, bp, 0, (uint32_t)(r0 + own.g), sweep0, w);
+    if (S == 1 && !T) philox_words<NB>(ra.keys, bp[0], 0, (uint32_t)(r0 + own.g), sweep0, w);
   }
 
   const int n_iv = xa.enabled ? ra.n_iv : 1;
@@ -211,21 +254,63 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   for (int iv = 0; iv < n_iv; ++iv) {
 #pragma unroll 1
     for (int s = 0; s < nsw; ++s, ++sweep) {
+      if constexpr (T > 0) {
+#pragma unroll
+        for (int coarse = 0; coarse < 2; ++coarse) {
+#pragma unroll 1
+          for (int hit = 0; hit < ra.mh; ++hit) {
+            const uint32_t ctr = sweep * (uint32_t)ra.mh + (uint32_t)hit;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              // WHOLE_TILES: the halos of a visit arrive before its first pass and leave after its last
+              const bool wait = S > 1 && h > 0 && (!WHOLE_TILES || (hit == 0 && c == 0));
+              const bool push = S > 1 && (!WHOLE_TILES || (hit == ra.mh - 1 && c == 1));
+              if (ONE) {
+                const int sh = first_block(own, coarse);
+                if (NB > 2) field_of(own, sh, c, hown[coarse][c]);
+                philox_words<NB>(ra.keys, bp[coarse], c, (uint32_t)(r0 + own.g), ctr, w);
+                if (wait) wait_halos(h - 1);
+                update(own, sh, c, w, hown[coarse][c], fbown[c], valid);
+              } else {
+#pragma unroll 1
+                for (int item = tid; item < (words + 31) / 32 * 32 * NP; item += nt) {
+                  bool in;
+                  const ResidentItem<NB> it = decode(item, 5, &in);
+                  const int sh = first_block(it, coarse);
+                  float4 hf[NB];
+                  field_of(it, sh, c, hf);
+                  const uint32_t fb = field_bits(it, c);
+                  bp[0] = parts_of(it, coarse);
+                  philox_words<NB>(ra.keys, bp[0], c, (uint32_t)(r0 + it.g), ctr, w);
+                  if (wait && item == tid) wait_halos(h - 1);
+                  update(it, sh, c, w, hf, fb, in);
+                }
+              }
+              __syncthreads();
+              if (push) {
+                push_halos(c, h);
+                ++h;
+              }
+            }
+          }
+        }
+        continue;
+      }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         if (ONE && S == 1) {
-          if (NB > 2) field_of(own, c, hown[c]);
+          if (NB > 2) field_of(own, own.sh, c, hown[0][c]);
           Words4 next[NB];
-          philox_words<NB>(ra.keys, bp, c ^ 1, (uint32_t)(r0 + own.g), sweep + (uint32_t)c, next);
-          update(own, c, w, hown[c], fbown[c], valid);
+          philox_words<NB>(ra.keys, bp[0], c ^ 1, (uint32_t)(r0 + own.g), sweep + (uint32_t)c, next);
+          update(own, own.sh, c, w, hown[0][c], fbown[c], valid);
 #pragma unroll
           for (int j = 0; j < NB; ++j) w[j] = next[j];
           __syncthreads();
         } else if (ONE) {
-          if (NB > 2) field_of(own, c, hown[c]);
-          philox_words<NB>(ra.keys, bp, c, (uint32_t)(r0 + own.g), sweep, w);
+          if (NB > 2) field_of(own, own.sh, c, hown[0][c]);
+          philox_words<NB>(ra.keys, bp[0], c, (uint32_t)(r0 + own.g), sweep, w);
           if (h > 0) wait_halos(h - 1);
-          update(own, c, w, hown[c], fbown[c], valid);
+          update(own, own.sh, c, w, hown[0][c], fbown[c], valid);
           __syncthreads();
           push_halos(c, h);
         } else {
@@ -233,12 +318,12 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
             bool in;
             const ResidentItem<NB> it = decode(item, 5, &in);
             float4 hf[NB];
-            field_of(it, c, hf);
+            field_of(it, it.sh, c, hf);
             const uint32_t fb = field_bits(it, c);
-            bp = block_parts<NB>(ra.keys, v.stage, (uint32_t)(8 * it.wq + it.sh));
-            philox_words<NB>(ra.keys, bp, c, (uint32_t)(r0 + it.g), sweep, w);
+            bp[0] = parts_of(it, 0);
+            philox_words<NB>(ra.keys, bp[0], c, (uint32_t)(r0 + it.g), sweep, w);
             if (S > 1 && item == tid && h > 0) wait_halos(h - 1);
-            update(it, c, w, hf, fb, in);
+            update(it, it.sh, c, w, hf, fb, in);
           }
           __syncthreads();
           if (S > 1) push_halos(c, h);

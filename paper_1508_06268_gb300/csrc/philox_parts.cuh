@@ -72,18 +72,24 @@ __device__ __forceinline__ void philox_words(const PhiloxKeys &k, const BlockPar
   }
 }
 
-template <int NB>
-__device__ __forceinline__ BlockParts<NB> block_parts(const PhiloxKeys &k, uint32_t stage, uint32_t block0) {
+// Blocks block0 + step(j).
+template <int NB, class F>
+__device__ __forceinline__ BlockParts<NB> block_parts(const PhiloxKeys &k, uint32_t stage, uint32_t block0, F step) {
   BlockParts<NB> bp;
 #pragma unroll
   for (int j = 0; j < NB; ++j) {
-    const uint64_t p = (uint64_t)kPhiloxM0 * (block0 + (uint32_t)j);
+    const uint64_t p = (uint64_t)kPhiloxM0 * (block0 + (uint32_t)step(j));
     bp.lo[j] = (uint32_t)p;
 #pragma unroll
     for (int c = 0; c < 2; ++c)
       bp.q[c][j] = (uint64_t)kPhiloxM1 * ((uint32_t)(p >> 32) ^ tag_word(kTagMetro, stage, (uint32_t)c) ^ k.k1[0]);
   }
   return bp;
+}
+
+template <int NB>
+__device__ __forceinline__ BlockParts<NB> block_parts(const PhiloxKeys &k, uint32_t stage, uint32_t block0) {
+  return block_parts<NB>(k, stage, block0, [](int j) { return j; });
 }
 
 }  // namespace rfim

@@ -18,12 +18,31 @@ struct ResidentShape {
   // slabs, replicas per cluster, Philox blocks per item (0: the kernel on bytes), threads per CTA
   int32_t S = 0, G = 0, NB = 0, threads = 0;
   bool one = true;  // one item per thread (else a thread may run several)
+  int32_t T = 0;    // tile edge of the multi-hit double checkerboard (0: the plain checkerboard)
   size_t smem = 0;
 };
 
+using ResidentFn = void (*)(RealView, ResidentArgs, uint32_t, int32_t, const float4 *, ExchArgs);
+
+struct ResidentInstance {
+  int32_t L, S, NB, NT;
+  bool one;  // one item per thread
+  int32_t T;
+  ResidentFn bim, flt;
+};
+
+template <int L, int S, int NB, int NT, bool ONE, int T = 0>
+constexpr ResidentInstance resident_instance() {
+  return {L, S, NB, NT, ONE, T, k_resident<L, S, NB, true, NT, ONE, T>, k_resident<L, S, NB, false, NT, ONE, T>};
+}
+
+// The multi-hit instances (kernels_resident_mh.cu).
+const std::vector<ResidentInstance> &resident_multihit_instances();
+
 // The shape with the lowest estimated half-sweep time (in cycles) for R replicas of edge L among the
-// instances whose CTAs are all resident at once; false when there is none.
-bool resident_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles);
+// instances whose CTAs are all resident at once; false when there is none.  T: tile edge of the
+// multi-hit double checkerboard (then the time of a pass), 0: plain.
+bool resident_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles, int32_t T = 0);
 // One shape per instance that fits R replicas, for the launch-shape tuner.
 std::vector<ResidentShape> resident_shapes(int32_t L, int32_t R, bool bimodal);
 // Whether the instance exists and all CTAs of R replicas are resident at once; fills s->smem.

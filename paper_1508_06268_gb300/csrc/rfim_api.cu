@@ -284,10 +284,10 @@ int do_run(rfim_ctx *c, int64_t n_sweeps, int32_t ex, int64_t measure_from) {
     const bool ends_interval = ex > 0 && (c->sweep + chunk) % ex == 0;
     int rc;
     // whole intervals on the grid-wide and resident plans: several per launch (not with the
-    // structure factor, which a separate kernel measures after every exchange step, nor with multi-hit)
-    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && c->plan.counter && c->plan.max_intervals() > 1 &&
-        !c->xi_on && c->mh.mh == 0) {
-      const int64_t k = std::min(left / ex, c->plan.max_intervals());
+    // structure factor, which a separate kernel measures after every exchange step)
+    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && c->plan.counter && c->plan.max_intervals(c->mh.mh) > 1 &&
+        !c->xi_on) {
+      const int64_t k = std::min(left / ex, c->plan.max_intervals(c->mh.mh));
       rc = do_sweeps_exchange_bits(c, ex, measure_from, (int32_t)k);
       if (rc) return rc;
       left -= k * ex;
@@ -591,6 +591,13 @@ int rfim_set_multihit(rfim_ctx *ctx, int32_t mh, int32_t tile) {
   const bool bim = c->kind == kBimodal;
   if (prepare_multihit(c->plan, bim) != cudaSuccess) {
     cudaGetLastError();
+    bool found = false;
+    // (fewer than four replicas at L = 64 have no cluster shape for multi-hit and stay refused below)
+    if (c->L < 64 || c->Rcap >= 4) CUDA_OR_FAIL(c, prepare_multihit_resident(c->plan, bim, tile, c->stream, &found));
+    if (found) {
+      c->mh = make_multihit(c->L, mh, tile);
+      return RFIM_OK;
+    }
     // the current launch shape has no multi-hit instance (e.g. the grid-wide plan): switch to the
     // default cluster / single-CTA shape of this L
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
@@ -746,7 +753,9 @@ int rfim_get_plan(const rfim_ctx *ctx, char *plan_out, int32_t plan_cap) {
     plan_out[0] = '\0';
     return RFIM_OK;
   }
-  snprintf(plan_out, (size_t)plan_cap, "%s", plan_name(p).c_str());
+  BitsPlan shown = p;  // multi-hit sweeps: their own resident shape, if they have one
+  if (ctx->mh.mh > 0 && p.mh_res.threads > 0) shown.res = p.mh_res;
+  snprintf(plan_out, (size_t)plan_cap, "%s", plan_name(shown).c_str());
   return RFIM_OK;
 }
 

@@ -45,10 +45,15 @@ struct BitsPlan {
   // records and the number of the last exchange interval that has been launched
   ResidentShape res;
   uint4 *rec = nullptr;
+  size_t rec_slots = 0;  // records of one interval the array holds (two intervals)
   mutable uint32_t epoch = 0;
+  ResidentShape mh_res;  // resident shape of the multi-hit sweeps in force (threads > 0 when they have one)
   bool resident() const { return res.threads > 0; }
-  // exchange intervals one launch takes at most
-  int64_t max_intervals() const { return resident() ? kResidentIntervals : S == 0 ? 64 : 1; }
+  // exchange intervals one launch takes at most (mh passes per visit; 0: plain sweeps)
+  int64_t max_intervals(int32_t mh) const {
+    if (mh > 0) return mh_res.threads > 0 && mh < kResidentIntervals ? kResidentIntervals / mh : 1;
+    return resident() ? kResidentIntervals : S == 0 ? 64 : 1;
+  }
 };
 
 // Multi-hit double 3D checkerboard (Sec. 3.2, kernels_mh.cuh): mh local passes per tile visit
@@ -62,6 +67,9 @@ bool multihit_tile_ok(int32_t L, int32_t tile);
 MultiHit make_multihit(int32_t L, int32_t mh, int32_t tile);
 // Whether the plan's shape has a multi-hit instance; sets its launch attributes.
 cudaError_t prepare_multihit(const BitsPlan &plan, bool bimodal);
+// Gives the plan a resident shape for multi-hit sweeps with tiles of edge `tile`, beside its shape for
+// plain sweeps; *found is false when there is none or the cluster kernel is expected to be faster.
+cudaError_t prepare_multihit_resident(BitsPlan &plan, bool bimodal, int32_t tile, cudaStream_t st, bool *found);
 
 bool bits_supported(int32_t L);
 // Launch-shape tuner support: a thread-local candidate shape for the next make_bits_plan, the

@@ -72,6 +72,49 @@ def test_resident_gaussian_equals_cluster_plan(L, R, plan, ref, monkeypatch):
         np.testing.assert_array_equal(p[k], q[k])
 
 
+MULTIHIT = [  # L, R, tile, "S,G,NB,threads,r": slabs of whole tiles and slabs that cut them, partial groups
+    (16, 3, 8, "1,2,1,512,r"), (16, 5, 8, "1,3,2,384,r"), (16, 5, 8, "1,4,4,256,r"), (32, 2, 8, "4,1,1,512,r"),
+    (32, 3, 8, "4,2,2,512,r"), (32, 3, 8, "2,1,2,512,r"), (32, 3, 8, "2,2,4,512,r"), (32, 2, 16, "4,1,1,512,r"),
+    (32, 3, 16, "2,1,2,512,r"), (32, 3, 16, "2,2,4,512,r"), (64, 4, 8, "16,1,2,512,r"), (64, 4, 8, "8,1,4,512,r"),
+    (64, 5, 8, "4,2,4,512,m"), (64, 4, 16, "16,1,2,512,r"), (64, 4, 16, "8,1,4,512,r"), (64, 5, 16, "4,3,4,512,m"),
+    (64, 4, 32, "16,1,2,512,r"), (64, 4, 32, "8,1,4,512,r"), (64, 5, 32, "4,2,4,512,m"),
+]
+
+
+@pytest.mark.parametrize("L,R,tile,plan", MULTIHIT)
+@pytest.mark.parametrize("kind", [rf.FIELD_BIMODAL, rf.FIELD_EXPLICIT])
+def test_resident_multihit(L, R, tile, plan, kind, monkeypatch):
+    """Multi-hit sweeps of the resident kernel, several intervals per launch: with a bimodal field equal
+    to the oracle's; with a float field equal to the cluster kernel's (the same float operations)."""
+    mh = 3 if L < 64 else 2
+    kw = dict(h=1.5, field_kind=kind, field=inputs.gaussian_field(L, 3) if kind == rf.FIELD_EXPLICIT else None, seed=8)
+    monkeypatch.setenv("RFIM_BITS_PLAN", plan)
+    g = rf.Realization(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
+    g.set_multihit(mh, tile)
+    assert g.plan() == plan
+    if kind == rf.FIELD_BIMODAL:
+        o = oracle.Oracle(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
+    else:
+        monkeypatch.setenv("RFIM_BITS_PLAN", {16: "1,4,1,512", 32: "2,1,1,256", 64: "4,4,4,512"}[L])
+        o = rf.Realization(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
+    o.set_multihit(mh, tile)
+    n0 = g.launch_count
+    for x in (g, o):
+        x.run(4, 2, 1)
+        x.sweep(1)
+        x.exchange(0)
+    assert g.launch_count - n0 == 3
+    st = g.get_state()
+    if kind == rf.FIELD_BIMODAL:
+        want = (o.spins(), o.perm()[0], o.observables())
+    else:
+        assert o.plan() in ("1,4,1,512", "1,3,1,512", "2,1,1,256", "4,4,4,512")
+        want = (o.get_state()["spins"], o.get_state()["t2r"], o.observables()["sums"])
+    np.testing.assert_array_equal(st["spins"], want[0])
+    np.testing.assert_array_equal(st["t2r"], want[1])
+    np.testing.assert_array_equal(g.observables()["sums"], want[2])
+
+
 BYTES = [  # L, R, "S,G,4,threads,b": rows of whole blocks, even rows, odd rows; blocks across slabs
     (4, 2, "1,1,4,32,b"), (4, 9, "2,4,4,64,b"), (6, 5, "1,3,4,96,b"), (6, 3, "2,2,4,32,b"), (10, 3, "1,1,4,128,b"),
     (10, 5, "4,2,4,96,b"), (14, 3, "2,2,4,256,b"), (18, 2, "8,1,4,128,b"), (12, 5, "1,2,4,256,b"), (12, 3, "4,2,4,128,b"),
