@@ -23,7 +23,7 @@ struct ResidentState {
   uint8_t *swapped;
 };
 
-__host__ __device__ constexpr size_t resident_state_bytes(int rcap) { return (size_t)rcap * 29 + 32; }
+__host__ __device__ constexpr size_t resident_state_bytes(int rcap) { return ((size_t)rcap * 29 + 32 + 15) / 16 * 16; }
 
 struct alignas(16) ChunkSum {
   int B, M;
@@ -51,6 +51,20 @@ __device__ __forceinline__ void mbar_wait(uint32_t mbar, uint32_t par, unsigned 
     if ((it & 63u) == 63u && *(volatile unsigned *)err) return;
   }
   atomicOr(err, 2u);
+}
+
+// The same wait without the report and whatever has been reported: for pushes that are on their way
+// when a CTA ends after an expired wait.
+__device__ __forceinline__ void mbar_drain(uint32_t mbar, uint32_t par) {
+  for (unsigned it = 0; it < kMbarSpinLimit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(mbar), "r"(par)
+        : "memory");
+    if (done) return;
+  }
 }
 
 constexpr unsigned kRecordSpinLimit = 1u << 22;

@@ -68,6 +68,10 @@ cudaError_t launch_exchange(const RealView &v, uint32_t j, int64_t measure_from,
 // Adds each replica's structure factor F (Sec. 7 correlation length) to sumF[r2t[r]].
 cudaError_t launch_measure_xi(const RealView &v, const double *kcos, const double *ksin, double *sumF, bool bitpack,
                               cudaStream_t st);
+// The same for the measuring intervals iv in [first, n) of one launch from their marginals
+// marg[iv][R][3][L] and the replica at every temperature t2r[iv][R], added in interval order.
+cudaError_t launch_xi_sums(const RealView &v, const int32_t *marg, const int32_t *t2r, int32_t first, int32_t n,
+                           const double *kcos, const double *ksin, double *sumF, cudaStream_t st);
 cudaError_t launch_to_natural(const RealView &v, int32_t R, bool bitpack, int8_t *out, cudaStream_t st);
 cudaError_t launch_from_natural(const RealView &v, int32_t R, bool bitpack, const int8_t *in, cudaStream_t st);
 // Per-(replica, CTA) partial sums of the multi-CTA int8 energy reduction, owned by the caller:

@@ -430,6 +430,7 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
     p.S = rs.S; p.G = rs.G; p.GT = 1; p.threads = rs.threads; p.NS = 1;
     p.res = rs;
     p.smem = rs.smem;
+    p.xi = resident_xi_fits(L, Rcap, bimodal, rs);
   }
   if (p.S != 0 && !resident) {
     if (p.G > Rcap) p.G = Rcap;
@@ -490,10 +491,12 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
     if (!rc) rc = grab((void **)&p.fquant, sizeof(FieldQuant), "field quantum");
   }
   const size_t parts = (size_t)Rcap * p.S;
-  if (!rc) rc = grab((void **)&p.partB, parts * 8, "partials");
-  if (!rc) rc = grab((void **)&p.partM, parts * 8, "partials");
-  if (!rc) rc = grab((void **)&p.partFi, parts * 8, "partials");
-  if (!rc) rc = grab((void **)&p.partF, parts * 8, "partials");
+  if (!resident) {  // the resident plan sends energy records instead
+    if (!rc) rc = grab((void **)&p.partB, parts * 8, "partials");
+    if (!rc) rc = grab((void **)&p.partM, parts * 8, "partials");
+    if (!rc) rc = grab((void **)&p.partFi, parts * 8, "partials");
+    if (!rc) rc = grab((void **)&p.partF, parts * 8, "partials");
+  }
   if (!rc) rc = grab((void **)&p.counter, 16, "counter");  // cluster arrivals, error word, grid-wide arrival count
   if (!rc && gfn) {
     const size_t gslots = 2 * (size_t)Rcap * (L + 1);  // two intervals' partials
@@ -569,7 +572,7 @@ cudaError_t build_field4(const RealView &v, BitsPlan &plan, cudaStream_t st) {
 
 cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t sweep0, int32_t n_sweeps,
                                bool exchange, uint32_t j, int64_t measure_from, double J, double h,
-                               cudaStream_t st, const MultiHit *mh, int32_t n_intervals) {
+                               cudaStream_t st, const MultiHit *mh, int32_t n_intervals, const XiWork *xi) {
   ExchArgs xa{};
   xa.enabled = exchange ? 1 : 0;
   xa.j = j;
@@ -602,6 +605,13 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
     ra.epoch0 = plan.epoch + 1;
     ra.rec = plan.rec;
     ra.i8 = plan.i8;
+    if (xi && exchange) {
+      if (!plan.measures_xi(ra.mh) || n_intervals > xi->intervals) return cudaErrorInvalidValue;
+      ra.xi_marg = xi->marg;
+      ra.xi_t2r = xi->t2r;
+      const cudaError_t e = cudaMemsetAsync(xi->marg, 0, (size_t)n_intervals * v.R * 3 * v.L * sizeof(int32_t), st);
+      if (e != cudaSuccess) return e;
+    }
     const cudaError_t e = rs.NB ? launch_resident(v, rs, ra, sweep0, n_sweeps, plan.field4, xa, st)
                                 : launch_resident_bytes(v, rs, ra, sweep0, n_sweeps, xa, st);
     if (e == cudaSuccess && exchange) plan.epoch += (uint32_t)n_intervals;

@@ -334,7 +334,11 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     if (ok && iv + 1 < n_iv) tab_fill_temps<BIM, false>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
-  if (S > 1) sync_slabs<2>();  // a CTA stays until its neighbours' pushes have landed
+  if (S > 1) {  // a CTA stays until its neighbours' pushes have landed, also those whose wait expired
+    if (*(volatile unsigned *)xa.err & 2u)
+      for (uint32_t q = h > 2 ? h - 2 : 0; q < h; ++q) mbar_drain(mbar0 + 8 * (q & 1u), (q >> 1) & 1u);
+    sync_slabs<2>();
+  }
   copy_planes(1, PZ, false);
   if (xa.enabled && ok && blockIdx.x == 0)
     for (int r = tid; r < R; r += nt) {

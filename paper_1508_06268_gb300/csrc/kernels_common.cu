@@ -468,6 +468,44 @@ __global__ void k_measure_xi_rows64(RealView v, const double *kcos, const double
   }
 }
 
+// Structure factors from the marginals of many intervals: one CTA per temperature k, 32 intervals at
+// a time, one thread per Fourier sum (cosine and sine along each axis, each in the order of t, as
+// above), then F per interval and the sum over the intervals in order.
+constexpr int kXiBatch = 32;
+__global__ void __launch_bounds__(6 * kXiBatch) k_xi_sums(RealView v, const int32_t *__restrict__ marg,
+                                                          const int32_t *__restrict__ t2r, int32_t first, int32_t n,
+                                                          const double *__restrict__ kcos, const double *__restrict__ ksin,
+                                                          double *sumF) {
+  __shared__ double part[kXiBatch][6], F[kXiBatch];
+  const int k = blockIdx.x, L = v.L, b = threadIdx.x / 6, q = threadIdx.x % 6;
+  double sum = sumF[k];
+  for (int iv0 = first; iv0 < n; iv0 += kXiBatch) {
+    const int iv = iv0 + b;
+    if (iv < n) {
+      const int32_t *S = marg + ((int64_t)iv * v.R + t2r[(int64_t)iv * v.R + k]) * 3 * L + (q >> 1) * L;
+      const double *wave = q & 1 ? ksin : kcos;
+      double a = 0.0;
+#pragma unroll 8
+      for (int t = 0; t < L; ++t) a = __dadd_rn(a, __dmul_rn(wave[t], (double)S[t]));
+      part[b][q] = a;
+    }
+    __syncthreads();
+    if (threadIdx.x < kXiBatch && iv0 + (int)threadIdx.x < n) {
+      const double *p = part[threadIdx.x];
+      double f = 0.0;
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+        f = __dadd_rn(f, __dadd_rn(__dmul_rn(p[2 * d], p[2 * d]), __dmul_rn(p[2 * d + 1], p[2 * d + 1])));
+      F[threadIdx.x] = f / (3.0 * (double)v.N);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int i = 0; i < kXiBatch && iv0 + i < n; ++i) sum = __dadd_rn(sum, F[i]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) sumF[k] = sum;
+}
+
 // One exchange step j plus measurement (exchange.cuh), one CTA.
 __global__ void k_exchange(RealView v, uint32_t j, int64_t measure_from) { exchange_and_measure(v, j, measure_from); }
 
@@ -564,6 +602,12 @@ cudaError_t launch_measure_xi(const RealView &v, const double *kcos, const doubl
     k_measure_xi_rows64<true><<<v.R, 512, 0, st>>>(v, kcos, ksin, sumF);
   else
     k_measure_xi<<<v.R, 512, (size_t)3 * v.L * sizeof(int), st>>>(v, kcos, ksin, sumF, bitpack);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_xi_sums(const RealView &v, const int32_t *marg, const int32_t *t2r, int32_t first, int32_t n,
+                           const double *kcos, const double *ksin, double *sumF, cudaStream_t st) {
+  k_xi_sums<<<v.R, 6 * kXiBatch, 0, st>>>(v, marg, t2r, first, n, kcos, ksin, sumF);
   return cudaGetLastError();
 }
 

@@ -85,6 +85,9 @@ size_t resident_smem(int32_t L, int32_t S, int32_t G, int32_t R) {
   return (size_t)G * 2 * planes * (L * L / 64) * 4 + tab_bytes(G) + (size_t)G * chunks * sizeof(ChunkSum) + resident_state_bytes(R);
 }
 
+// With the marginals of the structure factor.
+size_t resident_xi_smem(int32_t L, const ResidentShape &s) { return s.smem + (size_t)s.G * 3 * L * sizeof(int); }
+
 // log2 of the words whose items of one part are neighbouring threads: a warp's worth, or all of a
 // CTA's words when they are fewer (several parts then share a warp).
 int lane_words(const Instance &i, int32_t G) {
@@ -158,6 +161,14 @@ bool resident_fits(int32_t L, int32_t R, bool bimodal, ResidentShape *s) {
   return ctas <= resident_ctas((const void *)(bimodal ? i->bim : i->flt), s->S, s->threads, s->smem);
 }
 
+bool resident_xi_fits(int32_t L, int32_t R, bool bimodal, const ResidentShape &s) {
+  const ResidentFn fn = s.T || !s.NB ? nullptr : resident_xi_kernel(L, s.S, s.NB, s.one, bimodal);
+  const size_t smem = resident_xi_smem(L, s);
+  if (!fn || smem > 227 * 1024) return false;
+  const int64_t ctas = (int64_t)((R + s.G - 1) / s.G) * s.S;
+  return ctas <= resident_ctas((const void *)fn, s.S, s.threads, smem);
+}
+
 bool resident_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles, int32_t T) {
   for (const Candidate &c : candidates(L, R, bimodal, T)) {
     ResidentShape s = c.shape;
@@ -207,8 +218,16 @@ cudaError_t launch_resident(const RealView &v, const ResidentShape &s, const Res
   ra.keys = philox_keys(v.seed, v.realization);
   ra.lw = lane_words(*i, s.G);
   const int clusters = (v.R + s.G - 1) / s.G;
-  ResidentLaunch l(clusters, s, xa.enabled, st);
-  return cudaLaunchKernelEx(&l.cfg, v.kind == kBimodal ? i->bim : i->flt, v, ra, sweep0, n_sweeps, field4, xa);
+  const bool bim = v.kind == kBimodal;
+  ResidentFn fn = bim ? i->bim : i->flt;
+  ResidentShape ls = s;
+  if (ra.xi_marg) {
+    fn = resident_xi_kernel(v.L, s.S, s.NB, s.one, bim);
+    if (!fn || s.T) return cudaErrorInvalidConfiguration;
+    ls.smem = resident_xi_smem(v.L, s);
+  }
+  ResidentLaunch l(clusters, ls, xa.enabled, st);
+  return cudaLaunchKernelEx(&l.cfg, fn, v, ra, sweep0, n_sweeps, field4, xa);
 }
 
 }  // namespace rfim

@@ -48,6 +48,9 @@ struct ResidentArgs {
   int32_t i8;       // the realization is stored as bytes (v.spins8) and staged as bits
   int32_t lw;       // log2 of the words whose items of one part are neighbouring threads (ONE; else 5)
   int32_t mh;       // passes per tile visit (T > 0)
+  // structure factor (XI): of every measuring interval iv, the marginals S_d[t] of every
+  // replica, [iv][R][3][L], zero when the launch starts, and the replica at every temperature, [iv][R]
+  int32_t *xi_marg, *xi_t2r;
 };
 
 // Planes of a slab in shared memory: with S > 1 a halo plane before and after the slab's own.
@@ -75,6 +78,54 @@ __host__ __device__ constexpr uint32_t item_pattern() {
   return m;
 }
 
+// 32 x 32 bits over a warp, transposed: bit k of lane i was bit i of lane k.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane) {
+  uint32_t m = 0x0000FFFFu;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+    x = lane & s ? (x & ~m) | ((y & ~m) >> s) : (x & m) | ((y & m) << s);
+    m ^= m << (s / 2);
+  }
+  return x;
+}
+
+// Marginals S_d[t] (sums of the spins with coordinate t along axis d, Sec. 7's structure factor) of
+// gact replicas over the planes z0 .. of a slab, first in marg[g][3][L] (zero at the call) and then added to
+// out[g][3][L] in global memory; replica g's colours are CW words each, the slab's own planes from word
+// `first` of a colour on.  A warp takes 32 words: their transpose gives lane b the 32 bits of in-word
+// bit b, i.e. of one x up to the row parity.
+template <int L, int PZ>
+__device__ __forceinline__ void slab_marginals(const uint32_t *sp, int CW, int first, int *marg, int gact, int z0, int32_t *out) {
+  constexpr int P = BitsGeom<L>::P, Lh = L / 2, RW = 64 / L, WC = PZ * P, NCK = (WC + 31) / 32;
+  constexpr uint32_t kRow = ((1u << (Lh / 4)) - 1u) * 0x01010101u;
+  const int lane = threadIdx.x & 31, p = 4 * (lane & 7) + (lane >> 3);  // in-word position of bit `lane`
+  for (int u = threadIdx.x >> 5; u < gact * 2 * NCK; u += blockDim.x >> 5) {
+    const int g = u / (2 * NCK), c = u / NCK & 1, wl = u % NCK * 32 + lane;
+    const bool in = wl < WC;
+    const uint32_t w = in ? sp[(g * 2 + c) * CW + first + wl] : 0u;
+    int *mg = marg + g * 3 * L;
+    const int z = z0 + (in ? wl : 0) / P, y0 = wl % P * RW;
+    if (in) {
+#pragma unroll
+      for (int rr = 0; rr < RW; ++rr) atomicAdd(&mg[L + y0 + rr], 2 * __popc(w & (kRow << (rr * (Lh / 4)))) - Lh);
+    }
+    if (P >= 32) {  // the warp's words share one plane
+      const int zs = __reduce_add_sync(0xffffffffu, 2 * __popc(w) - 32);
+      if (lane == 0) atomicAdd(&mg[2 * L + z], zs);
+    } else if (in) {
+      atomicAdd(&mg[2 * L + z], 2 * __popc(w) - 32);
+    }
+    const uint32_t have = __ballot_sync(0xffffffffu, in), odd0 = __ballot_sync(0xffffffffu, in && ((c + y0 + z) & 1));
+    const uint32_t col = transpose_bits(w, lane), odd = (p / Lh & 1) ? have & ~odd0 : odd0, even = have & ~odd;
+    atomicAdd(&mg[2 * (p % Lh)], 2 * __popc(col & even) - __popc(even));
+    atomicAdd(&mg[2 * (p % Lh) + 1], 2 * __popc(col & odd) - __popc(odd));
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < gact * 3 * L; t += blockDim.x)
+    if (marg[t] != 0) atomicAdd(out + t, marg[t]);
+}
+
 // One item: word iw of plane zl of replica g of the slab, blocks sh + item_block(0 .. NB - 1) of it (T > 0:
 // sh for the tiles of even x index, T / 8 further on for the odd ones).
 template <int NB>
@@ -86,7 +137,9 @@ struct ResidentItem {
   uint32_t p0;                    // row-parity mask of colour 0 (colour 1: its complement)
 };
 
-template <int L, int S, int NB, bool BIM, int NT, bool ONE, int T = 0>
+// XI: measures the structure factor too (an instance of its own: as a run-time choice it slowed runs
+// that do not measure it, L = 16, R = 32 5.7 -> 5.9 us per interval).
+template <int L, int S, int NB, bool BIM, int NT, bool ONE, int T = 0, bool XI = false>
 __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_constant__ ResidentArgs ra, uint32_t sweep0,
                                                  int32_t nsw, const float4 *__restrict__ field4, const ExchArgs xa) {
   using Gm = BitsGeom<L>;
@@ -118,11 +171,13 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   xs.t2r = xs.M + ra.rcap;
   xs.r2t = xs.t2r + ra.rcap;
   xs.swapped = reinterpret_cast<uint8_t *>(xs.r2t + ra.rcap);
+  int *marg = reinterpret_cast<int *>(reinterpret_cast<char *>(xs.E) + resident_state_bytes(ra.rcap) / 16 * 16);  // [G][3][L]
 
   // debug build: the replica range, the shared-memory plan and the cluster must be the launch's
   const bool ok = RFIM_DCHECK(xa.err, gact >= 1 && gact <= ra.G && r0 + gact <= R && R <= ra.rcap, kDbgGlobal) &&
-                  RFIM_DCHECK(xa.err, (uint32_t)__cvta_generic_to_shared(xs.swapped + ra.rcap) <=
-                                          (uint32_t)__cvta_generic_to_shared(sm) + dyn_smem_bytes(),
+                  RFIM_DCHECK(xa.err, xs.swapped + ra.rcap <= reinterpret_cast<uint8_t *>(marg) &&
+                                          (uint32_t)__cvta_generic_to_shared(marg + (XI ? 3 * L * ra.G : 0)) <=
+                                              (uint32_t)__cvta_generic_to_shared(sm) + dyn_smem_bytes(),
                               kDbgTable) &&
                   RFIM_DCHECK(xa.err, S == 1 || cluster_ctas() == (uint32_t)S, kDbgRank);
   // the slab with its halo planes (the halos of colour 0 are pushed before they are needed)
@@ -333,6 +388,9 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     }
     if (S > 1 && h > 0) wait_halos(h - 1);
     if (!xa.enabled) break;
+    const bool xi = XI && (int64_t)(xa.j + (uint32_t)iv) >= xa.measure_from;
+    if (xi)
+      for (int t = tid; t < gact * 3 * L; t += nt) marg[t] = 0;
 
     // ---- energies (Eq. 1) of this slab's replicas, one ChunkSum per SEG words --------------------
     for (int e = tid; e < (gact * 2 * WC + 31) / 32 * 32; e += nt) {
@@ -422,16 +480,25 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
       if (NCH <= 4 || lane == 0) record_store(rec + (size_t)(r0 + g) * S + rank, epoch, s.B, s.M, s.F);
     }
 
+    // ---- structure factor: the slab's marginals, while the records are on their way -----------------
+    if (xi && ok) slab_marginals<L, PZ>(sp, CW, Z1 * P, marg, gact, z0, ra.xi_marg + ((int64_t)iv * R + r0) * 3 * L);
+
     // ---- exchange step, then the tables of the temperatures it assigned ------------------------------
     auto energy_of = [&](int B, long long F) {
       const double Fd = BIM ? xa.h * (double)F : (double)(2 * F - Htot) * fscale;
       return -xa.J * (double)B - Fd;
     };
     if (ok) exchange_from_records<false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, energy_of);
+    if (xi && ok && blockIdx.x == 0)
+      for (int k = tid; k < R; k += nt) ra.xi_t2r[(int64_t)iv * R + k] = xs.t2r[k];
     if (ok && iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
-  if (S > 1) sync_slabs<S>();  // a CTA stays until its neighbours' pushes have landed
+  if (S > 1) {  // a CTA stays until its neighbours' pushes have landed, also those whose wait expired
+    if (*(volatile unsigned *)xa.err & 2u)
+      for (uint32_t q = h > 2 ? h - 2 : 0; q < h; ++q) mbar_drain(mbar0 + 8 * (q & 1u), (q >> 1) & 1u);
+    sync_slabs<S>();
+  }
 
   for (int t = tid; ok && t < gact * 2 * WC; t += nt) {
     const int g = t / (2 * WC), rem = t % (2 * WC), c = rem / WC, wl = rem % WC;

@@ -36,6 +36,11 @@ constexpr ResidentInstance resident_instance() {
   return {L, S, NB, NT, ONE, T, k_resident<L, S, NB, true, NT, ONE, T>, k_resident<L, S, NB, false, NT, ONE, T>};
 }
 
+// The instance that measures the structure factor too (kernels_resident_xi.cu), or null.
+ResidentFn resident_xi_kernel(int32_t L, int32_t S, int32_t NB, bool one, bool bimodal);
+// Whether launches of shape s for up to R replicas can measure it: the instance exists and its CTAs fit.
+bool resident_xi_fits(int32_t L, int32_t R, bool bimodal, const ResidentShape &s);
+
 // The multi-hit instances (kernels_resident_mh.cu).
 const std::vector<ResidentInstance> &resident_multihit_instances();
 

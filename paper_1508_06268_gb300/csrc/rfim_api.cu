@@ -47,7 +47,8 @@ struct rfim_ctx {
   EnergyParts eparts{};        // int8 layout: partials of the multi-CTA energy reduction
   // structure-factor measurement (correlation length, Sec. 7): off unless enabled
   bool xi_on = false;
-  double *sumF = nullptr, *kcos = nullptr, *ksin = nullptr;
+  double *sumF = nullptr, *kcos = nullptr, *ksin = nullptr;  // one block, with xi's arrays
+  XiWork xi;  // of launches that measure the structure factor themselves
   BitsPlan plan;
   MultiHit mh;  // multi-hit double checkerboard (mh.mh == 0: plain checkerboard)
   std::string err;
@@ -150,7 +151,7 @@ void free_all(rfim_ctx *c) {
   free_events(c);
   void *ptrs[] = {c->spins8, c->bits, c->hraw, c->hh_c, c->hbit_c, c->hbits, c->thr, c->gjn, c->b2, c->b2l,
                   c->beta_d, c->t2r, c->r2t, c->E, c->M, c->att, c->acc, c->obs, c->n_meas, c->scratch8,
-                  c->sumF, c->kcos, c->ksin, c->eparts.B, c->eparts.M, c->eparts.Fi, c->eparts.F,
+                  c->sumF, c->eparts.B, c->eparts.M, c->eparts.Fi, c->eparts.F,
                   c->eparts.count};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -249,14 +250,20 @@ int measure_xi_after(rfim_ctx *c, int64_t j, int64_t measure_from) {
 int do_sweeps_exchange_bits(rfim_ctx *c, int64_t n, int64_t measure_from, int32_t k = 1) {
   RealView v = view_of(c);
   cudaEvent_t stop;
+  const int64_t j0 = c->xstep;
+  const bool xi = c->xi_on && j0 + k - 1 >= measure_from && c->xi.intervals > 0 && c->plan.measures_xi(c->mh.mh);
   CUDA_OR_FAIL(c, prof_begin(c, 0, &stop, k));
-  CUDA_OR_FAIL(c, launch_sweeps_bits(v, c->plan, (uint32_t)c->sweep, (int32_t)n, true, (uint32_t)c->xstep,
-                                     measure_from, (double)c->J, (double)c->h, c->stream, &c->mh, k));
+  CUDA_OR_FAIL(c, launch_sweeps_bits(v, c->plan, (uint32_t)c->sweep, (int32_t)n, true, (uint32_t)j0, measure_from,
+                                     (double)c->J, (double)c->h, c->stream, &c->mh, k, xi ? &c->xi : nullptr));
   CUDA_OR_FAIL(c, prof_end(c, stop));
   c->launches += 1;
   c->sweep += n * k;
   c->xstep += k;
-  return measure_xi_after(c, c->xstep - 1, measure_from);
+  if (!xi) return measure_xi_after(c, c->xstep - 1, measure_from);
+  const int32_t first = (int32_t)std::max<int64_t>(0, measure_from - j0);
+  CUDA_OR_FAIL(c, launch_xi_sums(v, c->xi.marg, c->xi.t2r, first, k, c->kcos, c->ksin, c->sumF, c->stream));
+  c->launches += 1;
+  return RFIM_OK;
 }
 
 int do_exchange(rfim_ctx *c, int64_t measure_from) {
@@ -283,11 +290,15 @@ int do_run(rfim_ctx *c, int64_t n_sweeps, int32_t ex, int64_t measure_from) {
     }
     const bool ends_interval = ex > 0 && (c->sweep + chunk) % ex == 0;
     int rc;
-    // whole intervals on the grid-wide and resident plans: several per launch (not with the
-    // structure factor, which a separate kernel measures after every exchange step)
-    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && c->plan.counter && c->plan.max_intervals(c->mh.mh) > 1 &&
-        !c->xi_on) {
-      const int64_t k = std::min(left / ex, c->plan.max_intervals(c->mh.mh));
+    // whole intervals on the grid-wide and resident plans: several per launch (with the structure
+    // factor, where it is measured inside the launch: elsewhere a separate kernel does so after every step)
+    const int64_t most = !c->plan.counter ? 1
+                         : !c->xi_on      ? c->plan.max_intervals(c->mh.mh)
+                         : c->plan.measures_xi(c->mh.mh)
+                             ? std::min<int64_t>(c->plan.max_intervals(c->mh.mh), c->xi.intervals)
+                             : 1;
+    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && most > 1) {
+      const int64_t k = std::min(left / ex, most);
       rc = do_sweeps_exchange_bits(c, ex, measure_from, (int32_t)k);
       if (rc) return rc;
       left -= k * ex;
@@ -561,15 +572,22 @@ int rfim_set_measure_xi(rfim_ctx *ctx, int32_t on) {
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
   if (nm > 0 && !c->xi_on) return fail(c, RFIM_ESTATE, "enable the structure-factor measurement before the first measurement");
   if (!c->sumF) {
-    int rc;
-    if ((rc = dalloc(c, &c->sumF, (size_t)c->Rcap))) return rc;
-    if ((rc = dalloc(c, &c->kcos, (size_t)c->L))) return rc;
-    if ((rc = dalloc(c, &c->ksin, (size_t)c->L))) return rc;
-    std::vector<double> kc(c->L), ks(c->L);
-    wave_tables(c->L, kc.data(), ks.data());
-    CUDA_OR_FAIL(c, cudaMemcpy(c->kcos, kc.data(), c->L * 8, cudaMemcpyHostToDevice));
-    CUDA_OR_FAIL(c, cudaMemcpy(c->ksin, ks.data(), c->L * 8, cudaMemcpyHostToDevice));
-    CUDA_OR_FAIL(c, cudaMemsetAsync(c->sumF, 0, (size_t)c->Rcap * 8, c->stream));
+    // one block: sums, wave tables, then the workspace of launches that measure by themselves (marginals
+    // of their intervals, 512 KiB or one interval; without room for it the separate kernel measures)
+    const size_t R = (size_t)c->Rcap, L = (size_t)c->L, tables = R + 2 * L, per = R * 3 * L;
+    size_t iv = 0;
+    if (c->plan.xi) iv = std::max<size_t>(1, std::min<size_t>((size_t)kResidentIntervals, ((size_t)128 << 10) / per));
+    int rc = dalloc(c, &c->sumF, tables + (iv * (R + per) + 1) / 2);
+    if (rc && iv) rc = dalloc(c, &c->sumF, tables + (iv = 0));
+    if (rc) return rc;
+    c->kcos = c->sumF + R;
+    c->ksin = c->kcos + L;
+    c->xi.t2r = reinterpret_cast<int32_t *>(c->sumF + tables);
+    c->xi.marg = c->xi.t2r + iv * R;
+    c->xi.intervals = (int32_t)iv;
+    std::vector<double> init(tables, 0.0);
+    wave_tables(c->L, init.data() + R, init.data() + R + L);
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(c->sumF, init.data(), tables * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
   }
   c->xi_on = true;

@@ -49,6 +49,8 @@ struct BitsPlan {
   mutable uint32_t epoch = 0;
   ResidentShape mh_res;  // resident shape of the multi-hit sweeps in force (threads > 0 when they have one)
   bool resident() const { return res.threads > 0; }
+  bool xi = false;  // plain resident launches can measure the structure factor (XiWork)
+  bool measures_xi(int32_t mh) const { return xi && mh == 0; }
   // exchange intervals one launch takes at most (mh passes per visit; 0: plain sweeps)
   int64_t max_intervals(int32_t mh) const {
     if (mh > 0) return mh_res.threads > 0 && mh < kResidentIntervals ? kResidentIntervals / mh : 1;
@@ -61,6 +63,13 @@ struct BitsPlan {
 // instantiated per tile edge).
 struct MultiHit {
   int32_t mh = 0, tile = 0;
+};
+
+// Workspace of the structure factor measured inside resident launches: marginals and the replica at
+// every temperature of up to `intervals` exchange intervals (0: not allocated).
+struct XiWork {
+  int32_t *marg = nullptr, *t2r = nullptr;
+  int32_t intervals = 0;
 };
 // Whether tiles of edge `tile` are supported at L; the setting for (L, mh, tile).
 bool multihit_tile_ok(int32_t L, int32_t tile);
@@ -100,6 +109,7 @@ std::string plan_name(const BitsPlan &plan);
 // of n_sweeps sweeps each in one launch, exchange steps j, j + 1, ...
 cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t sweep0, int32_t n_sweeps,
                                bool exchange, uint32_t j, int64_t measure_from, double J, double h,
-                               cudaStream_t st, const MultiHit *mh = nullptr, int32_t n_intervals = 1);
+                               cudaStream_t st, const MultiHit *mh = nullptr, int32_t n_intervals = 1,
+                               const XiWork *xi = nullptr);
 
 }  // namespace rfim

@@ -115,6 +115,29 @@ def test_resident_multihit(L, R, tile, plan, kind, monkeypatch):
     np.testing.assert_array_equal(g.observables()["sums"], want[2])
 
 
+@pytest.mark.parametrize("L,R,plan", [(8, 7, "1,3,1,256,r"), (16, 13, "1,3,4,384,r"), (16, 5, "2,2,2,256,r"),
+                                      (32, 3, "8,1,2,256,r"), (32, 3, "1,2,4,512,m"), (64, 2, "16,1,4,512,r"),
+                                      (64, 3, "8,2,4,512,m")])
+def test_resident_structure_factor(L, R, plan, monkeypatch):
+    """The structure factor measured inside a launch of several intervals, some before measure_from, then
+    call by call: integers, the same Fourier sums and the same order as one kernel per measuring
+    step, so the sums are the oracle's to its tests' 1e-11 (exact marginals, sums in double)."""
+    kw = dict(h=1.5, field_kind=rf.FIELD_BIMODAL, field_seed=3, seed=6)
+    g = make(monkeypatch, L, R, plan, **kw)
+    o = oracle.Oracle(L, inputs.geometric_temps(1.0, 5.0, R), **kw)
+    g.set_measure_xi()
+    o.set_measure_xi(True)
+    n0 = g.launch_count
+    for x in (g, o):
+        x.run(12, 2, 2)
+        x.exchange(0)
+        x.run(6, 2, 100)
+        x.run(4, 2, 0)
+    assert g.launch_count - n0 == 7  # four launches of intervals, three of Fourier sums
+    np.testing.assert_array_equal(g.observables()["sums"], o.observables())
+    np.testing.assert_allclose(g.observables()["F"], o.observables_F(), rtol=1e-11, atol=1e-20)
+
+
 BYTES = [  # L, R, "S,G,4,threads,b": rows of whole blocks, even rows, odd rows; blocks across slabs
     (4, 2, "1,1,4,32,b"), (4, 9, "2,4,4,64,b"), (6, 5, "1,3,4,96,b"), (6, 3, "2,2,4,32,b"), (10, 3, "1,1,4,128,b"),
     (10, 5, "4,2,4,96,b"), (14, 3, "2,2,4,256,b"), (18, 2, "8,1,4,128,b"), (12, 5, "1,2,4,256,b"), (12, 3, "4,2,4,128,b"),
