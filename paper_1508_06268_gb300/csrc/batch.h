@@ -26,7 +26,8 @@ struct BatchItem {
   int32_t slot, r0, gact, pad;
 };
 
-// Work queue: CTAs take items in order (largest first); the last CTA to leave resets it.
+// Work queue: CTAs take items in order (largest first, interval by interval); the last CTA to leave
+// resets it.
 struct BatchQueue {
   unsigned int head;
   unsigned int done_ctas;
@@ -42,7 +43,8 @@ size_t batch_smem(int L, int G);
 int batch_max_gt(int L);
 cudaError_t batch_prepare(size_t smem);
 cudaError_t batch_occupancy(size_t smem, int *blocks_per_sm);
-cudaError_t launch_batch(int grid, size_t smem, const SlotDesc *slots, SlotCtl *ctls, const BatchItem *items,
-                         BatchQueue *queue, cudaStream_t st);
+// `intervals` exchange intervals of every slot in one launch (ctls: nslots entries).
+cudaError_t launch_batch(int grid, size_t smem, const SlotDesc *slots, SlotCtl *ctls, int nslots, const BatchItem *items,
+                         BatchQueue *queue, int intervals, unsigned *err, cudaStream_t st);
 
 }  // namespace rfim

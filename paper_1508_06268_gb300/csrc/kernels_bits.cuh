@@ -41,6 +41,9 @@ struct SlotCtl {
   int32_t nsw;             // sweeps per interval
   int64_t measure_from;
   unsigned long long done_ns;  // device time stamp when intervals_left reached 0
+  // intervals that were left when the launch started and intervals it has completed since
+  int32_t left0;
+  uint32_t done;
 };
 
 // Arguments of the fused exchange tail.  Partials are [Rcap][S]; counter is zero between launches
@@ -555,7 +558,10 @@ __device__ __forceinline__ void interval_tail(const RealView &v, int G, int r0, 
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
         c->done_ns = t;
       }
+      // the realization's next interval may start: everything its CTAs wrote is ordered before this by
+      // their arrivals and the barriers above
       __threadfence();
+      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&c->done), "r"(c->done + 1u) : "memory");
     }
   }
   __syncthreads();

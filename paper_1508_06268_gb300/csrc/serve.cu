@@ -162,7 +162,7 @@ struct rfim_server {
   SlotCtl *d_ctls = nullptr;
   BatchItem *d_items = nullptr;
   BatchQueue *d_queue = nullptr;
-  unsigned int *d_err = nullptr;  // device error word of the batched launches (debug-build checks)
+  unsigned int *d_err = nullptr;  // device error word of the batched launches, after d_ctls' last entry
   std::vector<Slot> slots;
   std::vector<SlotCtl> h_ctls;
   std::deque<Request> pending;
@@ -431,6 +431,7 @@ void refresh(rfim_server *s) {
       ctl.intervals_left = (int32_t)(rq.sweeps / rq.ex);
       ctl.nsw = rq.ex;
       ctl.measure_from = rq.measure_from;
+      ctl.left0 = ctl.intervals_left;
       s->h_ctls[free_slot] = ctl;
       copy_sync(s, s->d_ctls + free_slot, &ctl, sizeof ctl, cudaMemcpyHostToDevice);
       s->items_dirty = true;
@@ -474,16 +475,15 @@ void worker_loop(rfim_server *s) {
     cudaError_t e = cudaGraphLaunch(s->gexec, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e == cudaSuccess)
-      e = copy_sync(s, s->h_ctls.data(), s->d_ctls, sizeof(SlotCtl) * s->max_slots, cudaMemcpyDeviceToHost);
-    if (kDebugBuild && e == cudaSuccess) {  // debug build: bounds checks of this replay
-      unsigned int word = 0;
-      e = copy_sync(s, &word, s->d_err, 4, cudaMemcpyDeviceToHost);
-      if (e == cudaSuccess && word) {
-        std::lock_guard<std::mutex> lk(s->mu);
-        s->fatal = RFIM_EBOUNDS;
-        s->err = "batched launch: a bounds check of the debug build failed";
-        return;
-      }
+      e = copy_sync(s, s->h_ctls.data(), s->d_ctls, sizeof(SlotCtl) * (s->max_slots + 1), cudaMemcpyDeviceToHost);
+    unsigned int word = 0;  // bounded waits and, in the debug build, bounds checks of this replay
+    memcpy(&word, s->h_ctls.data() + s->max_slots, sizeof word);
+    if (e == cudaSuccess && word) {
+      std::lock_guard<std::mutex> lk(s->mu);
+      s->fatal = word & kDbgMask ? RFIM_EBOUNDS : RFIM_ETIMEOUT;
+      s->err = word & kDbgMask ? "batched launch: a bounds check of the debug build failed"
+                               : "batched launch: a bounded device wait expired";
+      return;
     }
     s->busy_s += seconds(t0, Clock::now());
     s->graph_launches += 1;
@@ -508,7 +508,7 @@ void destroy_server(rfim_server *s) {
   if (s->stream) cudaStreamSynchronize(s->stream);
   if (s->gexec) cudaGraphExecDestroy(s->gexec);
   if (s->graph) cudaGraphDestroy(s->graph);
-  void *ptrs[] = {s->arena.base, s->d_slots, s->d_ctls, s->d_items, s->d_queue, s->d_err};
+  void *ptrs[] = {s->arena.base, s->d_slots, s->d_ctls, s->d_items, s->d_queue};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (s->stream) cudaStreamDestroy(s->stream);
@@ -541,7 +541,7 @@ int rfim_server_create(const rfim_server_config *cfg, rfim_server **out) {
   s->K = cfg->intervals_per_launch > 0 ? cfg->intervals_per_launch : (tuned_k > 0 ? tuned_k : 4);
   s->measure_xi = cfg->measure_xi != 0;
   s->slots.resize(s->max_slots);
-  s->h_ctls.assign(s->max_slots, SlotCtl{});
+  s->h_ctls.assign(s->max_slots + 1, SlotCtl{});  // the last entry stands for the error word
   auto bail = [&](int code, const std::string &msg) {
     g_server_error = msg;
     cudaGetLastError();
@@ -556,13 +556,12 @@ int rfim_server_create(const rfim_server_config *cfg, rfim_server **out) {
   s->arena.free_[0] = cfg->mem_budget_bytes;
   const size_t nitems_max = (size_t)s->max_slots * kMaxItemsPerSlot;
   if ((e = cudaMalloc(&s->d_slots, sizeof(SlotDesc) * s->max_slots)) != cudaSuccess ||
-      (e = cudaMalloc(&s->d_ctls, sizeof(SlotCtl) * s->max_slots)) != cudaSuccess ||
+      (e = cudaMalloc(&s->d_ctls, sizeof(SlotCtl) * (s->max_slots + 1))) != cudaSuccess ||
       (e = cudaMalloc(&s->d_items, sizeof(BatchItem) * nitems_max)) != cudaSuccess ||
-      (e = cudaMalloc(&s->d_queue, sizeof(BatchQueue))) != cudaSuccess ||
-      (e = cudaMalloc(&s->d_err, sizeof(unsigned int))) != cudaSuccess)
+      (e = cudaMalloc(&s->d_queue, sizeof(BatchQueue))) != cudaSuccess)
     return bail(RFIM_ENOMEM, std::string("tables: ") + cudaGetErrorString(e));
-  cudaMemsetAsync(s->d_err, 0, sizeof(unsigned int), s->stream);
-  cudaMemsetAsync(s->d_ctls, 0, sizeof(SlotCtl) * s->max_slots, s->stream);
+  s->d_err = reinterpret_cast<unsigned int *>(s->d_ctls + s->max_slots);
+  cudaMemsetAsync(s->d_ctls, 0, sizeof(SlotCtl) * (s->max_slots + 1), s->stream);
   cudaMemsetAsync(s->d_queue, 0, sizeof(BatchQueue), s->stream);
   cudaStreamSynchronize(s->stream);
   for (const auto &kv : s->shapes) s->smem = std::max(s->smem, batch_smem(kv.first, kv.second.G));
@@ -572,10 +571,12 @@ int rfim_server_create(const rfim_server_config *cfg, rfim_server **out) {
   if ((e = batch_occupancy(s->smem, &per_sm)) != cudaSuccess || per_sm < 1)
     return bail(RFIM_ECUDA, "batched kernel does not fit on an SM");
   s->grid = sms * per_sm;
-  // capture K persistent launches once; every later step replays the graph
+  // capture the persistent launch (K intervals) once; every later step replays the graph
   e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
-  for (int k = 0; k < s->K && e == cudaSuccess; ++k)
-    e = launch_batch(s->grid, s->smem, s->d_slots, s->d_ctls, s->d_items, s->d_queue, s->stream);
+  // (the queue counts items in 32 bits: fewer intervals per launch than asked for where they would not fit)
+  const int intervals = (int)std::min<int64_t>(s->K, std::max<int64_t>(1, ((int64_t)1 << 30) / (int64_t)nitems_max));
+  if (e == cudaSuccess)
+    e = launch_batch(s->grid, s->smem, s->d_slots, s->d_ctls, s->max_slots, s->d_items, s->d_queue, intervals, s->d_err, s->stream);
   cudaError_t e2 = cudaStreamEndCapture(s->stream, &s->graph);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&s->gexec, s->graph, 0);
