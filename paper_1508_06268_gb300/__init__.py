@@ -345,9 +345,9 @@ class Realization:
 
     def get_state(self, spins=True, t2r=True, energies=False):
         R, N = self._R, self.N
-        s = np.zeros((R, N), dtype=np.int8) if spins else None
-        p = np.zeros(R, dtype=np.int32) if t2r else None
-        E = np.zeros(R, dtype=np.float64) if energies else None
+        s = np.empty((R, N), dtype=np.int8) if spins else None  # written whole by the library
+        p = np.empty(R, dtype=np.int32) if t2r else None
+        E = np.empty(R, dtype=np.float64) if energies else None
         sw, xs = C.c_int64(), C.c_int64()
         self._check(self._lib.rfim_get_state(self._h, _ptr(s), _ptr(p), _ptr(E), C.byref(sw),
                                              C.byref(xs)))

@@ -39,7 +39,7 @@ void temperature_tables(const double *T, int32_t R, float J, float h, uint32_t *
     beta[k] = 1.0 / T[k];
     b2[k] = 2.0f * (float)beta[k];
     b2l[k] = (float)(-1.4426950408889634 * (double)b2[k]);
-    bimodal_row(beta[k], J, h, &thr[(size_t)k * 32]);
+    if (thr) bimodal_row(beta[k], J, h, &thr[(size_t)k * 32]);
   }
   for (int u = 0; u < 8; ++u) gjn[u] = J * (float)(2 * u - 6);
 }

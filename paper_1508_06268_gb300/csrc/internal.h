@@ -53,7 +53,7 @@ int set_thread_error(int code, const std::string &msg);
 cudaError_t raise_smem_limit(const void *fn, size_t bytes);
 
 // host_tables.cu: bimodal thresholds (thr - 1, 32 entries per temperature), b2 = 2 beta,
-// b2l = -2 beta log2 e, beta = 1/T, gjn[u] = J (2u - 6)
+// b2l = -2 beta log2 e, beta = 1/T, gjn[u] = J (2u - 6).  thr may be null (float fields have no use for it).
 void bimodal_row(double beta, float J, float h, uint32_t out[32]);
 void temperature_tables(const double *T, int32_t R, float J, float h, uint32_t *thr, float *b2, float *b2l,
                         double *beta, float gjn[8]);

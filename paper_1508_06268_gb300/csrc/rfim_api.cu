@@ -34,6 +34,10 @@ struct rfim_ctx {
   float *hraw = nullptr, *hh_c = nullptr;
   uint8_t *hbit_c = nullptr;
   uint32_t *hbits = nullptr;
+  // the temperature tables and the exchange state are one allocation each (beta_d and n_meas first), so that
+  // uploads, resets and reads are one copy; host images of the uploads
+  std::vector<char> tables_img, state_img;
+  unsigned int err_word = 0;  // the plan's error word as last read
   uint32_t *thr = nullptr;
   float *gjn = nullptr, *b2 = nullptr, *b2l = nullptr;
   double *beta_d = nullptr;
@@ -149,8 +153,7 @@ void free_events(rfim_ctx *c) {
 
 void free_all(rfim_ctx *c) {
   free_events(c);
-  void *ptrs[] = {c->spins8, c->bits, c->hraw, c->hh_c, c->hbit_c, c->hbits, c->thr, c->gjn, c->b2, c->b2l,
-                  c->beta_d, c->t2r, c->r2t, c->E, c->M, c->att, c->acc, c->obs, c->n_meas, c->scratch8,
+  void *ptrs[] = {c->spins8, c->bits, c->hraw, c->hh_c, c->hbit_c, c->hbits, c->beta_d, c->n_meas, c->scratch8,
                   c->sumF, c->eparts.B, c->eparts.M, c->eparts.Fi, c->eparts.F,
                   c->eparts.count};
   for (void *p : ptrs)
@@ -158,20 +161,22 @@ void free_all(rfim_ctx *c) {
   free_bits_plan(c->plan);
 }
 
+// Bytes of the temperature tables (beta, gjn, b2, b2l, then the bimodal thresholds) and of the state (measurement
+// count, sums, pair counts, energies, magnetisations, then the permutation) at capacity Rcap.
+size_t tables_bytes(size_t Rcap, bool thr) { return Rcap * (8 + 4 + 4 + (thr ? 128 : 0)) + 32; }
+size_t state_bytes(size_t Rcap) { return 8 + Rcap * (40 + 8 + 8 + 8 + 8 + 4 + 4); }
+
+// Tables of the current temperatures.  The copy reads tables_img until the caller next synchronises.
 int upload_temps(rfim_ctx *c) {
-  const int32_t R = c->R;
-  std::vector<uint32_t> thr((size_t)R * 32);
-  std::vector<float> b2(R), b2l(R);
-  std::vector<double> beta(R);
-  float gjn[8];
-  temperature_tables(c->T.data(), R, c->J, c->h, thr.data(), b2.data(), b2l.data(), beta.data(), gjn);
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->thr, thr.data(), thr.size() * 4, cudaMemcpyHostToDevice, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->b2, b2.data(), R * 4, cudaMemcpyHostToDevice, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->b2l, b2l.data(), R * 4, cudaMemcpyHostToDevice, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->beta_d, beta.data(), R * 8, cudaMemcpyHostToDevice, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->gjn, gjn, sizeof gjn, cudaMemcpyHostToDevice, c->stream));
-  // pageable sources: make sure the copies have consumed the host vectors before they go away
-  CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
+  const bool bim = c->kind == RFIM_FIELD_BIMODAL;
+  const size_t Rcap = (size_t)c->Rcap;
+  c->tables_img.resize(tables_bytes(Rcap, bim));
+  char *img = c->tables_img.data();
+  auto at = [&](const void *dev) { return img + (reinterpret_cast<const char *>(dev) - reinterpret_cast<const char *>(c->beta_d)); };
+  temperature_tables(c->T.data(), c->R, c->J, c->h, bim ? reinterpret_cast<uint32_t *>(at(c->thr)) : nullptr,
+                     reinterpret_cast<float *>(at(c->b2)), reinterpret_cast<float *>(at(c->b2l)),
+                     reinterpret_cast<double *>(at(c->beta_d)), reinterpret_cast<float *>(at(c->gjn)));
+  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->beta_d, img, c->tables_img.size(), cudaMemcpyHostToDevice, c->stream));
   return RFIM_OK;
 }
 
@@ -183,29 +188,30 @@ int reset_state(rfim_ctx *c, uint32_t stage) {
   RealView v = view_of(c);
   CUDA_OR_FAIL(c, launch_init_spins(v, c->R, stage, c->layout == RFIM_LAYOUT_BITPACK, c->stream));
   c->launches += 1;
-  std::vector<int32_t> id(c->Rcap);
-  std::iota(id.begin(), id.end(), 0);
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->t2r, id.data(), c->Rcap * 4, cudaMemcpyHostToDevice, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->r2t, id.data(), c->Rcap * 4, cudaMemcpyHostToDevice, c->stream));
-  CUDA_OR_FAIL(c, cudaMemsetAsync(c->att, 0, c->Rcap * 8, c->stream));
-  CUDA_OR_FAIL(c, cudaMemsetAsync(c->acc, 0, c->Rcap * 8, c->stream));
-  CUDA_OR_FAIL(c, cudaMemsetAsync(c->obs, 0, (size_t)c->Rcap * 5 * 8, c->stream));
+  c->state_img.assign(state_bytes((size_t)c->Rcap), 0);
+  for (const int32_t *dev : {c->t2r, c->r2t}) {
+    int32_t *id = reinterpret_cast<int32_t *>(c->state_img.data() +
+                                              (reinterpret_cast<const char *>(dev) - reinterpret_cast<const char *>(c->n_meas)));
+    std::iota(id, id + c->Rcap, 0);
+  }
+  CUDA_OR_FAIL(c, cudaMemcpyAsync(c->n_meas, c->state_img.data(), c->state_img.size(), cudaMemcpyHostToDevice, c->stream));
   if (c->sumF) CUDA_OR_FAIL(c, cudaMemsetAsync(c->sumF, 0, (size_t)c->Rcap * 8, c->stream));
-  CUDA_OR_FAIL(c, cudaMemsetAsync(c->n_meas, 0, 8, c->stream));
-  CUDA_OR_FAIL(c, cudaMemsetAsync(c->E, 0, c->Rcap * 8, c->stream));
-  CUDA_OR_FAIL(c, cudaMemsetAsync(c->M, 0, c->Rcap * 8, c->stream));
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
   return RFIM_OK;
 }
 
 // Bounded device waits that expired (bit-layout kernels) surface as RFIM_ETIMEOUT, failed bounds
-// checks of the debug build as RFIM_EBOUNDS; the word is cleared once reported.  Synchronises the
-// stream.
-int check_device_error(rfim_ctx *c) {
+// checks of the debug build as RFIM_EBOUNDS; the word is cleared once reported.  read_error enqueues
+// the copy of the word, report_error comes after the caller's synchronisation.
+int read_error(rfim_ctx *c) {
+  c->err_word = 0;
   if (!c->plan.counter) return RFIM_OK;  // no plan (one int8 launch per half-sweep)
-  unsigned int word = 0;
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(&word, c->plan.counter + 1, 4, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
+  CUDA_OR_FAIL(c, cudaMemcpyAsync(&c->err_word, c->plan.counter + 1, 4, cudaMemcpyDeviceToHost, c->stream));
+  return RFIM_OK;
+}
+
+int report_error(rfim_ctx *c) {
+  const unsigned int word = c->err_word;
   if (!word) return RFIM_OK;
   CUDA_OR_FAIL(c, cudaMemsetAsync(c->plan.counter + 1, 0, 4, c->stream));
   CUDA_OR_FAIL(c, reset_bits_plan(c->plan, c->stream));
@@ -412,19 +418,24 @@ int rfim_create(const rfim_config *cfg, rfim_ctx **out) {
   if ((rc = dalloc(c, &c->hraw, N))) return bail(rc);
   if ((rc = dalloc(c, &c->hh_c, N))) return bail(rc);
   if ((rc = dalloc(c, &c->hbit_c, N))) return bail(rc);
-  if ((rc = dalloc(c, &c->thr, (size_t)Rcap * 32))) return bail(rc);
-  if ((rc = dalloc(c, &c->gjn, 8))) return bail(rc);
-  if ((rc = dalloc(c, &c->b2, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->b2l, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->beta_d, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->t2r, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->r2t, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->E, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->M, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->att, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->acc, Rcap))) return bail(rc);
-  if ((rc = dalloc(c, &c->obs, (size_t)Rcap * 5))) return bail(rc);
-  if ((rc = dalloc(c, &c->n_meas, 1))) return bail(rc);
+  {
+    char *base = nullptr;
+    if ((rc = dalloc(c, &base, tables_bytes((size_t)Rcap, cfg->field_kind == RFIM_FIELD_BIMODAL)))) return bail(rc);
+    c->beta_d = reinterpret_cast<double *>(base);
+    c->gjn = reinterpret_cast<float *>(c->beta_d + Rcap);
+    c->b2 = c->gjn + 8;
+    c->b2l = c->b2 + Rcap;
+    c->thr = reinterpret_cast<uint32_t *>(c->b2l + Rcap);
+    if ((rc = dalloc(c, &base, state_bytes((size_t)Rcap)))) return bail(rc);
+    c->n_meas = reinterpret_cast<int64_t *>(base);
+    c->obs = reinterpret_cast<double *>(c->n_meas + 1);
+    c->att = reinterpret_cast<uint64_t *>(c->obs + (size_t)Rcap * 5);
+    c->acc = c->att + Rcap;
+    c->E = reinterpret_cast<double *>(c->acc + Rcap);
+    c->M = reinterpret_cast<int64_t *>(c->E + Rcap);
+    c->t2r = reinterpret_cast<int32_t *>(c->M + Rcap);
+    c->r2t = c->t2r + Rcap;
+  }
   (void)half;
   if (c->layout == RFIM_LAYOUT_BITPACK || staged_i8) {
     if ((rc = make_bits_plan(L, Rcap, c->kind == kBimodal, &c->plan, &c->err, staged_i8))) return bail(rc);
@@ -498,10 +509,10 @@ int rfim_adapt_temps(rfim_ctx *ctx, int32_t n_trials, int64_t sweeps_per_trial, 
     if ((rc = reset_state(c, (uint32_t)t))) return rc;
     if ((rc = do_run(c, sweeps_per_trial, exchange_every, INT64_MAX))) return rc;
     const int32_t np = c->R - 1;
-    std::vector<uint64_t> att(np), acc(np);
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(att.data(), c->att, np * 8, cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(acc.data(), c->acc, np * 8, cudaMemcpyDeviceToHost, c->stream));
+    std::vector<uint64_t> counts(2 * (size_t)c->Rcap);  // att, then acc
+    CUDA_OR_FAIL(c, cudaMemcpyAsync(counts.data(), c->att, counts.size() * 8, cudaMemcpyDeviceToHost, c->stream));
     CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
+    const uint64_t *att = counts.data(), *acc = att + c->Rcap;
     std::vector<double> rate(np);
     for (int32_t k = 0; k < np; ++k) rate[k] = att[k] ? (double)acc[k] / (double)att[k] : 0.0;
     if (rates_out)
@@ -530,32 +541,31 @@ int rfim_adapt_temps(rfim_ctx *ctx, int32_t n_trials, int64_t sweeps_per_trial, 
 int rfim_observables(rfim_ctx *ctx, rfim_obs *out) {
   if (!ctx || !out) return RFIM_EINVAL;
   rfim_ctx *c = ctx;
-  if (int rc = check_device_error(c)) return rc;
+  // everything is read behind one synchronisation: the count, the sums and the pair counts are one span
   const int32_t R = c->R;
-  std::vector<double> obs((size_t)R * 5);
-  std::vector<uint64_t> att(R), acc(R);
-  int64_t nm = 0;
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(obs.data(), c->obs, obs.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(att.data(), c->att, R * 8, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(acc.data(), c->acc, R * 8, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_OR_FAIL(c, cudaMemcpyAsync(&nm, c->n_meas, 8, cudaMemcpyDeviceToHost, c->stream));
+  const size_t Rcap = (size_t)c->Rcap;
+  std::vector<double> span(1 + Rcap * 7), F(c->sumF && out->F ? R : 0);
+  if (int rc = read_error(c)) return rc;
+  CUDA_OR_FAIL(c, cudaMemcpyAsync(span.data(), c->n_meas, span.size() * 8, cudaMemcpyDeviceToHost, c->stream));
+  if (!F.empty()) CUDA_OR_FAIL(c, cudaMemcpyAsync(F.data(), c->sumF, F.size() * 8, cudaMemcpyDeviceToHost, c->stream));
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
+  if (int rc = report_error(c)) return rc;
+  const double *obs = span.data() + 1;
+  const char *att = reinterpret_cast<const char *>(obs + Rcap * 5), *acc = att + Rcap * 8;
   out->R = R;
-  out->n_meas = nm;
+  memcpy(&out->n_meas, span.data(), 8);
   double *cols[5] = {out->e, out->e2, out->absm, out->m2, out->m4};
   for (int q = 0; q < 5; ++q)
     if (cols[q])
       for (int32_t k = 0; k < R; ++k) cols[q][k] = obs[(size_t)k * 5 + q];
   if (out->T) std::copy(c->T.begin(), c->T.end(), out->T);
-  if (out->att) std::copy(att.begin(), att.begin() + (R - 1), out->att);
-  if (out->acc) std::copy(acc.begin(), acc.begin() + (R - 1), out->acc);
+  if (out->att) memcpy(out->att, att, (size_t)(R - 1) * 8);
+  if (out->acc) memcpy(out->acc, acc, (size_t)(R - 1) * 8);
   if (out->F) {
-    if (c->sumF) {
-      CUDA_OR_FAIL(c, cudaMemcpyAsync(out->F, c->sumF, (size_t)R * 8, cudaMemcpyDeviceToHost, c->stream));
-      CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
-    } else {
+    if (!F.empty())
+      std::copy(F.begin(), F.end(), out->F);
+    else
       std::fill(out->F, out->F + R, 0.0);
-    }
   }
   return RFIM_OK;
 }
@@ -691,7 +701,7 @@ int rfim_disorder_average(const double *thermals, int32_t n, int32_t R, double *
 int rfim_get_state(rfim_ctx *ctx, int8_t *spins, int32_t *t2r, double *E, int64_t *sweep, int64_t *xstep) {
   if (!ctx) return RFIM_EINVAL;
   rfim_ctx *c = ctx;
-  if (int rc = check_device_error(c)) return rc;
+  if (int rc = read_error(c)) return rc;
   const size_t RN = (size_t)c->R * c->N;
   RealView v = view_of(c);
   if (spins) {
@@ -712,6 +722,7 @@ int rfim_get_state(rfim_ctx *ctx, int8_t *spins, int32_t *t2r, double *E, int64_
     CUDA_OR_FAIL(c, cudaMemcpyAsync(E, c->E, c->R * 8, cudaMemcpyDeviceToHost, c->stream));
   }
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
+  if (int rc = report_error(c)) return rc;
   if (sweep) *sweep = c->sweep;
   if (xstep) *xstep = c->xstep;
   return RFIM_OK;

@@ -101,6 +101,9 @@ struct Slot {
   Clock::time_point arrival, admitted;
   std::vector<double> T;
   int64_t attempts = 0;
+  std::vector<char> image;           // host side of the slot's upload
+  const char *results = nullptr;     // device span of att, acc, obs, n_meas and sumF
+  size_t results_bytes = 0;
 };
 
 // Replicas per work item and per thread for each L in batched launches (S = 1: whole replicas).
@@ -239,6 +242,8 @@ int init_slot(rfim_server *s, Slot &sl, const Request &rq) {
   float *hraw = (float *)take(N * 4);
   float *hh_c = (float *)take(N * 4);
   uint8_t *hbit_c = (uint8_t *)take(N);
+  // from here on the slot is uploaded as one image: tables, identity permutation, zeros
+  char *const image = p;
   uint32_t *thr = (uint32_t *)take((size_t)R * 32 * 4);
   float *gjn = (float *)take(32);
   float *b2 = (float *)take(R * 4);
@@ -248,10 +253,6 @@ int init_slot(rfim_server *s, Slot &sl, const Request &rq) {
   v.r2t = (int32_t *)take(R * 4);
   v.E = (double *)take(R * 8);
   v.M = (int64_t *)take(R * 8);
-  v.att = (uint64_t *)take(R * 8);
-  v.acc = (uint64_t *)take(R * 8);
-  v.obs = (double *)take((size_t)R * 40);
-  v.n_meas = (int64_t *)take(8);
   ExchArgs xa{};
   xa.partB = (long long *)take(R * 8);
   xa.partM = (long long *)take(R * 8);
@@ -262,12 +263,19 @@ int init_slot(rfim_server *s, Slot &sl, const Request &rq) {
   double *kwave = nullptr;
   if (s->measure_xi) {
     xa.Fr = (double *)take(R * 8);
-    xa.sumF = (double *)take(R * 8);
     kwave = (double *)take(L * 8);
     double *ks = (double *)take(L * 8);
     xa.kcos = kwave;
     xa.ksin = ks;
   }
+  // the results, read back as one span
+  v.att = (uint64_t *)take(R * 8);
+  v.acc = (uint64_t *)take(R * 8);
+  v.obs = (double *)take((size_t)R * 40);
+  v.n_meas = (int64_t *)take(8);
+  if (s->measure_xi) xa.sumF = (double *)take(R * 8);
+  sl.results = (char *)v.att;
+  sl.results_bytes = (size_t)(p - sl.results);
   v.hh_c = hh_c; v.hbit_c = hbit_c; v.hbits = hbits; v.thr = thr; v.gjn = gjn; v.b2 = b2; v.b2l = b2l;
   v.beta_d = beta;
 
@@ -297,31 +305,17 @@ int init_slot(rfim_server *s, Slot &sl, const Request &rq) {
     xa.fquant = fquant;
   }
   if (!ck(launch_init_spins(v, R, 0, true, st), "init")) return RFIM_ECUDA;
-  std::vector<uint32_t> thr_h((size_t)R * 32);
-  std::vector<float> b2_h(R), b2l_h(R);
-  std::vector<double> beta_h(R);
-  float gjn_h[8];
-  temperature_tables(rq.temps.data(), R, c.J, c.h, thr_h.data(), b2_h.data(), b2l_h.data(), beta_h.data(), gjn_h);
-  std::vector<int32_t> id(R);
-  std::iota(id.begin(), id.end(), 0);
-  std::vector<double> wave(2 * (size_t)L);
-  if (kwave) wave_tables(L, wave.data(), wave.data() + L);
-  bool ok = ck(cudaMemcpyAsync(thr, thr_h.data(), thr_h.size() * 4, cudaMemcpyHostToDevice, st), "tables") &&
-            ck(cudaMemcpyAsync(b2, b2_h.data(), R * 4, cudaMemcpyHostToDevice, st), "tables") &&
-            ck(cudaMemcpyAsync(b2l, b2l_h.data(), R * 4, cudaMemcpyHostToDevice, st), "tables") &&
-            ck(cudaMemcpyAsync(beta, beta_h.data(), R * 8, cudaMemcpyHostToDevice, st), "tables") &&
-            ck(cudaMemcpyAsync(gjn, gjn_h, 32, cudaMemcpyHostToDevice, st), "tables") &&
-            ck(cudaMemcpyAsync(v.t2r, id.data(), R * 4, cudaMemcpyHostToDevice, st), "perm") &&
-            ck(cudaMemcpyAsync(v.r2t, id.data(), R * 4, cudaMemcpyHostToDevice, st), "perm") &&
-            ck(cudaMemsetAsync(v.E, 0, R * 8, st), "zero") && ck(cudaMemsetAsync(v.M, 0, R * 8, st), "zero") &&
-            ck(cudaMemsetAsync(v.att, 0, R * 8, st), "zero") && ck(cudaMemsetAsync(v.acc, 0, R * 8, st), "zero") &&
-            ck(cudaMemsetAsync(v.obs, 0, (size_t)R * 40, st), "zero") &&
-            ck(cudaMemsetAsync(v.n_meas, 0, 8, st), "zero") && ck(cudaMemsetAsync(xa.counter, 0, 4, st), "zero") &&
-            (!kwave || (ck(cudaMemsetAsync(xa.sumF, 0, R * 8, st), "zero") &&
-                        ck(cudaMemcpyAsync(kwave, wave.data(), L * 8, cudaMemcpyHostToDevice, st), "tables") &&
-                        ck(cudaMemcpyAsync((void *)xa.ksin, wave.data() + L, L * 8, cudaMemcpyHostToDevice, st), "tables"))) &&
-            ck(cudaStreamSynchronize(st), "slot init");
-  if (!ok) return RFIM_ECUDA;
+  std::vector<char> &img = sl.image;  // read by the copy until refresh next synchronises
+  img.assign((size_t)(p - image), 0);
+  auto host = [&](const void *dev) { return img.data() + ((const char *)dev - image); };
+  temperature_tables(rq.temps.data(), R, c.J, c.h, c.field_kind == kBimodal ? (uint32_t *)host(thr) : nullptr, (float *)host(b2),
+                     (float *)host(b2l), (double *)host(beta), (float *)host(gjn));
+  std::iota((int32_t *)host(v.t2r), (int32_t *)host(v.t2r) + R, 0);
+  std::iota((int32_t *)host(v.r2t), (int32_t *)host(v.r2t) + R, 0);
+  if (kwave) wave_tables(L, (double *)host(xa.kcos), (double *)host(xa.ksin));
+  if (!ck(cudaMemcpyAsync(image, img.data(), img.size(), cudaMemcpyHostToDevice, st), "slot image")) return RFIM_ECUDA;
+  // the caller's field array is gone once the request is: its upload must be done before this returns
+  if (c.field_kind == RFIM_FIELD_EXPLICIT && !ck(cudaStreamSynchronize(st), "slot init")) return RFIM_ECUDA;
   const BatchShape sh = s->shapes.at(L);
   xa.J = (double)c.J;
   xa.h = (double)c.h;
@@ -341,23 +335,32 @@ int init_slot(rfim_server *s, Slot &sl, const Request &rq) {
 // Retires finished realizations (reads their observables), admits pending requests while slots
 // and arena memory allow, and refreshes the device descriptors and work queue.  Stream idle.
 void refresh(rfim_server *s) {
+  std::vector<std::pair<int, std::vector<char>>> finished;
+  finished.reserve((size_t)s->max_slots);  // the copies' destinations stay where they are
   for (int i = 0; i < s->max_slots; ++i) {
     Slot &sl = s->slots[i];
     if (!sl.used || s->h_ctls[i].intervals_left > 0) continue;
+    finished.emplace_back(i, std::vector<char>(sl.results_bytes));
+    cudaMemcpyAsync(finished.back().second.data(), sl.results, sl.results_bytes, cudaMemcpyDeviceToHost, s->stream);
+  }
+  if (!finished.empty()) cudaStreamSynchronize(s->stream);
+  for (const auto &f : finished) {
+    Slot &sl = s->slots[f.first];
     Result res;
     const RealView &v = sl.desc.v;
+    auto read = [&](void *out, const void *dev, size_t bytes) { memcpy(out, f.second.data() + ((const char *)dev - sl.results), bytes); };
     res.R = sl.R;
     res.T = sl.T;
     res.obs.resize((size_t)sl.R * 5);
     res.att.resize(sl.R);
     res.acc.resize(sl.R);
-    copy_sync(s, res.obs.data(), v.obs, res.obs.size() * 8, cudaMemcpyDeviceToHost);
-    copy_sync(s, res.att.data(), v.att, sl.R * 8, cudaMemcpyDeviceToHost);
-    copy_sync(s, res.acc.data(), v.acc, sl.R * 8, cudaMemcpyDeviceToHost);
-    copy_sync(s, &res.n_meas, v.n_meas, 8, cudaMemcpyDeviceToHost);
+    read(res.obs.data(), v.obs, res.obs.size() * 8);
+    read(res.att.data(), v.att, sl.R * 8);
+    read(res.acc.data(), v.acc, sl.R * 8);
+    read(&res.n_meas, v.n_meas, 8);
     if (sl.desc.xa.sumF) {
       res.F.resize(sl.R);
-      copy_sync(s, res.F.data(), sl.desc.xa.sumF, sl.R * 8, cudaMemcpyDeviceToHost);
+      read(res.F.data(), sl.desc.xa.sumF, sl.R * 8);
     }
     const Clock::time_point now = Clock::now();
     res.latency_s = seconds(sl.arrival, now);
@@ -420,6 +423,7 @@ void refresh(rfim_server *s) {
         bad.code = rc;
         bad.msg = s->err;
         s->done[rq.ticket] = bad;
+        cudaStreamSynchronize(s->stream);  // nothing reads the slot's image any more
         s->arena.release(off, need);
         sl.used = false;
         s->resident -= 1;
@@ -433,25 +437,30 @@ void refresh(rfim_server *s) {
       ctl.measure_from = rq.measure_from;
       ctl.left0 = ctl.intervals_left;
       s->h_ctls[free_slot] = ctl;
-      copy_sync(s, s->d_ctls + free_slot, &ctl, sizeof ctl, cudaMemcpyHostToDevice);
       s->items_dirty = true;
     }
   }
   if (!s->items_dirty) return;
   std::vector<BatchItem> items;
+  std::vector<SlotDesc> descs((size_t)s->max_slots);
   for (int i = 0; i < s->max_slots; ++i) {
     Slot &sl = s->slots[i];
     if (!sl.used) continue;
     for (int r0 = 0; r0 < sl.R; r0 += sl.desc.G) items.push_back(BatchItem{i, r0, std::min(sl.desc.G, sl.R - r0), 0});
-    copy_sync(s, s->d_slots + i, &sl.desc, sizeof(SlotDesc), cudaMemcpyHostToDevice);
+    descs[(size_t)i] = sl.desc;
   }
   // largest items first so that the long ones start early
   std::stable_sort(items.begin(), items.end(), [&](const BatchItem &a, const BatchItem &b) {
     return (int64_t)a.gact * s->slots[a.slot].N > (int64_t)b.gact * s->slots[b.slot].N;
   });
-  if (!items.empty()) copy_sync(s, s->d_items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice);
+  // the device's control words are those of h_ctls but for the realizations admitted here
+  auto put = [&](void *dst, const void *src, size_t bytes) { cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s->stream); };
+  put(s->d_slots, descs.data(), descs.size() * sizeof(SlotDesc));
+  put(s->d_ctls, s->h_ctls.data(), (size_t)s->max_slots * sizeof(SlotCtl));
+  if (!items.empty()) put(s->d_items, items.data(), items.size() * sizeof(BatchItem));
   BatchQueue q{0u, 0u, (int32_t)items.size(), 0};
-  copy_sync(s, s->d_queue, &q, sizeof q, cudaMemcpyHostToDevice);
+  put(s->d_queue, &q, sizeof q);
+  cudaStreamSynchronize(s->stream);
   s->items_dirty = false;
 }
 
