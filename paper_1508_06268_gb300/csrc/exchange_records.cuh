@@ -88,34 +88,15 @@ __device__ __forceinline__ void record_load(const uint4 *rec, long long *F, unsi
 __device__ __forceinline__ int record_bonds(unsigned long long hi) { return (int)((hi >> 20) & 0x3FFFFFu) - (1 << 21); }
 __device__ __forceinline__ int record_spin(unsigned long long hi) { return (int)(hi & 0xFFFFFu) - (1 << 19); }
 
-// Sums of n consecutive records of interval `epoch`, polled at most kRecordSpinLimit times; false
-// when they did not all arrive (recorded in *err) or an earlier wait of this launch expired.
-// REAL: the 64-bit field sums are doubles, added in record order.
-template <bool REAL>
-__device__ __forceinline__ bool records_sum(const uint4 *rec, int n, uint32_t epoch, unsigned *err, int *B, int *M,
-                                            long long *F) {
+// The record of interval `epoch`, polled at most kRecordSpinLimit times; false when it did not arrive
+// (recorded in *err) or an earlier wait of this launch expired.
+__device__ __forceinline__ bool record_await(const uint4 *rec, uint32_t epoch, unsigned *err, int *B, int *M, long long *F) {
   for (unsigned it = 0; it < kRecordSpinLimit; ++it) {
-    int b = 0, m = 0;
-    long long f = 0;
-    double fd = 0.0;
-    bool all = true;
-#pragma unroll 4
-    for (int q = 0; q < n; ++q) {
-      long long fq;
-      unsigned long long hi;
-      record_load(rec + q, &fq, &hi);
-      all = all && (uint32_t)(hi >> 42) == epoch;
-      b += record_bonds(hi);
-      m += record_spin(hi);
-      if (REAL)
-        fd = __dadd_rn(fd, __longlong_as_double(fq));
-      else
-        f += fq;
-    }
-    if (all) {
-      *B = b;
-      *M = m;
-      *F = REAL ? __double_as_longlong(fd) : f;
+    unsigned long long hi;
+    record_load(rec, F, &hi);
+    if ((uint32_t)(hi >> 42) == epoch) {
+      *B = record_bonds(hi);
+      *M = record_spin(hi);
       return true;
     }
     if ((it & 63u) == 63u && *(volatile unsigned *)err) break;
@@ -174,12 +155,44 @@ __device__ __forceinline__ void exchange_from_records(const RealView &v, const E
   };
   // the random number of the first pair does not depend on the energies
   const uint32_t u0 = p0 + 1 < R ? random_of(p0) : 0u;
-  for (int r = tid; r < R; r += nt) {
-    int B, M;
-    long long Fs;
-    records_sum<REAL>(rec + (size_t)r * S, S, epoch, xa.err, &B, &M, &Fs);
-    xs.E[r] = energy_of(B, Fs);
-    xs.M[r] = M;
+  // One lane per record, the S lanes of a replica (a power of two up to 16) then add theirs in a tree;
+  // REAL: the 64-bit field sums are doubles.  Every CTA polls every record, so the lines they lie in
+  // are what the step waits for: a warp's load takes each line once (a lane per replica that read
+  // its S records one after another took it S times; L = 24, R = 40, eight slabs: 8.7 us for the
+  // whole tail of an interval, now 6.4).
+  if (S == 1 || (S & (S - 1)) != 0) {  // one slab, or a number of slabs that no default shape has
+    for (int r = tid; r < R; r += nt) {
+      int B = 0, M = 0;
+      long long F = 0;
+      for (int q = 0; q < S; ++q) {
+        int b, m;
+        long long f;
+        record_await(rec + (size_t)r * S + q, epoch, xa.err, &b, &m, &f);
+        B += b;
+        M += m;
+        F = REAL && q > 0 ? __double_as_longlong(__dadd_rn(__longlong_as_double(F), __longlong_as_double(f))) : F + f;
+      }
+      xs.E[r] = energy_of(B, F);
+      xs.M[r] = M;
+    }
+  } else {
+    for (int n0 = (tid >> 5) * 32; n0 < R * S; n0 += nt & ~31) {
+      const int n = n0 + (tid & 31), r = n / S;
+      int B = 0, M = 0;
+      long long F = 0;
+      if (n < R * S) record_await(rec + n, epoch, xa.err, &B, &M, &F);
+      __syncwarp();
+      for (int o = S / 2; o > 0; o >>= 1) {
+        B += __shfl_xor_sync(0xffffffffu, B, o);
+        M += __shfl_xor_sync(0xffffffffu, M, o);
+        const long long G = __shfl_xor_sync(0xffffffffu, F, o);
+        F = REAL ? __double_as_longlong(__dadd_rn(__longlong_as_double(F), __longlong_as_double(G))) : F + G;
+      }
+      if (n < R * S && n % S == 0) {
+        xs.E[r] = energy_of(B, F);
+        xs.M[r] = M;
+      }
+    }
   }
   __syncthreads();
   for (int k = p0; k + 1 < R; k += 2 * nt) {

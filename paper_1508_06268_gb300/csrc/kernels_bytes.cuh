@@ -275,17 +275,15 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     if (!xa.enabled) break;
 
     // ---- energies (Eq. 1): small replicas by one warp each, others by the whole CTA ---------------
+    // ONE with one replica: every thread has its block's places and field in registers, for both colours
     const uint32_t epoch = ba.epoch0 + (uint32_t)iv;
     uint4 *rec = ba.rec + (size_t)(epoch & 1u) * ba.rcap * S;
-    const bool by_warp = nblk <= 256 && gact > 1;
+    const bool own_blocks = ONE && gact == 1, by_warp = nblk <= 256 && gact > 1;
     const int t0 = by_warp ? lane : tid, dt = by_warp ? 32 : nt;
     for (int g = by_warp ? wid : 0; ok && g < gact; g += by_warp ? nw : 1) {
       int B = 0, M = 0, Fi = 0;
       float fs = 0.f, fe = 0.f;
-      for (int t = t0; t < 2 * nblk; t += dt) {
-        const int c = t >= nblk, b = b0 + t - (c ? nblk : 0);
-        RowWord rw[NR];
-        locate(b, c, rw);
+      auto add_block = [&](int c, const RowWord (&rw)[NR], uint32_t hb, const float4 &h4) {
         uint32_t cur, up, mine;
         gather(lat + (size_t)(2 * g) * CS, c, rw, cur, up, mine);
         const int n = __popc(mine), ups = __popc(cur);
@@ -293,9 +291,8 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
         // sum of s (2 up - 6) over the sites, s = 2 cur - 1 (colour 0: every bond once)
         if (c == 0) B += 4 * (int)__dp4a(cur, up, 0u) - 12 * ups - 2 * (int)__dp4a(up, 0x01010101u, 0u) + 6 * n;
         if (BIM) {
-          Fi += n - 2 * __popc((cur ^ field_bytes(c, b)) & mine);
+          Fi += n - 2 * __popc((cur ^ hb) & mine);
         } else {
-          const float4 h4 = field_of(c, b);
           const float hk[4] = {h4.x, h4.y, h4.z, h4.w};
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -306,6 +303,19 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
             fe = __fadd_rn(fe, __fadd_rn(__fsub_rn(fs, __fsub_rn(sum, bp)), __fsub_rn(term, bp)));
             fs = sum;
           }
+        }
+      };
+      if (own_blocks) {
+        if (valid) {
+#pragma unroll
+          for (int c = 0; c < 2; ++c) add_block(c, own, hbown[c], hown[c]);
+        }
+      } else {
+        for (int t = t0; t < 2 * nblk; t += dt) {
+          const int c = t >= nblk, b = b0 + t - (c ? nblk : 0);
+          RowWord rw[NR];
+          locate(b, c, rw);
+          add_block(c, rw, field_bytes(c, b), field_of(c, b));
         }
       }
       ChunkSum sum;

@@ -175,3 +175,10 @@ def test_resident_bytes_match_oracle(L, R, plan, kind, monkeypatch):
         x.exchange(0)
     np.testing.assert_array_equal(g.get_state()["t2r"], o.perm()[0])
     np.testing.assert_allclose(g.observables()["sums"], o.observables(), rtol=1e-9)
+
+
+@pytest.mark.parametrize("L,R,plan", [(6, 3, "3,1,4,32,b"), (14, 5, "5,2,4,256,b")])
+@pytest.mark.parametrize("kind", [rf.FIELD_BIMODAL, rf.FIELD_EXPLICIT])
+def test_resident_bytes_slabs_not_a_power_of_two(L, R, plan, kind, monkeypatch):
+    """Slab counts that only a named shape has: their records are added one after another."""
+    test_resident_bytes_match_oracle(L, R, plan, kind, monkeypatch)
