@@ -143,7 +143,8 @@ int rfim_observables(rfim_ctx *ctx, rfim_obs *out);
    length of Sec. 7 needs, read with the spins s_i for the printed h_i:
    F = (F1 + F2) / (3 L^3), F1 = sum over the axes d of (sum_i s_i cos(K i_d))^2, F2 the same with
    sin, K = 2 pi / L.  When enabled, every measuring exchange step (j >= measure_from) adds each
-   replica's F to the sum of its temperature index, one extra launch per step.  Enable it before the
+   replica's F to the sum of its temperature index: on the resident plan inside the sweep launch and by
+   one kernel after it, else by one extra launch per step.  Enable it before the
    first measurement (RFIM_ESTATE otherwise); rfim_adapt_temps and restarts clear the sums with the
    other accumulators.  Synchronous. */
 int rfim_set_measure_xi(rfim_ctx *ctx, int32_t on);
@@ -157,9 +158,9 @@ int rfim_set_measure_xi(rfim_ctx *ctx, int32_t on);
    (q >> 2, r, s mh + h mod 2^32, c3(METRO, stage, fine colour)), so counters repeat after
    2^32 / mh sweeps.  The paper keeps mh = 0 for its physics results; the multi-hit chain has the
    same Boltzmann law but other dynamics.  Bit layout only; tile in {8, 16, 32}, L in {16, 32, 64}
-   divisible by 2 tile.  When the current launch shape has no multi-hit kernel (the grid-wide plan
-   of L = 64) the context switches to the default cluster shape of its L (synchronous in that
-   case).  Errors: RFIM_EINVAL (mh < 0, int8 layout, unsupported tile), RFIM_ENOMEM / RFIM_ECUDA
+   divisible by 2 tile.  When the current launch shape has no multi-hit kernel the context gets a
+   resident shape for multi-hit sweeps beside it, or, where there is none or it would be slower (many
+   replicas at L = 64), switches to the default cluster shape of its L (synchronous in both cases).  Errors: RFIM_EINVAL (mh < 0, int8 layout, unsupported tile), RFIM_ENOMEM / RFIM_ECUDA
    from the plan switch. */
 int rfim_set_multihit(rfim_ctx *ctx, int32_t mh, int32_t tile);
 
@@ -202,7 +203,7 @@ int64_t rfim_launch_count(const rfim_ctx *ctx);
    The quenched average (Sec. 7) needs many independent realizations.  A server owns a device
    memory arena and a worker thread: submitted realizations are admitted in arrival order as slots
    and arena memory free up; all resident ones advance together, intervals_per_launch exchange
-   intervals per replay of a captured CUDA graph of persistent batched kernels; finished ones are
+   intervals per replay of a captured launch of the persistent batched kernel; finished ones are
    retired between replays and their observables kept until polled.  Each result is the same as
    the realization run alone through the server (nothing is shared between realizations).  The
    bit layout is used (L in {8, 16, 32, 64}, R <= 1024). */

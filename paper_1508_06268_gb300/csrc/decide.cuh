@@ -47,7 +47,7 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // Rejections of a bimodal test collected as carries: the table holds ~(thr - 1), so that
 // word + ~(thr - 1) carries out exactly when word > thr - 1, and fk becomes 2 fk + carry.  Two
 // additions, which issue at twice the rate of a comparison and a predicated logic operation
-// (5.9 against 5.5 attempts per clock and SM with Philox).
+// (5.92 attempts per clock and SM with Philox against 5.46, round keys from the constant bank in both).
 __device__ __forceinline__ void collect_reject(uint32_t word, uint32_t not_thr, uint32_t &fk) {
   asm("{\n\t.reg .u32 x;\n\tadd.cc.u32 x, %1, %2;\n\taddc.u32 %0, %0, %0;\n\t}" : "+r"(fk) : "r"(word), "r"(not_thr));
 }
@@ -60,8 +60,9 @@ __device__ __forceinline__ uint32_t accept_float_sign(uint32_t word, float bjn, 
   return __float_as_uint(__fmaf_rn(ex2_approx(boltzmann_exponent(bjn, hh, b)), -4294967296.0f, __uint2float_rz(word)));
 }
 
-// accept_float_sign of two sites, the two differences by one packed FMA (each rounded on its own):
-// 5.09 against 4.96 attempts per clock and SM with Philox, 5.21 with the signs collected by prmt.
+// accept_float_sign of two sites, the two differences by one packed FMA (each rounded on its own).
+// With the signs collected by prmt 5.11 attempts per clock and SM with Philox against 4.96 for one
+// difference and one shift per site (round keys from the constant bank in both).
 __device__ __forceinline__ uint2 accept_float_signs(uint32_t w0, uint32_t w1, float2 e0, float2 e1, float h0, float h1) {
   uint2 r;
   asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\tmov.b64 c, {%5, %6};\n\t"

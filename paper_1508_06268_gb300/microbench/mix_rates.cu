@@ -8,20 +8,24 @@
 // sweep, instead of derived from a random word), the random word converted from a 64-bit
 // integer, and tables holding two sites per 16-byte entry (one permute and one load per pair;
 // the pair index is taken from random bits here, its formation from the bit slices not counted).
+// Modes 6-8 are the forms the sweep kernels use: round keys from the kernel's parameters, bimodal
+// rejections as carries, packed differences with their signs collected by byte permutes.
 #include <cstdint>
 #include <cstdio>
 
 #include <cuda_runtime.h>
 
 #include "decide.cuh"
-#include "philox.cuh"
+#include "philox_parts.cuh"
 
 using namespace rfim;
 
 // MODE 0: Philox only, 1: + bimodal test, 2: + float-field test, 3: float test with the field in
-// registers, 4: the same with a 64-bit-source conversion, 5: the same with two-site table entries
+// registers, 4: the same with a 64-bit-source conversion, 5: the same with two-site table entries,
+// 6-8: modes 0, 1 and 3 in the sweep kernels' forms
 template <int MODE, int BAR>
-__global__ void __launch_bounds__(512, 1) k_mix(uint32_t seed, int iters, uint32_t *out, unsigned long long *cyc) {
+__global__ void __launch_bounds__(512, 1) k_mix(uint32_t seed, const __grid_constant__ PhiloxKeys keys, int iters,
+                                                uint32_t *out, unsigned long long *cyc) {
   __shared__ __align__(256) float2 tabf[64];
   __shared__ __align__(256) uint32_t tabu[128];
   __shared__ __align__(256) float4 tabp[256];  // two-site entries {b J n_a, b_a, b J n_b, b_b}
@@ -45,8 +49,29 @@ __global__ void __launch_bounds__(512, 1) k_mix(uint32_t seed, int iters, uint32
     for (int jb = 0; jb < 8; ++jb) {
 #pragma unroll
       for (int gg = 0; gg < 4; ++gg) {
-        const Words4 w = philox10(seed, 7u, tid * 8u + jb, (uint32_t)gg, (uint32_t)it, 0x20000000u);
-        if (MODE == 0) {
+        const Words4 w = MODE >= 6 ? philox_keyed(keys, tid * 8u + jb, (uint32_t)gg, (uint32_t)it, 0x20000000u)
+                                   : philox10(seed, 7u, tid * 8u + jb, (uint32_t)gg, (uint32_t)it, 0x20000000u);
+        if (MODE == 7) {
+          const uint32_t offs = (w.w[0] ^ (uint32_t)(it * 0x9E3779B9u + gg)) & 0x7C7C7C7Cu;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t t;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t) : "r"(__byte_perm(offs, slotu, 0x7650u | q)));
+            collect_reject(w.w[q], t, fk[q]);
+          }
+        } else if (MODE == 8) {
+          const uint32_t offs = (w.w[0] ^ (uint32_t)(it * 0x9E3779B9u + gg)) & 0x78787878u;
+          float2 e[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];"
+                         : "=f"(e[q].x), "=f"(e[q].y)
+                         : "r"(__byte_perm(offs, slotf, 0x7650u | q)));
+          const uint2 a = accept_float_signs(w.w[0], w.w[1], e[0], e[1], hh4[jb].x, hh4[jb].y);
+          const uint2 b = accept_float_signs(w.w[2], w.w[3], e[2], e[3], hh4[jb].z, hh4[jb].w);
+          acc[gg] |= prmt(a.x, a.y, 0x00FBu) & (0x00000101u << jb);
+          acc[gg] |= prmt(b.x, b.y, 0xFB00u) & (0x01010000u << jb);
+        } else if (MODE == 0 || MODE == 6) {
 #pragma unroll
           for (int q = 0; q < 4; ++q) acc[q] ^= w.w[q];
         } else if (MODE == 1) {
@@ -97,7 +122,7 @@ __global__ void __launch_bounds__(512, 1) k_mix(uint32_t seed, int iters, uint32
 template <int M, int B>
 double rate(int sms, uint32_t *out, unsigned long long *cyc, unsigned long long *h) {
   const int threads = 512, iters = 200;
-  for (int rep = 0; rep < 2; ++rep) k_mix<M, B><<<sms, threads>>>(1u, iters, out, cyc);
+  for (int rep = 0; rep < 2; ++rep) k_mix<M, B><<<sms, threads>>>(1u, philox_keys(1u, 7u), iters, out, cyc);
   if (cudaDeviceSynchronize() != cudaSuccess) return -1.0;
   cudaMemcpy(h, cyc, sms * sizeof(unsigned long long), cudaMemcpyDeviceToHost);
   unsigned long long mx = 0;
@@ -120,6 +145,9 @@ int main() {
   printf("attempts/clk/SM  float test, field in registers:       %.3f\n", rate<3, 0>(sms, out, cyc, h));
   printf("attempts/clk/SM  the same, 64-bit-source conversion:   %.3f\n", rate<4, 0>(sms, out, cyc, h));
   printf("attempts/clk/SM  the same, two-site table entries:     %.3f\n", rate<5, 0>(sms, out, cyc, h));
+  printf("attempts/clk/SM  Philox only, keys from the constant bank: %.3f\n", rate<6, 0>(sms, out, cyc, h));
+  printf("attempts/clk/SM  bimodal test, rejections as carries:  %.3f\n", rate<7, 0>(sms, out, cyc, h));
+  printf("attempts/clk/SM  float test, packed, signs by prmt:    %.3f\n", rate<8, 0>(sms, out, cyc, h));
   delete[] h;
   cudaFree(out);
   cudaFree(cyc);
