@@ -114,6 +114,7 @@ def load():
             L.rfim_exchange_noalloc.argtypes = [C.POINTER(ExchangeBuffers), u32, i64, P]
             L.rfim_selftest_grid.argtypes = [i32, i32, i32]
             L.rfim_selftest_wait.argtypes = [i32, i32]
+            L.rfim_selftest_resident.argtypes = [P, i32, i32, u32]
             L.rfim_debug_build.argtypes = []
             L.rfim_selftest_debug.argtypes = []
             L.rfim_set_measure_xi.argtypes = [P, i32]
@@ -134,7 +135,7 @@ def load():
                          "rfim_exchange_noalloc", "rfim_tune", "rfim_selftest_grid", "rfim_selftest_wait",
                          "rfim_set_measure_xi", "rfim_set_multihit", "rfim_thermal",
                          "rfim_disorder_average", "rfim_server_tune", "rfim_debug_build",
-                         "rfim_selftest_debug", "rfim_get_plan"):
+                         "rfim_selftest_debug", "rfim_get_plan", "rfim_selftest_resident"):
                 getattr(L, name).restype = C.c_int
             _lib = L
     return _lib
@@ -362,6 +363,11 @@ class Realization:
         out = np.zeros(self.N, dtype=np.float32)
         self._check(self._lib.rfim_get_field(self._h, _ptr(out)))
         return out
+
+    def selftest_resident(self, stop_cta=-1, stop_interval=0, number=0):
+        """The following resident launches give up a wait in CTA stop_cta (-1: none) at their interval
+        stop_interval; number > 0 numbers the exchange intervals on from there (rfim_selftest_resident)."""
+        self._check(self._lib.rfim_selftest_resident(self._h, stop_cta, stop_interval, number))
 
     def plan(self) -> str:
         """Launch shape of the sweep kernel ("S,G,GT,threads[,4][,int8]"; "" for the int8 kernels)."""

@@ -30,41 +30,15 @@ struct alignas(16) ChunkSum {
   long long F;
 };
 
-constexpr unsigned kMbarSpinLimit = 1u << 20;
-
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-
-// Bounded wait for the phase of parity `par` of an mbarrier of this CTA.
-__device__ __forceinline__ void mbar_wait(uint32_t mbar, uint32_t par, unsigned *err) {
-  for (unsigned it = 0; it < kMbarSpinLimit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(mbar), "r"(par)
-        : "memory");
-    if (done) return;
-    if ((it & 63u) == 63u && *(volatile unsigned *)err) return;
-  }
-  atomicOr(err, 2u);
-}
-
-// The same wait without the report and whatever has been reported: for pushes that are on their way
-// when a CTA ends after an expired wait.
-__device__ __forceinline__ void mbar_drain(uint32_t mbar, uint32_t par) {
-  for (unsigned it = 0; it < kMbarSpinLimit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(mbar), "r"(par)
-        : "memory");
-    if (done) return;
-  }
+// Self-test of waits that are given up: CTA `cta` of a launch acts as if it had given up a wait when it
+// starts interval `iv` of the launch (-1: no CTA does).
+struct SelftestStop {
+  int32_t cta, iv;
+};
+__device__ __forceinline__ bool stops_here(const SelftestStop &s, int iv, unsigned *err) {
+  if ((int)blockIdx.x != s.cta || iv != s.iv) return false;
+  if (threadIdx.x == 0) atomicOr(err, 2u);
+  return true;
 }
 
 constexpr unsigned kRecordSpinLimit = 1u << 22;
@@ -144,10 +118,12 @@ __device__ __forceinline__ void measure_red(double *acc, double E, long long M, 
 // the launch on its own copy xs of the temperature assignment: energies E = energy_of(bonds, field
 // sum), the swap decisions of the disjoint pairs (Eq. 2, Sec. 3.3), and, for the temperatures
 // k = CTA mod number of CTAs, the pair counts and the measurement (Sec. 7).  All threads of the CTA
-// call it; the assignment is complete when it returns.
+// call it; the assignment is complete when it returns.  False, and nothing is exchanged, when a thread of the
+// CTA has given up a wait: for a record here, or before with *gave_up set (in shared memory).
 template <bool REAL, bool POW2 = !REAL, class F>
-__device__ __forceinline__ void exchange_from_records(const RealView &v, const ExchArgs &xa, const ResidentState &xs,
-                                                      const uint4 *rec, int S, uint32_t epoch, uint32_t j, F energy_of) {
+__device__ __forceinline__ bool exchange_from_records(const RealView &v, const ExchArgs &xa, const ResidentState &xs,
+                                                      const uint4 *rec, int S, uint32_t epoch, uint32_t j,
+                                                      volatile uint32_t *gave_up, F energy_of) {
   const int nt = blockDim.x, tid = threadIdx.x, R = v.R;
   const int p0 = (int)(j & 1u) + 2 * tid;  // this thread's first pair
   auto random_of = [&](int k) {
@@ -167,7 +143,7 @@ __device__ __forceinline__ void exchange_from_records(const RealView &v, const E
       for (int q = 0; q < S; ++q) {
         int b, m;
         long long f;
-        record_await(rec + (size_t)r * S + q, epoch, xa.err, &b, &m, &f);
+        if (!record_await(rec + (size_t)r * S + q, epoch, xa.err, &b, &m, &f)) *gave_up = 1u;
         B += b;
         M += m;
         F = REAL && q > 0 ? __double_as_longlong(__dadd_rn(__longlong_as_double(F), __longlong_as_double(f))) : F + f;
@@ -180,7 +156,7 @@ __device__ __forceinline__ void exchange_from_records(const RealView &v, const E
       const int n = n0 + (tid & 31), r = n / S;
       int B = 0, M = 0;
       long long F = 0;
-      if (n < R * S) record_await(rec + n, epoch, xa.err, &B, &M, &F);
+      if (n < R * S && !record_await(rec + n, epoch, xa.err, &B, &M, &F)) *gave_up = 1u;
       __syncwarp();
       for (int o = S / 2; o > 0; o >>= 1) {
         B += __shfl_xor_sync(0xffffffffu, B, o);
@@ -195,6 +171,7 @@ __device__ __forceinline__ void exchange_from_records(const RealView &v, const E
     }
   }
   __syncthreads();
+  if (*gave_up) return false;
   for (int k = p0; k + 1 < R; k += 2 * nt) {
     const int a = xs.t2r[k], b = xs.t2r[k + 1];
     const uint32_t u = k == p0 ? u0 : random_of(k);
@@ -218,6 +195,7 @@ __device__ __forceinline__ void exchange_from_records(const RealView &v, const E
     if (measure) measure_red<POW2>(v.obs + (int64_t)k * 5, xs.E[a], xs.M[a], (double)v.N);
     if (k == 0 && measure) atomicAdd(reinterpret_cast<unsigned long long *>(v.n_meas), 1ull);
   }
+  return true;
 }
 
 }  // namespace rfim

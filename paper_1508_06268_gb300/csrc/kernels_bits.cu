@@ -605,6 +605,7 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
     ra.epoch0 = plan.epoch + 1;
     ra.rec = plan.rec;
     ra.i8 = plan.i8;
+    ra.stop = plan.stop;
     if (xi && exchange) {
       if (!plan.measures_xi(ra.mh) || n_intervals > xi->intervals) return cudaErrorInvalidValue;
       ra.xi_marg = xi->marg;

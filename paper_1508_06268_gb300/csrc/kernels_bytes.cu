@@ -150,6 +150,7 @@ cudaError_t launch_resident_bytes(const RealView &v, const ResidentShape &s, con
   ba.n_iv = ra.n_iv;
   ba.epoch0 = ra.epoch0;
   ba.rec = ra.rec;
+  ba.stop = ra.stop;
   ba.stride = plane_stride(v.L);
   ba.planes = slab_planes(v.L, s.S);
   const int clusters = (v.R + s.G - 1) / s.G;

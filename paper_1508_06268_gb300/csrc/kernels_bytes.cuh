@@ -16,6 +16,7 @@
 
 #include "decide_bytes.cuh"
 #include "exchange_records.cuh"
+#include "halos.cuh"
 #include "philox_parts.cuh"
 
 namespace rfim {
@@ -26,6 +27,7 @@ struct BytesArgs {
   uint32_t epoch0;           // interval number of the first
   uint4 *rec;                // [2][rcap * S] energy records
   int32_t stride, planes;    // padded plane (bytes), planes of the largest slab
+  SelftestStop stop;
 };
 
 // floor(n / d) for n d < 2^32 and d >= 2 with m = recip(d).
@@ -55,7 +57,8 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
   using Word = typename BytesWord<VW>::type;
   using Copy = typename BytesWord<VW>::copy;
   extern __shared__ __align__(16) uint32_t sm[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) HaloBars hb;
+  __shared__ volatile GaveUp gave_up;
   __shared__ ChunkSum part[16];
   const int L = v.L, Lh = v.Lh, plane = L * Lh, S = ba.S, PS = ba.stride, R = v.R;
   const int64_t half = (int64_t)plane * L;
@@ -101,14 +104,9 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
       xs.r2t[r] = v.r2t[r];
       xs.beta[r] = v.beta_d[r];
     }
-  const uint32_t mbar0 = (uint32_t)__cvta_generic_to_shared(mbar);
+  if (tid == 0) gave_up.sweep[0] = gave_up.sweep[1] = gave_up.exchange = 0u;
   if (S > 1) {
-    if (tid == 0) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;" ::"r"(mbar0),
-                   "r"(mbar0 + 8)
-                   : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (tid == 0) halo_init(&hb);
     sync_slabs<2>();
   } else {
     __syncthreads();
@@ -178,26 +176,29 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
   auto field_of = [&](int c, int b) {
     return BIM ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(reinterpret_cast<const float4 *>(v.hh_c + c * half) + b);
   };
-  // after half-sweep number h: the slab's end planes into the neighbours' halo planes (see
-  // kernels_resident.cuh for the order of the two mbarriers)
+  // after half-sweep number h: the slab's end planes into the neighbours' halo planes (halos.cuh)
+  const uint32_t push_bytes = (uint32_t)(gact * PS);  // to each neighbour
+  uint32_t pushed = 0;  // (thread 0) pushes made
+  bool stopped = !ok;   // (threads that push) no more pushes
   auto push_halos = [&](int c, uint32_t h) {
-    const uint32_t bar = mbar0 + 8 * (h & 1u);
     const int vec = PS / 16;
-    if (tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)(gact * 2 * PS)) : "memory");
+    if (tid >= gact * 2 * vec) return;
+    stopped |= gave_up.sweep[c] != 0u;
+    if (stopped) return;
+    pushed = h + 1;
+    if (tid == 0) halo_expect(&hb, h, 2 * push_bytes);
     for (int t = tid; t < gact * 2 * vec; t += nt) {
       const int q = t % vec, side = t / vec & 1, g = t / (2 * vec);
       const uint32_t peer = (uint32_t)(rank + (side ? 1 : S - 1)) % S;
       const int peer_planes = ((int)peer + 1) * L / S - (int)peer * L / S;
       const size_t base = (size_t)(2 * g + c) * CS + 16 * q;
-      const uint4 x = *reinterpret_cast<const uint4 *>(lat + base + (size_t)(side ? PZ : 1) * PS);
-      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
-                       mapa_shared((uint32_t)__cvta_generic_to_shared(lat + base + (size_t)(side ? 0 : peer_planes + 1) * PS), peer)),
-                   "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(mapa_shared(bar, peer))
-                   : "memory");
+      halo_store(&hb, h, lat + base + (size_t)(side ? 0 : peer_planes + 1) * PS, peer,
+                 *reinterpret_cast<const uint4 *>(lat + base + (size_t)(side ? PZ : 1) * PS));
     }
   };
-  auto wait_halos = [&](uint32_t h) { mbar_wait(mbar0 + 8 * (h & 1u), (h >> 1) & 1u, xa.err); };
+  auto wait_halos = [&](uint32_t h, int c) {
+    if (!halo_wait(&hb, h, xa.err)) gave_up.sweep[c] = 1u;
+  };
 
   auto update = [&](int g, int c, const RowWord (&rw)[NR], const Words4 &w, const float4 &h4, uint32_t hb, bool valid) {
     uint8_t *lat_g = lat + (size_t)(2 * g) * CS;
@@ -232,8 +233,12 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
   const int n_iv = xa.enabled ? ba.n_iv : 1;
   uint32_t h = 0, sweep = sweep0;
   for (int iv = 0; iv < n_iv; ++iv) {
+    if (!ok || stops_here(ba.stop, iv, xa.err)) {
+      gave_up.exchange = 1u;
+      break;
+    }
 #pragma unroll 1
-    for (int s = 0; s < nsw; ++s, ++sweep) {
+    for (int s = 0; s < nsw && (S == 1 || !gave_up.sweep[1]); ++s, ++sweep) {
       if (ONE) {
 #pragma unroll
         for (int c = 0; c < 2; ++c, ++h) {
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
             __syncthreads();
           } else {  // this half-sweep's words while the halos are on their way
             philox_words<1>(ba.keys, bp, c, (uint32_t)(r0 + own_g), sweep, w);
-            if (h > 0) wait_halos(h - 1);
+            if (h > 0) wait_halos(h - 1, c);
             update(own_g, c, own, w[0], hown[c], hbown[c], valid);
             __syncthreads();
             push_halos(c, h);
@@ -259,19 +264,19 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
           for (int item = tid; item < items; item += nt) {
             const int g = quot(item, m_blk), b = b0 + item - g * nblk;
             const float4 h4 = field_of(c, b);
-            const uint32_t hb = field_bytes(c, b);
+            const uint32_t hbits = field_bytes(c, b);
             RowWord rw[NR];
             locate(b, c, rw);
             const Words4 wi = philox_keyed(ba.keys, (uint32_t)b, (uint32_t)(r0 + g), sweep, tag);
-            if (S > 1 && item == tid && h > 0) wait_halos(h - 1);
-            update(g, c, rw, wi, h4, hb, true);
+            if (S > 1 && item == tid && h > 0) wait_halos(h - 1, c);
+            update(g, c, rw, wi, h4, hbits, true);
           }
           __syncthreads();
           if (S > 1) push_halos(c, h);
         }
       }
     }
-    if (S > 1 && h > 0) wait_halos(h - 1);
+    if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) gave_up.exchange = 1u;
     if (!xa.enabled) break;
 
     // ---- energies (Eq. 1): small replicas by one warp each, others by the whole CTA ---------------
@@ -340,17 +345,15 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     auto energy_of = [&](int B, long long F) {
       return -xa.J * (double)B - (BIM ? xa.h * (double)F : __longlong_as_double(F));
     };
-    if (ok) exchange_from_records<!BIM, false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, energy_of);
-    if (ok && iv + 1 < n_iv) tab_fill_temps<BIM, false>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
+    if (!exchange_from_records<!BIM, false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, &gave_up.exchange, energy_of)) break;
+    if (iv + 1 < n_iv) tab_fill_temps<BIM, false>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
-  if (S > 1) {  // a CTA stays until its neighbours' pushes have landed, also those whose wait expired
-    if (*(volatile unsigned *)xa.err & 2u)
-      for (uint32_t q = h > 2 ? h - 2 : 0; q < h; ++q) mbar_drain(mbar0 + 8 * (q & 1u), (q >> 1) & 1u);
-    sync_slabs<2>();
-  }
+  __syncthreads();
+  const bool gone = gave_up.exchange != 0u;  // this launch's results are not to be had
+  if (S > 1) halo_leave(&hb, rank, S, pushed, gone, push_bytes);
   copy_planes(1, PZ, false);
-  if (xa.enabled && ok && blockIdx.x == 0)
+  if (xa.enabled && !gone && blockIdx.x == 0)
     for (int r = tid; r < R; r += nt) {
       v.t2r[r] = xs.t2r[r];
       v.r2t[r] = xs.r2t[r];

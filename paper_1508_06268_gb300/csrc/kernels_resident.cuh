@@ -33,6 +33,7 @@
 #include <cstdint>
 
 #include "exchange_records.cuh"
+#include "halos.cuh"
 #include "kernels_bits.cuh"
 #include "philox_parts.cuh"
 
@@ -48,6 +49,7 @@ struct ResidentArgs {
   int32_t i8;       // the realization is stored as bytes (v.spins8) and staged as bits
   int32_t lw;       // log2 of the words whose items of one part are neighbouring threads (ONE; else 5)
   int32_t mh;       // passes per tile visit (T > 0)
+  SelftestStop stop;
   // structure factor (XI): of every measuring interval iv, the marginals S_d[t] of every
   // replica, [iv][R][3][L], zero when the launch starts, and the replica at every temperature, [iv][R]
   int32_t *xi_marg, *xi_t2r;
@@ -154,7 +156,8 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   static_assert(T == 0 || (T % 8 == 0 && L % (2 * T) == 0 && NB <= 4 && (NB >= T / 8 || T / 8 % NB == 0)),
                 "an item's blocks lie in tiles of one x parity");
   extern __shared__ __align__(16) uint32_t sm[];
-  __shared__ __align__(8) uint64_t mbar[2];  // halos pushed after even / odd half-sweeps
+  __shared__ __align__(8) HaloBars hb;
+  __shared__ volatile GaveUp gave_up;
   const int rank = S > 1 ? (int)cluster_rank() : 0;
   const int z0 = rank * PZ, r0 = (int)(blockIdx.x / S) * ra.G, gact = min(ra.G, v.R - r0);
   const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
@@ -197,14 +200,9 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   const bool limbs = !BIM && xa.flimb != nullptr;
   const double fscale = limbs ? ldexp(1.0, xa.fquant->qe) : 1.0;
   const long long Htot = limbs ? xa.fquant->Htot : 0;
-  const uint32_t mbar0 = (uint32_t)__cvta_generic_to_shared(mbar);
+  if (tid == 0) gave_up.sweep[0] = gave_up.sweep[1] = gave_up.exchange = 0u;
   if (S > 1) {
-    if (tid == 0) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;" ::"r"(mbar0),
-                   "r"(mbar0 + 8)
-                   : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (tid == 0) halo_init(&hb);
     sync_slabs<S>();  // every CTA's mbarriers are ready before the first push
   } else {
     __syncthreads();
@@ -261,28 +259,29 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     if (valid) atomicXor(self, flip << sh);
   };
   // After half-sweep number h of this launch (all of the CTA's updates of colour c done): the slab's
-  // first and last planes into the halo planes of the slabs below and above.  Two mbarriers in turn:
-  // a neighbour can push half-sweep h + 2 only after it has this slab's push of h + 1, which
-  // follows this slab's wait for h.  (WHOLE_TILES: both colours after tile visit number h.)
-  auto push_halos = [&](int colour, uint32_t h) {
-    constexpr int NC = WHOLE_TILES ? 2 : 1;
-    const uint32_t bar = mbar0 + 8 * (h & 1u);
+  // first and last planes into the halo planes of the slabs below and above (halos.cuh).
+  // WHOLE_TILES: both colours after tile visit number h.
+  constexpr int NC = WHOLE_TILES ? 2 : 1;
+  const uint32_t push_bytes = (uint32_t)(gact * NC * P * 4);  // to each neighbour
+  uint32_t pushed = 0;  // (thread 0) pushes made
+  bool stopped = !ok;   // (threads that push) no more pushes
+  auto push_halos = [&](int colour, int flag, uint32_t h) {
     constexpr int VEC = P >= 4 ? P / 4 : 1;
-    if (tid == 0)
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)(gact * 2 * NC * P * 4))
-                   : "memory");
+    if (tid >= gact * 2 * NC * VEC) return;
+    stopped |= gave_up.sweep[flag] != 0u;
+    if (stopped) return;
+    pushed = h + 1;
+    if (tid == 0) halo_expect(&hb, h, 2 * push_bytes);
     for (int t = tid; t < gact * 2 * NC * VEC; t += nt) {
       const int g = t / (2 * NC * VEC), c = NC == 2 ? t / (2 * VEC) & 1 : colour, side = t / VEC & 1, q = t % VEC * 4;
       const uint32_t peer = (uint32_t)(rank + (side ? 1 : S - 1)) % S;
       const int from = (g * 2 + c) * CW + (side ? PZ : 1) * P + q, to = (g * 2 + c) * CW + (side ? 0 : PZ + 1) * P + q;
-      const uint4 x = *reinterpret_cast<const uint4 *>(sp + from);
-      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
-                       mapa_shared((uint32_t)__cvta_generic_to_shared(sp + to), peer)),
-                   "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(mapa_shared(bar, peer))
-                   : "memory");
+      halo_store(&hb, h, sp + to, peer, *reinterpret_cast<const uint4 *>(sp + from));
     }
   };
-  auto wait_halos = [&](uint32_t h) { mbar_wait(mbar0 + 8 * (h & 1u), (h >> 1) & 1u, xa.err); };
+  auto wait_halos = [&](uint32_t h, int flag) {
+    if (!halo_wait(&hb, h, xa.err)) gave_up.sweep[flag] = 1u;
+  };
 
   bool valid;
   const ResidentItem<NB> own = decode(tid, ONE ? ra.lw : 5, &valid);
@@ -307,8 +306,12 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   const int n_iv = xa.enabled ? ra.n_iv : 1;
   uint32_t h = 0, sweep = sweep0;  // half-sweeps done in this launch; current sweep
   for (int iv = 0; iv < n_iv; ++iv) {
+    if (!ok || stops_here(ra.stop, iv, xa.err)) {
+      gave_up.exchange = 1u;
+      break;
+    }
 #pragma unroll 1
-    for (int s = 0; s < nsw; ++s, ++sweep) {
+    for (int s = 0; s < nsw && (S == 1 || !gave_up.sweep[1]); ++s, ++sweep) {
       if constexpr (T > 0) {
 #pragma unroll
         for (int coarse = 0; coarse < 2; ++coarse) {
@@ -324,7 +327,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
                 const int sh = first_block(own, coarse);
                 if (NB > 2) field_of(own, sh, c, hown[coarse][c]);
                 philox_words<NB>(ra.keys, bp[coarse], c, (uint32_t)(r0 + own.g), ctr, w);
-                if (wait) wait_halos(h - 1);
+                if (wait) wait_halos(h - 1, WHOLE_TILES ? coarse : c);
                 update(own, sh, c, w, hown[coarse][c], fbown[c], valid);
               } else {
 #pragma unroll 1
@@ -337,13 +340,13 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
                   const uint32_t fb = field_bits(it, c);
                   bp[0] = parts_of(it, coarse);
                   philox_words<NB>(ra.keys, bp[0], c, (uint32_t)(r0 + it.g), ctr, w);
-                  if (wait && item == tid) wait_halos(h - 1);
+                  if (wait && item == tid) wait_halos(h - 1, WHOLE_TILES ? coarse : c);
                   update(it, sh, c, w, hf, fb, in);
                 }
               }
               __syncthreads();
               if (push) {
-                push_halos(c, h);
+                push_halos(c, WHOLE_TILES ? coarse : c, h);
                 ++h;
               }
             }
@@ -364,10 +367,10 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
         } else if (ONE) {
           if (NB > 2) field_of(own, own.sh, c, hown[0][c]);
           philox_words<NB>(ra.keys, bp[0], c, (uint32_t)(r0 + own.g), sweep, w);
-          if (h > 0) wait_halos(h - 1);
+          if (h > 0) wait_halos(h - 1, c);
           update(own, own.sh, c, w, hown[0][c], fbown[c], valid);
           __syncthreads();
-          push_halos(c, h);
+          push_halos(c, c, h);
         } else {
           for (int item = tid; item < (words + 31) / 32 * 32 * NP; item += nt) {
             bool in;
@@ -377,16 +380,16 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
             const uint32_t fb = field_bits(it, c);
             bp[0] = parts_of(it, 0);
             philox_words<NB>(ra.keys, bp[0], c, (uint32_t)(r0 + it.g), sweep, w);
-            if (S > 1 && item == tid && h > 0) wait_halos(h - 1);
+            if (S > 1 && item == tid && h > 0) wait_halos(h - 1, c);
             update(it, it.sh, c, w, hf, fb, in);
           }
           __syncthreads();
-          if (S > 1) push_halos(c, h);
+          if (S > 1) push_halos(c, c, h);
         }
         ++h;
       }
     }
-    if (S > 1 && h > 0) wait_halos(h - 1);
+    if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) gave_up.exchange = 1u;
     if (!xa.enabled) break;
     const bool xi = XI && (int64_t)(xa.j + (uint32_t)iv) >= xa.measure_from;
     if (xi)
@@ -488,17 +491,15 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
       const double Fd = BIM ? xa.h * (double)F : (double)(2 * F - Htot) * fscale;
       return -xa.J * (double)B - Fd;
     };
-    if (ok) exchange_from_records<false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, energy_of);
-    if (xi && ok && blockIdx.x == 0)
+    if (!exchange_from_records<false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, &gave_up.exchange, energy_of)) break;
+    if (xi && blockIdx.x == 0)
       for (int k = tid; k < R; k += nt) ra.xi_t2r[(int64_t)iv * R + k] = xs.t2r[k];
-    if (ok && iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
+    if (iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
-  if (S > 1) {  // a CTA stays until its neighbours' pushes have landed, also those whose wait expired
-    if (*(volatile unsigned *)xa.err & 2u)
-      for (uint32_t q = h > 2 ? h - 2 : 0; q < h; ++q) mbar_drain(mbar0 + 8 * (q & 1u), (q >> 1) & 1u);
-    sync_slabs<S>();
-  }
+  __syncthreads();
+  const bool gone = gave_up.exchange != 0u;  // this launch's results are not to be had
+  if (S > 1) halo_leave(&hb, rank, S, pushed, gone, push_bytes);
 
   for (int t = tid; ok && t < gact * 2 * WC; t += nt) {
     const int g = t / (2 * WC), rem = t % (2 * WC), c = rem / WC, wl = rem % WC;
@@ -509,7 +510,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     else
       v.bits[gw] = word;
   }
-  if (xa.enabled && ok && blockIdx.x == 0)
+  if (xa.enabled && !gone && blockIdx.x == 0)
     for (int r = tid; r < R; r += nt) {
       v.t2r[r] = xs.t2r[r];
       v.r2t[r] = xs.r2t[r];

@@ -788,6 +788,17 @@ int rfim_get_plan(const rfim_ctx *ctx, char *plan_out, int32_t plan_cap) {
   return RFIM_OK;
 }
 
+int rfim_selftest_resident(rfim_ctx *ctx, int32_t stop_cta, int32_t stop_interval, uint32_t number) {
+  if (!ctx) return RFIM_EINVAL;
+  BitsPlan &p = ctx->plan;
+  if (stop_cta < -1 || stop_interval < 0 || number >= kRecordEpochs - 1 || (number > 0 && number <= p.epoch))
+    return fail(ctx, RFIM_EINVAL, "invalid self-test arguments");
+  if (!p.resident() && p.mh_res.threads == 0) return fail(ctx, RFIM_ESTATE, "not a resident plan");
+  p.stop = SelftestStop{stop_cta, stop_interval};
+  if (number > 0) p.epoch = number - 1;
+  return RFIM_OK;
+}
+
 int rfim_tune(int32_t L, int32_t R, int32_t field_kind, char *plan_out, int32_t plan_cap, double *attempts_per_ns) {
   if (!bits_supported(L) || R < 2 || field_kind < 0 || field_kind > 2)
     return fail(nullptr, RFIM_EINVAL, "rfim_tune: L in {8,16,32,64}, R >= 2, known field kind");

@@ -47,6 +47,7 @@ struct BitsPlan {
   uint4 *rec = nullptr;
   size_t rec_slots = 0;  // records of one interval the array holds (two intervals)
   mutable uint32_t epoch = 0;
+  SelftestStop stop{-1, 0};  // self-test: where the resident launches give up a wait
   ResidentShape mh_res;  // resident shape of the multi-hit sweeps in force (threads > 0 when they have one)
   bool resident() const { return res.threads > 0; }
   bool xi = false;  // plain resident launches can measure the structure factor (XiWork)

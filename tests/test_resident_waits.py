@@ -1,0 +1,61 @@
+"""Bounded waits inside the resident launches: one that is given up ends the launch in order (no CTA pushes
+or arrives again, none leaves while a push to it is on its way), the error is reported once, and
+the realization goes on from a state that is set."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1508_06268_gb300 as rf
+from paper_1508_06268_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+SLABS = [  # L, R, "S,G,NB,threads,r" (m: several items per thread, b: bytes), tile (0: plain checkerboard)
+    (8, 7, "1,3,1,256,r", 0), (10, 3, "1,1,4,128,b", 0), (16, 5, "1,3,2,384,r", 8),
+    (16, 5, "2,2,2,256,r", 0), (32, 3, "8,1,2,256,r", 0), (32, 2, "4,1,4,256,r", 0), (32, 5, "2,3,4,512,m", 0),
+    (64, 2, "16,1,4,512,r", 0), (64, 3, "8,2,4,512,m", 0), (14, 5, "5,2,4,256,b", 0), (24, 5, "4,2,4,512,b", 0),
+    (28, 2, "8,1,4,448,b", 0), (32, 3, "4,2,2,512,r", 8), (32, 3, "2,2,4,512,r", 16), (64, 4, "8,1,4,512,r", 8),
+    (64, 5, "4,2,4,512,m", 32), (64, 4, "16,1,2,512,r", 16),
+]
+
+
+def pair(monkeypatch, L, R, plan, tile):
+    kw = dict(h=1.5, field_kind=rf.FIELD_BIMODAL, field_seed=3, seed=42)
+    temps = inputs.geometric_temps(1.0, 5.0, R)
+    monkeypatch.setenv("RFIM_BITS_PLAN", plan)
+    g = rf.Realization(L, temps, layout=rf.LAYOUT_INT8 if plan[-1] == "b" else rf.LAYOUT_BITPACK, **kw)
+    o = oracle.Oracle(L, temps, **kw)
+    if tile:
+        g.set_multihit(2, tile)
+        o.set_multihit(2, tile)
+    monkeypatch.delenv("RFIM_BITS_PLAN")
+    assert g.plan() == plan
+    return g, o
+
+
+@pytest.mark.parametrize("L,R,plan,tile", SLABS)
+def test_given_up_wait_ends_in_order(L, R, plan, tile, monkeypatch):
+    """One CTA gives up a wait: at once, in a later interval, and in launches that are queued behind the failed
+    one.  Its neighbours in the cluster, at every distance, and the other clusters stop too."""
+    g, o = pair(monkeypatch, L, R, plan, tile)
+    S, G = int(plan.split(",")[0]), int(plan.split(",")[1])
+    ctas = (R + G - 1) // G * S
+    g.run(4, 2, 0)
+    o.run(4, 2, 0)
+    good = g.get_state()
+    np.testing.assert_array_equal(good["spins"], o.spins())
+    for cta, interval in ((0, 0), (ctas - 1, 1), (S // 2, 2)):
+        g.selftest_resident(cta, interval)
+        g.run(12, 2, 0)
+        g.sweep(3)
+        g.exchange(0)
+        with pytest.raises(rf.RfimError) as e:
+            g.get_state()
+        assert e.value.code == rf.ETIMEOUT
+        g.selftest_resident()
+        g.set_state(good["spins"], good["t2r"], good["sweep"], good["xstep"])
+    g.run(6, 2, 0)
+    o.run(6, 2, 0)
+    st = g.get_state()
+    np.testing.assert_array_equal(st["spins"], o.spins())
+    np.testing.assert_array_equal(st["t2r"], o.perm()[0])
