@@ -610,6 +610,7 @@ cudaError_t launch_sweeps_bits(const RealView &v, const BitsPlan &plan, uint32_t
       if (!plan.measures_xi(ra.mh) || n_intervals > xi->intervals) return cudaErrorInvalidValue;
       ra.xi_marg = xi->marg;
       ra.xi_t2r = xi->t2r;
+      ra.xi_first = xi->first;
       const cudaError_t e = cudaMemsetAsync(xi->marg, 0, (size_t)n_intervals * v.R * 3 * v.L * sizeof(int32_t), st);
       if (e != cudaSuccess) return e;
     }

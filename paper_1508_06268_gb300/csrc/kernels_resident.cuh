@@ -50,9 +50,10 @@ struct ResidentArgs {
   int32_t lw;       // log2 of the words whose items of one part are neighbouring threads (ONE; else 5)
   int32_t mh;       // passes per tile visit (T > 0)
   SelftestStop stop;
-  // structure factor (XI): of every measuring interval iv, the marginals S_d[t] of every
+  // structure factor (XI): of every interval iv >= xi_first, the marginals S_d[t] of every
   // replica, [iv][R][3][L], zero when the launch starts, and the replica at every temperature, [iv][R]
   int32_t *xi_marg, *xi_t2r;
+  int32_t xi_first;
 };
 
 // Planes of a slab in shared memory: with S > 1 a halo plane before and after the slab's own.
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     }
     if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) gave_up.exchange = 1u;
     if (!xa.enabled) break;
-    const bool xi = XI && (int64_t)(xa.j + (uint32_t)iv) >= xa.measure_from;
+    const bool xi = XI && iv >= ra.xi_first;
     if (xi)
       for (int t = tid; t < gact * 3 * L; t += nt) marg[t] = 0;
 

@@ -258,6 +258,7 @@ int do_sweeps_exchange_bits(rfim_ctx *c, int64_t n, int64_t measure_from, int32_
   cudaEvent_t stop;
   const int64_t j0 = c->xstep;
   const bool xi = c->xi_on && j0 + k - 1 >= measure_from && c->xi.intervals > 0 && c->plan.measures_xi(c->mh.mh);
+  c->xi.first = measure_from > j0 ? (int32_t)std::min<int64_t>(measure_from - j0, k) : 0;
   CUDA_OR_FAIL(c, prof_begin(c, 0, &stop, k));
   CUDA_OR_FAIL(c, launch_sweeps_bits(v, c->plan, (uint32_t)c->sweep, (int32_t)n, true, (uint32_t)j0, measure_from,
                                      (double)c->J, (double)c->h, c->stream, &c->mh, k, xi ? &c->xi : nullptr));
@@ -266,8 +267,7 @@ int do_sweeps_exchange_bits(rfim_ctx *c, int64_t n, int64_t measure_from, int32_
   c->sweep += n * k;
   c->xstep += k;
   if (!xi) return measure_xi_after(c, c->xstep - 1, measure_from);
-  const int32_t first = (int32_t)std::max<int64_t>(0, measure_from - j0);
-  CUDA_OR_FAIL(c, launch_xi_sums(v, c->xi.marg, c->xi.t2r, first, k, c->kcos, c->ksin, c->sumF, c->stream));
+  CUDA_OR_FAIL(c, launch_xi_sums(v, c->xi.marg, c->xi.t2r, c->xi.first, k, c->kcos, c->ksin, c->sumF, c->stream));
   c->launches += 1;
   return RFIM_OK;
 }

@@ -67,10 +67,11 @@ struct MultiHit {
 };
 
 // Workspace of the structure factor measured inside resident launches: marginals and the replica at
-// every temperature of up to `intervals` exchange intervals (0: not allocated).
+// every temperature of up to `intervals` exchange intervals (0: not allocated).  A launch fills in its
+// intervals `first` and later; which those are is decided once, on the host (its step numbers have 64 bits).
 struct XiWork {
   int32_t *marg = nullptr, *t2r = nullptr;
-  int32_t intervals = 0;
+  int32_t intervals = 0, first = 0;
 };
 // Whether tiles of edge `tile` are supported at L; the setting for (L, mh, tile).
 bool multihit_tile_ok(int32_t L, int32_t tile);
