@@ -14,6 +14,13 @@ namespace rfim {
 // Exchange intervals one launch takes at most (the host regains control between launches).
 constexpr int64_t kResidentIntervals = 512;
 
+// Most sweeps (multi-hit: passes) of an interval that ends with the exchange step in the same launch.  The
+// clusters run an interval independently and then wait for each other's energies, at most kRecordSpinLimit polls
+// (3.4 s measured, 1.2 s at the least): a cluster of one replica beside one of twenty at L = 64 waits 0.18 ms
+// per sweep.  Longer intervals are swept by a launch in which no cluster waits for another, and the exchange
+// step takes a launch of its own, some 5 us more after 0.3 ms or longer.
+constexpr int64_t kResidentSweeps = 2048;
+
 struct ResidentShape {
   // slabs, replicas per cluster, Philox blocks per item (0: the kernel on bytes), threads per CTA
   int32_t S = 0, G = 0, NB = 0, threads = 0;

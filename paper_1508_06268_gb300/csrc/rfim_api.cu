@@ -303,14 +303,15 @@ int do_run(rfim_ctx *c, int64_t n_sweeps, int32_t ex, int64_t measure_from) {
                          : c->plan.measures_xi(c->mh.mh)
                              ? std::min<int64_t>(c->plan.max_intervals(c->mh.mh), c->xi.intervals)
                              : 1;
-    if (ends_interval && chunk == ex && left >= 2 * (int64_t)ex && most > 1) {
+    const bool apart = c->plan.sweeps_apart(chunk, c->mh.mh);
+    if (ends_interval && !apart && chunk == ex && left >= 2 * (int64_t)ex && most > 1) {
       const int64_t k = std::min(left / ex, most);
       rc = do_sweeps_exchange_bits(c, ex, measure_from, (int32_t)k);
       if (rc) return rc;
       left -= k * ex;
       continue;
     }
-    if (ends_interval && c->plan.counter) {
+    if (ends_interval && !apart && c->plan.counter) {
       rc = do_sweeps_exchange_bits(c, chunk, measure_from);
       if (rc) return rc;
       left -= chunk;

@@ -52,6 +52,10 @@ struct BitsPlan {
   bool resident() const { return res.threads > 0; }
   bool xi = false;  // plain resident launches can measure the structure factor (XiWork)
   bool measures_xi(int32_t mh) const { return xi && mh == 0; }
+  // whether n sweeps and the exchange step after them are launches of their own
+  bool sweeps_apart(int64_t n, int32_t mh) const {
+    return (mh > 0 ? mh_res.threads > 0 : resident()) && n > kResidentSweeps / (mh > 1 ? mh : 1);
+  }
   // exchange intervals one launch takes at most (mh passes per visit; 0: plain sweeps)
   int64_t max_intervals(int32_t mh) const {
     if (mh > 0) return mh_res.threads > 0 && mh < kResidentIntervals ? kResidentIntervals / mh : 1;

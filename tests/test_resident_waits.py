@@ -59,3 +59,32 @@ def test_given_up_wait_ends_in_order(L, R, plan, tile, monkeypatch):
     st = g.get_state()
     np.testing.assert_array_equal(st["spins"], o.spins())
     np.testing.assert_array_equal(st["t2r"], o.perm()[0])
+
+
+def test_long_intervals_do_not_run_out_of_polls(monkeypatch):
+    """The last cluster holds one replica where the other holds twenty, so it waits for almost the whole
+    interval: 0.18 ms per sweep, 3.6 s in all."""
+    monkeypatch.setenv("RFIM_BITS_PLAN", "4,20,4,512,m")
+    g = rf.Realization(64, inputs.geometric_temps(1.0, 5.0, 21), field_kind=rf.FIELD_GAUSSIAN, seed=4)
+    assert g.plan() == "4,20,4,512,m"
+    g.run(20000, 20000, 0)
+    st = g.get_state()
+    assert st["sweep"] == 20000 and st["xstep"] == 1
+    assert g.observables()["n_meas"] == 1
+
+
+@pytest.mark.parametrize("mh,tile,every", [(0, 0, 2049), (700, 8, 3)])
+def test_intervals_swept_apart_match_oracle(mh, tile, every, monkeypatch):
+    """Above 2048 sweeps (multi-hit: passes) per interval the sweeps are a launch of their own."""
+    g, o = pair(monkeypatch, 16, 3, "1,1,1,512,r", 0)
+    if mh:
+        g.set_multihit(mh, tile)
+        o.set_multihit(mh, tile)
+    n0 = g.launch_count
+    g.run(2 * every, every, 0)
+    assert g.launch_count - n0 == 4
+    o.run(2 * every, every, 0)
+    st = g.get_state()
+    np.testing.assert_array_equal(st["spins"], o.spins())
+    np.testing.assert_array_equal(st["t2r"], o.perm()[0])
+    np.testing.assert_array_equal(g.observables()["sums"], o.observables())
