@@ -347,6 +347,11 @@ int rfim_selftest_bits(int32_t L, uint32_t seed);
    the number of violations (0 = pass) or -1 for invalid arguments. */
 int rfim_selftest_grid(int32_t L, int32_t R, int32_t P);
 
+/* Host-only self-check of the divisions by reciprocals in the resident kernel on bytes (int8 layout): plane
+   and row of every Philox block of a colour.  Returns the number of wrong ones, plus 1 if an argument
+   leaves the range in which they are exact (0 = pass), or -1 for an L the kernel does not take. */
+int rfim_selftest_bytes(int32_t L);
+
 /* Device self-test of the bounded waits that the grid-wide kernel uses between CTAs (the paper
    has no counterpart: its CTAs never wait on one another).  One thread waits for a progress word
    that nothing sets (set_flag = 0) or that is already set (set_flag = 1), for at most spin_limit

@@ -114,6 +114,7 @@ def load():
             L.rfim_exchange_noalloc.argtypes = [C.POINTER(ExchangeBuffers), u32, i64, P]
             L.rfim_selftest_grid.argtypes = [i32, i32, i32]
             L.rfim_selftest_wait.argtypes = [i32, i32]
+            L.rfim_selftest_bytes.argtypes = [i32]
             L.rfim_selftest_resident.argtypes = [P, i32, i32, u32]
             L.rfim_debug_build.argtypes = []
             L.rfim_selftest_debug.argtypes = []
@@ -135,7 +136,7 @@ def load():
                          "rfim_exchange_noalloc", "rfim_tune", "rfim_selftest_grid", "rfim_selftest_wait",
                          "rfim_set_measure_xi", "rfim_set_multihit", "rfim_thermal",
                          "rfim_disorder_average", "rfim_server_tune", "rfim_debug_build",
-                         "rfim_selftest_debug", "rfim_get_plan", "rfim_selftest_resident"):
+                         "rfim_selftest_debug", "rfim_get_plan", "rfim_selftest_resident", "rfim_selftest_bytes"):
                 getattr(L, name).restype = C.c_int
             _lib = L
     return _lib
@@ -201,6 +202,10 @@ def selftest_debug() -> int:
 
 def selftest_grid(L: int, R: int, P: int) -> int:
     return load().rfim_selftest_grid(L, R, P)
+
+
+def selftest_bytes(L: int) -> int:
+    return load().rfim_selftest_bytes(L)
 
 
 def selftest_bits(L: int, seed: int = 1) -> int:

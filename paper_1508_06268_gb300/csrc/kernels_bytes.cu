@@ -67,7 +67,7 @@ bool bytes_fits(int32_t L, int32_t R, bool bim, ResidentShape *s) {
 }  // namespace
 
 bool bytes_shape(int32_t L, int32_t R, bool bim, ResidentShape *out, double *cycles) {
-  if (L < 4 || L % 2 || bits_supported(L)) return false;
+  if (L < 4 || L % 2 || L > kBytesMaxL || bits_supported(L)) return false;
   ResidentShape s;
   s.NB = 0;
   const char *o = getenv("RFIM_BITS_PLAN");  // "S,G,4,threads,b" names a shape of this kernel
@@ -159,3 +159,15 @@ cudaError_t launch_resident_bytes(const RealView &v, const ResidentShape &s, con
 }
 
 }  // namespace rfim
+
+// Number of (block, or site of a plane) quotients of the kernel's arithmetic that are wrong or outside its bound.
+extern "C" int rfim_selftest_bytes(int32_t L) {
+  using namespace rfim;
+  if (L < 4 || L % 2 || L > kBytesMaxL) return -1;  // RFIM_EINVAL
+  const int plane = L * L / 2, Lh = L / 2, blocks = plane * L / 4;
+  const uint32_t m_plane = recip((uint32_t)plane / 2), m_row = recip((uint32_t)Lh);
+  int bad = (uint64_t)(2 * blocks) * (plane / 2) >= 1ull << 32;
+  for (int b = 0; b < blocks; ++b) bad += plane_of_block(b, m_plane) != 4 * b / plane;
+  for (int rem = 0; rem < plane; ++rem) bad += quot(rem, m_row) != rem / Lh;
+  return bad;
+}

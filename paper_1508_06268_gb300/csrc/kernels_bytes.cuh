@@ -30,9 +30,15 @@ struct BytesArgs {
   SelftestStop stop;
 };
 
-// floor(n / d) for n d < 2^32 and d >= 2 with m = recip(d).
-__device__ __forceinline__ uint32_t recip(uint32_t d) { return 0xFFFFFFFFu / d + 1u; }
-__device__ __forceinline__ int quot(int n, uint32_t m) { return (int)__umulhi((uint32_t)n, m); }
+// floor(n / d) for n d < 2^32 and d >= 2 with m = recip(d).  The largest argument is a half-plane number in a
+// colour (locate), L^5 / 16 < 2^32; rfim_selftest_bytes checks the bound and the quotients.
+constexpr int32_t kBytesMaxL = 144;
+__host__ __device__ __forceinline__ uint32_t recip(uint32_t d) { return 0xFFFFFFFFu / d + 1u; }
+__host__ __device__ __forceinline__ int quot(int n, uint32_t m) { return (int)(((uint64_t)(uint32_t)n * m) >> 32); }
+
+// Plane of the first site of block b (site 4 b of the colour) with m = recip(plane / 2): planes hold an even
+// number of sites, and halving both sides keeps the product below 2^32 (4 b and plane pass it at L = 112).
+__host__ __device__ __forceinline__ int plane_of_block(int b, uint32_t m) { return quot(2 * b, m); }
 
 template <int VW>
 struct BytesWord;
@@ -114,16 +120,15 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
 
   // Philox blocks that hold sites of this slab; with VW = 1 the first and last may hold others' too
   const int qa = z0 * plane, qb = qa + PZ * plane, b0 = qa >> 2, nblk = ((qb + 3) >> 2) - b0, items = ok ? gact * nblk : 0;
-  const uint32_t m_blk = recip((uint32_t)nblk), m_plane = recip((uint32_t)plane), m_row = recip((uint32_t)Lh);
+  const uint32_t m_blk = recip((uint32_t)nblk), m_plane = recip((uint32_t)plane / 2), m_row = recip((uint32_t)Lh);
   const int zup = S == 1 ? -(PZ - 1) * PS : PS, zdn = -zup;  // z neighbours of the slab's end planes
 
   constexpr int NR = 4 / VW;  // row words of a block
   // where block b's sites are (c < 0: for both colours, else with the x neighbour of colour c in both
   // places); sites outside the slab are placed on its first one and left out
   auto locate = [&](int b, int c, RowWord (&rw)[NR]) {
-    const int q = 4 * b;
-    int z = quot(q, m_plane);
-    const int rem = q - z * plane;
+    int z = plane_of_block(b, m_plane);
+    const int rem = 4 * b - z * plane;
     int y = quot(rem, m_row), xh = rem - y * Lh;
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
