@@ -349,6 +349,9 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
               if (push) {
                 push_halos(c, WHOLE_TILES ? coarse : c, h);
                 ++h;
+                // the next visit updates words of both colours at once; otherwise a pass of the other colour
+                // and its barrier lie between a push and the next update of the words it reads
+                if (WHOLE_TILES) __syncthreads();
               }
             }
           }
