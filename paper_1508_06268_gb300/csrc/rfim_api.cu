@@ -702,7 +702,6 @@ int rfim_disorder_average(const double *thermals, int32_t n, int32_t R, double *
 int rfim_get_state(rfim_ctx *ctx, int8_t *spins, int32_t *t2r, double *E, int64_t *sweep, int64_t *xstep) {
   if (!ctx) return RFIM_EINVAL;
   rfim_ctx *c = ctx;
-  if (int rc = read_error(c)) return rc;
   const size_t RN = (size_t)c->R * c->N;
   RealView v = view_of(c);
   if (spins) {
@@ -712,18 +711,20 @@ int rfim_get_state(rfim_ctx *ctx, int8_t *spins, int32_t *t2r, double *E, int64_
     }
     CUDA_OR_FAIL(c, launch_to_natural(v, c->R, c->layout == RFIM_LAYOUT_BITPACK, c->scratch8, c->stream));
     c->launches += 1;
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(spins, c->scratch8, RN, cudaMemcpyDeviceToHost, c->stream));
   }
-  if (t2r) CUDA_OR_FAIL(c, cudaMemcpyAsync(t2r, c->t2r, c->R * 4, cudaMemcpyDeviceToHost, c->stream));
-  if (E) {
-    // recompute from the current spins into the energy buffer, then read it
+  if (E) {  // recomputed from the current spins into the energy buffer
     CUDA_OR_FAIL(c, launch_energy(v, (double)c->J, (double)c->h, c->layout == RFIM_LAYOUT_BITPACK, c->stream,
                                  c->eparts.count ? &c->eparts : nullptr));
     c->launches += 1;
-    CUDA_OR_FAIL(c, cudaMemcpyAsync(E, c->E, c->R * 8, cudaMemcpyDeviceToHost, c->stream));
   }
+  // nothing of the caller's is written when an error is reported
+  if (int rc = read_error(c)) return rc;
   CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
   if (int rc = report_error(c)) return rc;
+  if (spins) CUDA_OR_FAIL(c, cudaMemcpyAsync(spins, c->scratch8, RN, cudaMemcpyDeviceToHost, c->stream));
+  if (t2r) CUDA_OR_FAIL(c, cudaMemcpyAsync(t2r, c->t2r, c->R * 4, cudaMemcpyDeviceToHost, c->stream));
+  if (E) CUDA_OR_FAIL(c, cudaMemcpyAsync(E, c->E, c->R * 8, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_OR_FAIL(c, cudaStreamSynchronize(c->stream));
   if (sweep) *sweep = c->sweep;
   if (xstep) *xstep = c->xstep;
   return RFIM_OK;

@@ -88,3 +88,16 @@ def test_intervals_swept_apart_match_oracle(mh, tile, every, monkeypatch):
     np.testing.assert_array_equal(st["spins"], o.spins())
     np.testing.assert_array_equal(st["t2r"], o.perm()[0])
     np.testing.assert_array_equal(g.observables()["sums"], o.observables())
+
+
+def test_reported_error_leaves_the_callers_arrays(monkeypatch):
+    """A read that reports an expired wait writes nothing of the caller's."""
+    import ctypes as C
+    g, _ = pair(monkeypatch, 16, 5, "2,2,2,256,r", 0)
+    g.selftest_resident(0)
+    g.run(4, 2, 0)
+    spins, t2r, E = np.full((5, 4096), 7, np.int8), np.full(5, -7, np.int32), np.full(5, 0.5)
+    sweep, xstep = C.c_int64(-7), C.c_int64(-7)
+    rc = rf.load().rfim_get_state(g._h, spins.ctypes.data, t2r.ctypes.data, E.ctypes.data, C.byref(sweep), C.byref(xstep))
+    assert rc == rf.ETIMEOUT
+    assert (spins == 7).all() and (t2r == -7).all() and (E == 0.5).all() and sweep.value == xstep.value == -7
