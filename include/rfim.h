@@ -361,6 +361,11 @@ int rfim_selftest_bytes(int32_t L);
    default stream; the context of the calling thread stays usable after an expiry. */
 int rfim_selftest_wait(int32_t spin_limit, int32_t set_flag);
 
+/* The same for the bounded waits inside launches: which = 0 a slab's wait for its neighbours' end planes (an
+   mbarrier phase), 1 the wait for an energy record, 2 the batched kernel's wait for an interval of its
+   realization.  spin_limit as above, up to 2^20 polls. */
+int rfim_selftest_waits(int32_t which, int32_t spin_limit, int32_t set_flag);
+
 /* Self-test of the resident plan's launches (the paper has no counterpart): what happens after a bounded wait
    inside one has been given up, and when the numbers that exchange intervals carry start again.
    In the following launches of ctx, CTA stop_cta (-1: none) acts at the start of interval stop_interval

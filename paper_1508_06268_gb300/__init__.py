@@ -114,6 +114,7 @@ def load():
             L.rfim_exchange_noalloc.argtypes = [C.POINTER(ExchangeBuffers), u32, i64, P]
             L.rfim_selftest_grid.argtypes = [i32, i32, i32]
             L.rfim_selftest_wait.argtypes = [i32, i32]
+            L.rfim_selftest_waits.argtypes = [i32, i32, i32]
             L.rfim_selftest_bytes.argtypes = [i32]
             L.rfim_selftest_resident.argtypes = [P, i32, i32, u32]
             L.rfim_debug_build.argtypes = []
@@ -136,7 +137,8 @@ def load():
                          "rfim_exchange_noalloc", "rfim_tune", "rfim_selftest_grid", "rfim_selftest_wait",
                          "rfim_set_measure_xi", "rfim_set_multihit", "rfim_thermal",
                          "rfim_disorder_average", "rfim_server_tune", "rfim_debug_build",
-                         "rfim_selftest_debug", "rfim_get_plan", "rfim_selftest_resident", "rfim_selftest_bytes"):
+                         "rfim_selftest_debug", "rfim_get_plan", "rfim_selftest_resident", "rfim_selftest_bytes",
+                         "rfim_selftest_waits"):
                 getattr(L, name).restype = C.c_int
             _lib = L
     return _lib
@@ -248,6 +250,11 @@ def disorder_average(thermals) -> np.ndarray:
 def selftest_wait(spin_limit: int, set_flag: bool) -> int:
     """Status of one bounded device wait on a flag that is unset (expires) or set."""
     return load().rfim_selftest_wait(spin_limit, 1 if set_flag else 0)
+
+
+def selftest_waits(which: int, spin_limit: int, set_flag: bool) -> int:
+    """The same for the waits inside launches: 0 halo planes, 1 an energy record, 2 a served interval."""
+    return load().rfim_selftest_waits(which, spin_limit, 1 if set_flag else 0)
 
 
 class Realization:

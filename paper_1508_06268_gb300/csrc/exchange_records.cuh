@@ -62,10 +62,11 @@ __device__ __forceinline__ void record_load(const uint4 *rec, long long *F, unsi
 __device__ __forceinline__ int record_bonds(unsigned long long hi) { return (int)((hi >> 20) & 0x3FFFFFu) - (1 << 21); }
 __device__ __forceinline__ int record_spin(unsigned long long hi) { return (int)(hi & 0xFFFFFu) - (1 << 19); }
 
-// The record of interval `epoch`, polled at most kRecordSpinLimit times; false when it did not arrive
+// The record of interval `epoch`, polled at most `polls` times; false when it did not arrive
 // (recorded in *err) or an earlier wait of this launch expired.
-__device__ __forceinline__ bool record_await(const uint4 *rec, uint32_t epoch, unsigned *err, int *B, int *M, long long *F) {
-  for (unsigned it = 0; it < kRecordSpinLimit; ++it) {
+__device__ __forceinline__ bool record_await(const uint4 *rec, uint32_t epoch, unsigned *err, int *B, int *M, long long *F,
+                                             unsigned polls = kRecordSpinLimit) {
+  for (unsigned it = 0; it < polls; ++it) {
     unsigned long long hi;
     record_load(rec, F, &hi);
     if ((uint32_t)(hi >> 42) == epoch) {

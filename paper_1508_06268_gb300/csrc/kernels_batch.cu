@@ -13,6 +13,7 @@
 // items of each interval finish: 24 mixed realizations have 2.8 rounds of items per interval, and 200
 // sweeps of them take 36.6 ms of device time instead of 39.5 (four intervals per launch).
 #include "batch.h"
+#include "batch_wait.cuh"
 
 namespace rfim {
 
@@ -35,22 +36,6 @@ __device__ __forceinline__ void run_item(const SlotDesc &sd, const BatchItem &bi
     bits_interval<L, 1, GT, false, true>(sd.v, sd.G, bi.r0, bi.gact, 0, sweep0, nsw, sd.field4, xa, keys);
 }
 
-// Waits until the realization has completed `iv` intervals of this launch.  The number of polls is
-// limited by more than its intervals so far can take (a sweep of an item is far below 1 ms per replica);
-// on expiry, or after another CTA's, the error word is set and the item is left out.
-__device__ __forceinline__ bool await_interval(const SlotCtl *ctl, uint32_t iv, int gact, unsigned *err) {
-  const unsigned long long limit = (1ull << 22) + (unsigned long long)iv * ctl->nsw * gact * 4096ull;
-  for (unsigned long long n = 0; n < limit; ++n) {
-    uint32_t done;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(done) : "l"(&ctl->done) : "memory");
-    if (done >= iv) return true;
-    if (*(volatile unsigned *)err & 2u) return false;
-    __nanosleep(200);
-  }
-  atomicOr(err, 2u);
-  return false;
-}
-
 __global__ void __launch_bounds__(kBatchThreads) k_batch_bits(const SlotDesc *__restrict__ slots, SlotCtl *ctls, int nslots,
                                                               const BatchItem *__restrict__ items, BatchQueue *q,
                                                               int intervals, unsigned *err) {
@@ -66,7 +51,7 @@ __global__ void __launch_bounds__(kBatchThreads) k_batch_bits(const SlotDesc *__
         item = (int)(n % (unsigned)nitems);
         const SlotCtl *ctl = ctls + items[item].slot;
         // finished realizations idle until they are retired
-        if ((int)iv >= ctl->left0 || (iv > 0 && !await_interval(ctl, iv, items[item].gact, err))) item = -2;
+        if ((int)iv >= ctl->left0 || (iv > 0 && !await_interval(ctl, iv, interval_polls(*ctl, iv, items[item].gact), err))) item = -2;
       }
       s_item = item;
     }

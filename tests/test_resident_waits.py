@@ -101,3 +101,28 @@ def test_reported_error_leaves_the_callers_arrays(monkeypatch):
     rc = rf.load().rfim_get_state(g._h, spins.ctypes.data, t2r.ctypes.data, E.ctypes.data, C.byref(sweep), C.byref(xstep))
     assert rc == rf.ETIMEOUT
     assert (spins == 7).all() and (t2r == -7).all() and (E == 0.5).all() and sweep.value == xstep.value == -7
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_each_wait_expires(which):
+    """A wait for what nobody sets ends with the status, one for what is set with success; the context goes on."""
+    assert rf.selftest_waits(which, 1000, False) == rf.ETIMEOUT
+    assert rf.selftest_waits(which, 1, True) == rf.OK
+    assert rf.selftest_waits(which, 1, False) == rf.ETIMEOUT
+    assert rf.selftest_waits(which, 0, True) == rf.EINVAL
+
+
+@pytest.mark.parametrize("L,R,plan", [(16, 5, "2,2,2,256,r"), (24, 5, "4,2,4,512,b")])
+def test_interval_numbers_start_again(L, R, plan, monkeypatch):
+    """The numbers that energy records carry end at 2^22 - 1; launches before, across and after that line."""
+    g, o = pair(monkeypatch, L, R, plan, 0)
+    g.selftest_resident(number=(1 << 22) - 12)
+    for sweeps in (4, 12, 6, 8):
+        g.run(sweeps, 2, 0)
+        o.run(sweeps, 2, 0)
+    st = g.get_state()
+    np.testing.assert_array_equal(st["spins"], o.spins())
+    np.testing.assert_array_equal(st["t2r"], o.perm()[0])
+    np.testing.assert_array_equal(g.observables()["sums"], o.observables())
+    with pytest.raises(rf.RfimError):
+        g.selftest_resident(number=(1 << 22) - 1)
