@@ -587,15 +587,18 @@ __device__ __forceinline__ uint32_t deposit_bits(uint32_t x) {
 // Metropolis update of one word (32 sites of colour c at plane zl, word iw of the slab) in the GT
 // replicas of group grp: neighbour counts from the other colour's words, one Philox block per
 // (block j, replica) with counter (8 wq + j, r, ctr2, tag), decisions, and the flipped words
-// written back.  Only the blocks with their bit set in PAT are updated (0xFF: all; otherwise four
-// of them, whose bimodal bits are collected side by side and then moved to their bytes' bit j).  Replicas past the end of a partial group repeat the last one; only their write is
-// skipped.
+// written back.  Only the four blocks with their bit set in PAT are updated.  Bimodal: tables of thr - 1 (tab_fill
+// with NEG = false), each accepted site's bit set by a comparison and a predicated OR, round keys formed
+// in registers.  Rejections collected as carries have to be moved to their bits afterwards and pay only
+// where all eight blocks are updated, and the keys' constant bank loses here too: L = 64, R = 128, tiles of 16,
+// 80 passes 2646 us; with keys from the constant bank 2713, with carries as well 2801.  Replicas
+// past the end of a partial group repeat the last one; only their write is skipped.
 template <int L, int S, int GT, bool BIM, uint32_t PAT>
 __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int c, int zl, int iw, int z0, int grp,
                                             int gact, int r0, uint32_t ctr2, uint32_t tag, uint32_t slot0,
                                             const float4 *__restrict__ field4, int up_rank, int dn_rank,
                                             const PhiloxKeys &keys) {
-  static_assert(PAT == 0xFFu || __builtin_popcount(PAT) == 4, "a pass updates all blocks or four of them");
+  static_assert(__builtin_popcount(PAT) == 4, "a pass updates four blocks of a word");
   using Gm = BitsGeom<L>;
   constexpr int P = Gm::P, W = Gm::W, PZ = L / S, WC = PZ * P;
   constexpr int64_t WPAD = (W + 31) / 32 * 32;
@@ -630,8 +633,17 @@ __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int
 #pragma unroll
       for (int gg = 0; gg < GT; ++gg) {
         const int g = min(grp * GT + gg, gact - 1);
-        const Words4 w = philox_keyed(keys, (uint32_t)(8 * wq + j), (uint32_t)(r0 + g), ctr2, tag);
-        decide_block<BIM>(w, ps[gg], j, slot0 + (uint32_t)g * kTabSlot, hh4[j], fl[gg]);
+        const uint32_t block = (uint32_t)(8 * wq + j), r = (uint32_t)(r0 + g);
+        const Words4 w = BIM ? philox10(v.seed, v.realization, block, r, ctr2, tag) : philox_keyed(keys, block, r, ctr2, tag);
+        const uint32_t slot = slot0 + (uint32_t)g * kTabSlot;
+        if constexpr (BIM) {
+          const uint32_t offs = block_offsets<true>(ps[gg], j);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (accept_table(w.w[k], lds_u32(__byte_perm(offs, slot, 0x7650u | (uint32_t)k)))) fl[gg].f[0] |= 1u << (8 * k + j);
+        } else {
+          decide_block<false>(w, ps[gg], j, slot, hh4[j], fl[gg]);
+        }
       }
     }
   }
@@ -639,8 +651,7 @@ __device__ __forceinline__ void update_word(const RealView &v, uint32_t *sp, int
   for (int gg = 0; gg < GT; ++gg) {
     const int g = grp * GT + gg;
     if (GT > 1 && g >= gact) continue;
-    const uint32_t flip = BIM && PAT != 0xFFu ? deposit_bits<PAT>(~fl[gg].rejects()) : fl[gg].template word<8>();
-    sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ flip;
+    sp[((size_t)g * 2 + c) * WC + wl] = sf[gg] ^ fl[gg].f[0];
   }
 }
 

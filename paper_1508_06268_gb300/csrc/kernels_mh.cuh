@@ -44,7 +44,7 @@ __device__ __forceinline__ void bits_interval_mh(const RealView &v, int G, int r
   const int nt = blockDim.x, tid = threadIdx.x;
 
   copy_slab<L, S, true>(v, sp, r0, gact, z0);
-  tab_fill<BIM>(v, tab, slot0, gact, [&](int g) { return r0 + g; });
+  tab_fill<BIM, false>(v, tab, slot0, gact, [&](int g) { return r0 + g; });
   sync_slabs<S>();
 
   const int ngroups = (gact + GT - 1) / GT;
