@@ -368,12 +368,12 @@ int rfim_selftest_waits(int32_t which, int32_t spin_limit, int32_t set_flag);
 
 /* Self-test of the resident plan's launches (the paper has no counterpart): what happens after a bounded wait
    inside one has been given up, and when the numbers that exchange intervals carry start again.
-   In the following launches of ctx, CTA stop_cta (-1: none) acts at the start of interval stop_interval
-   of the launch as if one of its waits had run out.  The launch then ends in order, the next
+   In the following launches of ctx, CTA stop_cta (-1: none; debug library only) acts at the start of interval
+   stop_interval of the launch as if one of its waits had run out.  The launch then ends in order, the next
    rfim_observables or rfim_get_state returns RFIM_ETIMEOUT, and the context stays usable
    (rfim_set_state gives it a valid state again).  number > 0: intervals are numbered on from there (below
    2^22 - 1).  Errors: RFIM_EINVAL (stop_cta < -1, stop_interval < 0, a number too large or already
-   used), RFIM_ESTATE when the plan is not a resident one. */
+   used), RFIM_ESTATE when the plan is not a resident one, and for stop_cta >= 0 in librfim.so. */
 int rfim_selftest_resident(rfim_ctx *ctx, int32_t stop_cta, int32_t stop_interval, uint32_t number);
 
 /* Bounds-checked build (no counterpart in the paper; it stands in for a memory checker).  The same

@@ -17,6 +17,12 @@ constexpr unsigned kDbgScratch = 1u << 12;   // no-alloc scratch slot beyond the
 constexpr unsigned kDbgGlobal = 1u << 13;    // global lattice index outside the realization
 constexpr unsigned kDbgMask = 0xFF00u;
 
+__device__ __forceinline__ uint32_t cluster_ctas() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
 #ifdef RFIM_DEBUG
 constexpr bool kDebugBuild = true;
 __device__ __forceinline__ bool dbg_check(unsigned *err, bool ok, unsigned bit) {
@@ -26,11 +32,6 @@ __device__ __forceinline__ bool dbg_check(unsigned *err, bool ok, unsigned bit) 
 __device__ __forceinline__ uint32_t dyn_smem_bytes() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_ctas() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
   return r;
 }
 #define RFIM_DCHECK(err, cond, bit) ::rfim::dbg_check((err), (cond), (bit))

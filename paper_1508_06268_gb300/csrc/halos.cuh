@@ -25,15 +25,16 @@ constexpr unsigned kMbarSpinLimit = 1u << 20;
 
 // Waits of a CTA that were given up.  Half-sweeps (or tile visits) alternate between two flags: a thread that
 // reads one late, just before the next barrier, must not see what others set in the half-sweep after.
-// (L = 32, R = 70: 1.24 us per half-sweep; with the flag read by every thread 1.27, with __syncthreads_or instead
-// of the flags 1.29, with waits whose end nobody looks at 1.20.)
+// (L = 32, R = 70: 1.22 us per half-sweep, 1.20 with waits whose end nobody looks at; the flag read by every
+// thread instead took 1.27, __syncthreads_or instead of the flags 1.29.)
 struct GaveUp {
   uint32_t sweep[2], exchange;
 };
 
 struct HaloBars {
   uint64_t mbar[2];
-  uint32_t pushed;   // pushes this CTA has made, once it is done
+  uint32_t bytes;    // of a push to one neighbour
+  uint32_t pushed;   // pushes this CTA has made
   uint32_t stopped;  // a CTA of the cluster has given up a wait
 };
 
@@ -48,11 +49,12 @@ __device__ __forceinline__ uint32_t halo_bar(const HaloBars *hb, uint32_t h) {
 }
 
 // By one thread, before the cluster barrier that precedes the first push.
-__device__ __forceinline__ void halo_init(HaloBars *hb) {
+__device__ __forceinline__ void halo_init(HaloBars *hb, uint32_t bytes) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;" ::"r"(halo_bar(hb, 0)),
                "r"(halo_bar(hb, 1))
                : "memory");
-  hb->stopped = 0u;
+  hb->bytes = bytes;
+  hb->pushed = hb->stopped = 0u;
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
@@ -78,9 +80,22 @@ __device__ __forceinline__ bool halo_wait(const HaloBars *hb, uint32_t h, unsign
   return mbar_wait(halo_bar(hb, h), (h >> 1) & 1u, kMbarSpinLimit, err);
 }
 
+// After the barrier that ends a half-sweep (tile visit), by the threads that push: whether they may, i.e. no wait of
+// the CTA for the push before was given up (flag `f` of the two), nor one earlier: who sees a flag set sets
+// the other one for the next time.
+__device__ __forceinline__ bool halo_may_push(volatile GaveUp *g, int f) {
+  if (g->sweep[f] == 0u) return true;
+  g->sweep[f ^ 1] = 1u;
+  return false;
+}
+
 // This CTA's arrival for push number h, `bytes` from both neighbours together (one thread).
-__device__ __forceinline__ void halo_expect(const HaloBars *hb, uint32_t h, uint32_t bytes) {
+__device__ __forceinline__ void halo_arrive(const HaloBars *hb, uint32_t h, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(halo_bar(hb, h)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void halo_expect(HaloBars *hb, uint32_t h, uint32_t bytes) {
+  *(volatile uint32_t *)&hb->pushed = h + 1;
+  halo_arrive(hb, h, bytes);
 }
 
 // 16 bytes of push number h to where `to` lies in CTA `peer`.
@@ -101,7 +116,7 @@ __device__ __forceinline__ void halo_drain(const HaloBars *hb, uint32_t mine, ui
     const uint32_t sent = bytes * (((int32_t)(below - p) > 0) + ((int32_t)(above - p) > 0));
     if (back == 0u) {
       if (sent == 0u) return;
-      halo_expect(hb, p, sent);
+      halo_arrive(hb, p, sent);
     } else if (sent < 2u * bytes) {
       asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(halo_bar(hb, p)), "r"(2u * bytes - sent)
                    : "memory");
@@ -111,20 +126,24 @@ __device__ __forceinline__ void halo_drain(const HaloBars *hb, uint32_t mine, ui
 }
 
 // End of a launch of slabs: all threads of all CTAs of the cluster call it, after a barrier that follows their
-// last wait.  `pushed`: this CTA's pushes (thread 0); `stop`: a wait of this CTA has been given up.  No CTA exits while a push to it is on its way.
-__device__ __forceinline__ void halo_leave(HaloBars *hb, int rank, int S, uint32_t pushed, bool stop, uint32_t bytes) {
-  if (threadIdx.x == 0) hb->pushed = pushed;
-  if (stop && (int)threadIdx.x < S)
+// last wait.  `stop`: a wait of this CTA has been given up.  No CTA exits while a push to it is on its way.
+// (What only this path needs is in shared memory or read from the hardware again: kept in registers through the
+// sweeps it cost 2 % at L = 40 on bytes.)
+__device__ __forceinline__ void halo_leave(HaloBars *hb, bool stop) {
+  const uint32_t S = cluster_ctas();
+  if (stop && threadIdx.x < S)
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
                      mapa_shared((uint32_t)__cvta_generic_to_shared(&hb->stopped), threadIdx.x)),
                  "r"(1u)
                  : "memory");
   __syncwarp();
   sync_slabs<2>();
-  if (*(volatile uint32_t *)&hb->stopped == 0u) return;  // every wait of the cluster was served
-  if (threadIdx.x == 0)
-    halo_drain(hb, pushed, dsmem_load(&hb->pushed, (uint32_t)(rank + S - 1) % S),
-               dsmem_load(&hb->pushed, (uint32_t)(rank + 1) % S), bytes);
+  volatile HaloBars *own = hb;
+  if (own->stopped == 0u) return;  // every wait of the cluster was served
+  if (threadIdx.x == 0) {
+    const uint32_t rank = cluster_rank();
+    halo_drain(hb, own->pushed, dsmem_load(&hb->pushed, (rank + S - 1) % S), dsmem_load(&hb->pushed, (rank + 1) % S), own->bytes);
+  }
   __syncwarp();
   sync_slabs<2>();
 }

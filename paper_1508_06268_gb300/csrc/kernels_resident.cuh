@@ -164,6 +164,9 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
   const int R = v.R;
 
+  constexpr int NC = WHOLE_TILES ? 2 : 1;                     // colours of a push
+  const uint32_t push_bytes = (uint32_t)(gact * NC * P * 4);  // to each neighbour
+
   uint32_t *sp = sm;                            // [G][2][CW]
   uint32_t *tab = sm + (size_t)ra.G * 2 * CW;   // G decision-table slots
   const uint32_t slot0 = tab_slot0(tab);
@@ -203,7 +206,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   const long long Htot = limbs ? xa.fquant->Htot : 0;
   if (tid == 0) gave_up.sweep[0] = gave_up.sweep[1] = gave_up.exchange = 0u;
   if (S > 1) {
-    if (tid == 0) halo_init(&hb);
+    if (tid == 0) halo_init(&hb, push_bytes);
     sync_slabs<S>();  // every CTA's mbarriers are ready before the first push
   } else {
     __syncthreads();
@@ -262,16 +265,9 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   // After half-sweep number h of this launch (all of the CTA's updates of colour c done): the slab's
   // first and last planes into the halo planes of the slabs below and above (halos.cuh).
   // WHOLE_TILES: both colours after tile visit number h.
-  constexpr int NC = WHOLE_TILES ? 2 : 1;
-  const uint32_t push_bytes = (uint32_t)(gact * NC * P * 4);  // to each neighbour
-  uint32_t pushed = 0;  // (thread 0) pushes made
-  bool stopped = !ok;   // (threads that push) no more pushes
   auto push_halos = [&](int colour, int flag, uint32_t h) {
     constexpr int VEC = P >= 4 ? P / 4 : 1;
-    if (tid >= gact * 2 * NC * VEC) return;
-    stopped |= gave_up.sweep[flag] != 0u;
-    if (stopped) return;
-    pushed = h + 1;
+    if (tid >= gact * 2 * NC * VEC || !halo_may_push(&gave_up, flag)) return;
     if (tid == 0) halo_expect(&hb, h, 2 * push_bytes);
     for (int t = tid; t < gact * 2 * NC * VEC; t += nt) {
       const int g = t / (2 * NC * VEC), c = NC == 2 ? t / (2 * VEC) & 1 : colour, side = t / VEC & 1, q = t % VEC * 4;
@@ -307,7 +303,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   const int n_iv = xa.enabled ? ra.n_iv : 1;
   uint32_t h = 0, sweep = sweep0;  // half-sweeps done in this launch; current sweep
   for (int iv = 0; iv < n_iv; ++iv) {
-    if (!ok || stops_here(ra.stop, iv, xa.err)) {
+    if (!ok || (kDebugBuild && stops_here(ra.stop, iv, xa.err))) {
       gave_up.exchange = 1u;
       break;
     }
@@ -503,7 +499,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
   }
   __syncthreads();
   const bool gone = gave_up.exchange != 0u;  // this launch's results are not to be had
-  if (S > 1) halo_leave(&hb, rank, S, pushed, gone, push_bytes);
+  if (S > 1) halo_leave(&hb, gone);
 
   for (int t = tid; ok && t < gact * 2 * WC; t += nt) {
     const int g = t / (2 * WC), rem = t % (2 * WC), c = rem / WC, wl = rem % WC;

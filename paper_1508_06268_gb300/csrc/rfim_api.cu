@@ -796,6 +796,7 @@ int rfim_selftest_resident(rfim_ctx *ctx, int32_t stop_cta, int32_t stop_interva
   if (stop_cta < -1 || stop_interval < 0 || number >= kRecordEpochs - 1 || (number > 0 && number <= p.epoch))
     return fail(ctx, RFIM_EINVAL, "invalid self-test arguments");
   if (!p.resident() && p.mh_res.threads == 0) return fail(ctx, RFIM_ESTATE, "not a resident plan");
+  if (stop_cta >= 0 && !kDebugBuild) return fail(ctx, RFIM_ESTATE, "stops are compiled only into librfim_debug.so");
   p.stop = SelftestStop{stop_cta, stop_interval};
   if (number > 0) p.epoch = number - 1;
   return RFIM_OK;

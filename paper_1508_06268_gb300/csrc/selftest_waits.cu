@@ -20,7 +20,7 @@ __global__ void k_selftest_waits(WaitWords *w, int which, unsigned limit, int se
   __shared__ __align__(8) HaloBars hb;
   if (threadIdx.x != 0) return;
   if (which == 0) {
-    halo_init(&hb);
+    halo_init(&hb, 0u);
     if (set) halo_expect(&hb, 0, 0);  // the only arrival, no bytes: phase 0 is complete
     mbar_wait(halo_bar(&hb, 0), 0u, limit, &w->err);
   } else if (which == 1) {

@@ -1,6 +1,10 @@
 """Bounded waits inside the resident launches: one that is given up ends the launch in order (no CTA pushes
 or arrives again, none leaves while a push to it is on its way), the error is reported once, and
 the realization goes on from a state that is set."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -9,6 +13,8 @@ import paper_1508_06268_gb300 as rf
 from paper_1508_06268_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 SLABS = [  # L, R, "S,G,NB,threads,r" (m: several items per thread, b: bytes), tile (0: plain checkerboard)
     (8, 7, "1,3,1,256,r", 0), (10, 3, "1,1,4,128,b", 0), (16, 5, "1,3,2,384,r", 8),
@@ -22,43 +28,85 @@ SLABS = [  # L, R, "S,G,NB,threads,r" (m: several items per thread, b: bytes), t
 def pair(monkeypatch, L, R, plan, tile):
     kw = dict(h=1.5, field_kind=rf.FIELD_BIMODAL, field_seed=3, seed=42)
     temps = inputs.geometric_temps(1.0, 5.0, R)
-    monkeypatch.setenv("RFIM_BITS_PLAN", plan)
+    env = monkeypatch or pytest.MonkeyPatch()
+    env.setenv("RFIM_BITS_PLAN", plan)
     g = rf.Realization(L, temps, layout=rf.LAYOUT_INT8 if plan[-1] == "b" else rf.LAYOUT_BITPACK, **kw)
     o = oracle.Oracle(L, temps, **kw)
     if tile:
         g.set_multihit(2, tile)
         o.set_multihit(2, tile)
-    monkeypatch.delenv("RFIM_BITS_PLAN")
+    env.delenv("RFIM_BITS_PLAN")
     assert g.plan() == plan
     return g, o
 
 
-@pytest.mark.parametrize("L,R,plan,tile", SLABS)
-def test_given_up_wait_ends_in_order(L, R, plan, tile, monkeypatch):
-    """One CTA gives up a wait: at once, in a later interval, and in launches that are queued behind the failed
-    one.  Its neighbours in the cluster, at every distance, and the other clusters stop too."""
-    g, o = pair(monkeypatch, L, R, plan, tile)
+CHILD = r"""
+import ctypes as C, os, sys
+import numpy as np
+sys.path.insert(0, os.environ["RFIM_ROOT"])
+import paper_1508_06268_gb300 as rf
+from tests.test_resident_waits import SLABS, pair
+
+assert rf.debug_build()
+
+
+def timed_out(f):
+    try:
+        f()
+    except rf.RfimError as e:
+        return e.code == rf.ETIMEOUT
+    return False
+
+
+for L, R, plan, tile in SLABS:
+    g, o = pair(None, L, R, plan, tile)
     S, G = int(plan.split(",")[0]), int(plan.split(",")[1])
     ctas = (R + G - 1) // G * S
     g.run(4, 2, 0)
     o.run(4, 2, 0)
     good = g.get_state()
-    np.testing.assert_array_equal(good["spins"], o.spins())
+    assert np.array_equal(good["spins"], o.spins()), plan
     for cta, interval in ((0, 0), (ctas - 1, 1), (S // 2, 2)):
         g.selftest_resident(cta, interval)
         g.run(12, 2, 0)
         g.sweep(3)
         g.exchange(0)
-        with pytest.raises(rf.RfimError) as e:
-            g.get_state()
-        assert e.value.code == rf.ETIMEOUT
+        assert timed_out(g.get_state), (plan, cta, interval)
         g.selftest_resident()
         g.set_state(good["spins"], good["t2r"], good["sweep"], good["xstep"])
     g.run(6, 2, 0)
     o.run(6, 2, 0)
     st = g.get_state()
-    np.testing.assert_array_equal(st["spins"], o.spins())
-    np.testing.assert_array_equal(st["t2r"], o.perm()[0])
+    assert np.array_equal(st["spins"], o.spins()), plan
+    assert np.array_equal(st["t2r"], o.perm()[0]), plan
+
+# a read that reports the error writes nothing of the caller's
+g, _ = pair(None, 16, 5, "2,2,2,256,r", 0)
+g.selftest_resident(0)
+g.run(4, 2, 0)
+spins, t2r, E = np.full((5, 4096), 7, np.int8), np.full(5, -7, np.int32), np.full(5, 0.5)
+sweep, xstep = C.c_int64(-7), C.c_int64(-7)
+rc = rf.load().rfim_get_state(g._h, spins.ctypes.data, t2r.ctypes.data, E.ctypes.data, C.byref(sweep), C.byref(xstep))
+assert rc == rf.ETIMEOUT
+assert (spins == 7).all() and (t2r == -7).all() and (E == 0.5).all() and sweep.value == xstep.value == -7
+print("waits ok")
+"""
+
+
+def test_given_up_wait_ends_in_order():
+    """Debug library: one CTA gives up a wait, at once, in a later interval, and in launches that are queued behind
+    the failed one.  Its neighbours in the cluster, at every distance, and the other clusters stop too."""
+    env = dict(os.environ, RFIM_LIBRARY="debug", RFIM_ROOT=ROOT)
+    env.pop("RFIM_BITS_PLAN", None)
+    r = subprocess.run([sys.executable, "-c", CHILD], cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
+    assert r.returncode == 0 and "waits ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
+def test_stops_are_refused_in_the_release_library(monkeypatch):
+    g, _ = pair(monkeypatch, 16, 5, "2,2,2,256,r", 0)
+    with pytest.raises(rf.RfimError) as e:
+        g.selftest_resident(0)
+    assert e.value.code == rf.ESTATE
 
 
 def test_long_intervals_do_not_run_out_of_polls(monkeypatch):
@@ -88,19 +136,6 @@ def test_intervals_swept_apart_match_oracle(mh, tile, every, monkeypatch):
     np.testing.assert_array_equal(st["spins"], o.spins())
     np.testing.assert_array_equal(st["t2r"], o.perm()[0])
     np.testing.assert_array_equal(g.observables()["sums"], o.observables())
-
-
-def test_reported_error_leaves_the_callers_arrays(monkeypatch):
-    """A read that reports an expired wait writes nothing of the caller's."""
-    import ctypes as C
-    g, _ = pair(monkeypatch, 16, 5, "2,2,2,256,r", 0)
-    g.selftest_resident(0)
-    g.run(4, 2, 0)
-    spins, t2r, E = np.full((5, 4096), 7, np.int8), np.full(5, -7, np.int32), np.full(5, 0.5)
-    sweep, xstep = C.c_int64(-7), C.c_int64(-7)
-    rc = rf.load().rfim_get_state(g._h, spins.ctypes.data, t2r.ctypes.data, E.ctypes.data, C.byref(sweep), C.byref(xstep))
-    assert rc == rf.ETIMEOUT
-    assert (spins == 7).all() and (t2r == -7).all() and (E == 0.5).all() and sweep.value == xstep.value == -7
 
 
 @pytest.mark.parametrize("which", [0, 1, 2])
