@@ -331,7 +331,8 @@ int rfim_tune(int32_t L, int32_t R, int32_t field_kind, char *plan_out, int32_t 
    "S,G,NB,threads,r" for the resident plan of small realizations (a cluster of S slabs holds G replicas
    for up to 512 exchange intervals per launch, NB Philox blocks of a word per thread item; "m" instead
    of "r" when a thread runs several items), with ",int8" appended when the int8 layout is staged as
-   bits; "S,G,4,threads,b" for the resident plan on bytes (int8 layout, L outside 8, 16, 32, 64), and ""
+   bits; "S,G,4,threads,b" for the resident plan on bytes (int8 layout, L outside 8, 16, 32, 64; calls whose
+   way into shared memory does not pay take a launch per half-sweep and two per exchange step), and ""
    when every half-sweep is a launch of its own (larger int8 realizations).  plan_out receives at most
    plan_cap chars (NUL included).
    Errors: RFIM_EINVAL (NULL ctx or plan_out, plan_cap < 1). */

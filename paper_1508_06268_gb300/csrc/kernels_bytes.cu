@@ -54,6 +54,26 @@ double bytes_cycles(int32_t L, const ResidentShape &s, int32_t R, int spread) {
          (s.S > 1 ? 300.0 + 200.0 * (per_sm - 1) : 0.0);
 }
 
+// Fitted to L = 4 to 116, R = 2 to 400 (Gaussian field; calls of two sweeps, of an exchange step, runs of 5 and of
+// 1 sweep per step), mostly within a fifth; bimodal ones are up to a sixth faster.  A few of the points, us per call, resident / apart: two sweeps
+// L = 116, R = 2 171 / 66, L = 40, R = 250 80 / 62, L = 24, R = 40 11 / 26, L = 10, R = 24 8.6 / 21; an exchange
+// step L = 40, R = 250 43 / 32, L = 50, R = 100 97 / 138, L = 24, R = 64 17 / 15.
+BytesCosts bytes_costs(int32_t L, const ResidentShape &s, int32_t R, double cycles) {
+  BytesCosts c;
+  const int w = row_width(L);
+  const double sites = 0.5 * (double)L * L * L * R * 1e-6, ksites = (double)L * L * L * 1e-3;  // per half-sweep, per replica
+  const double kib = (double)s.G * 2 * (slab_planes(L, s.S) + 2) * plane_stride(L) / 1024.0;
+  c.half = 0.3 + 1.12 * cycles / 2070.0;
+  c.launch = 7.0 + kib * (w == 4 ? 0.045 : w == 2 ? 0.09 : 0.35);
+  c.tail = 4.5 + (w == 1 ? 1.5 : 1.15) * c.half + 0.01 * R * s.S;
+  c.half_apart = std::min(4.2 + 0.35 * (R - 2), w == 4 ? 6.5 : 5.2) + (w == 4 ? 1.0 : 7.1) * sites;
+  const int waves = (R + 151) / 152;  // the energy kernels take a CTA per replica, several for rows of 16
+  c.step_apart = L % 16 == 0 ? 21.5 + 0.01 * ksites + sites
+                 : w == 4    ? 12.0 + 0.128 * ksites * waves + 0.02 * R
+                             : 12.0 + ksites * (1.0 + 0.45 * (waves - 1)) + 0.02 * R;
+  return c;
+}
+
 bool bytes_fits(int32_t L, int32_t R, bool bim, ResidentShape *s) {
   if (s->S < 1 || s->S > 8 || L < 2 * s->S || s->G < 1 || s->threads < 32 || s->threads > kBytesThreads || s->threads % 32)
     return false;
@@ -124,6 +144,7 @@ int make_bytes_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::
   p.threads = s.threads;
   p.smem = s.smem;
   p.res = s;
+  if (cycles > 0.0) p.cost = bytes_costs(L, s, Rcap, cycles);  // a named shape is taken for every launch
   p.rec_slots = (size_t)Rcap * s.S;
   const size_t rec_bytes = 2 * p.rec_slots * sizeof(uint4);
   cudaError_t e = cudaMalloc((void **)&p.rec, rec_bytes);

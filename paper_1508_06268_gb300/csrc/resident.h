@@ -72,6 +72,13 @@ struct ResidentLaunch {
   ResidentLaunch(const ResidentLaunch &) = delete;
 };
 
+// Estimated times (us) of the two ways to run a realization of the plan on bytes: a resident launch (a half-sweep,
+// the launch itself with the lattice's way in and out, the tail of an interval), or a launch per half-sweep and
+// two per exchange step.
+struct BytesCosts {
+  double half = 0.0, launch = 0.0, tail = 0.0, half_apart = 0.0, step_apart = 0.0;
+};
+
 // The same on bytes (kernels_bytes.cuh): realizations of the int8 layout at other even L.
 bool bytes_shape(int32_t L, int32_t R, bool bimodal, ResidentShape *out, double *cycles);
 cudaError_t launch_resident_bytes(const RealView &v, const ResidentShape &s, const ResidentArgs &args, uint32_t sweep0,

@@ -225,7 +225,7 @@ int do_sweeps(rfim_ctx *c, int64_t n) {
   RealView v = view_of(c);
   cudaEvent_t stop;
   CUDA_OR_FAIL(c, prof_begin(c, 0, &stop));
-  if (c->plan.counter) {  // bit layout, or the int8 layout staged as bits or resident as bytes
+  if (c->plan.counter && !c->plan.faster_apart(n, 1, false)) {  // bit layout, or the int8 layout staged as bits or resident as bytes
     CUDA_OR_FAIL(c, launch_sweeps_bits(v, c->plan, (uint32_t)c->sweep, (int32_t)n, false, 0u, 0, (double)c->J,
                                        (double)c->h, c->stream, &c->mh));
     c->launches += 1;
@@ -273,7 +273,7 @@ int do_sweeps_exchange_bits(rfim_ctx *c, int64_t n, int64_t measure_from, int32_
 }
 
 int do_exchange(rfim_ctx *c, int64_t measure_from) {
-  if (c->plan.counter) return do_sweeps_exchange_bits(c, 0, measure_from);
+  if (c->plan.counter && !c->plan.faster_apart(0, 1, true)) return do_sweeps_exchange_bits(c, 0, measure_from);
   RealView v = view_of(c);
   cudaEvent_t stop;
   CUDA_OR_FAIL(c, prof_begin(c, 1, &stop));
@@ -303,9 +303,9 @@ int do_run(rfim_ctx *c, int64_t n_sweeps, int32_t ex, int64_t measure_from) {
                          : c->plan.measures_xi(c->mh.mh)
                              ? std::min<int64_t>(c->plan.max_intervals(c->mh.mh), c->xi.intervals)
                              : 1;
-    const bool apart = c->plan.sweeps_apart(chunk, c->mh.mh);
-    if (ends_interval && !apart && chunk == ex && left >= 2 * (int64_t)ex && most > 1) {
-      const int64_t k = std::min(left / ex, most);
+    const int64_t k = chunk == ex ? std::max<int64_t>(1, std::min(left / ex, most)) : 1;
+    const bool apart = c->plan.sweeps_apart(chunk, c->mh.mh) || c->plan.faster_apart(chunk, k, true);
+    if (ends_interval && !apart && k > 1) {
       rc = do_sweeps_exchange_bits(c, ex, measure_from, (int32_t)k);
       if (rc) return rc;
       left -= k * ex;

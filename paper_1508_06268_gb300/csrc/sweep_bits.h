@@ -56,6 +56,18 @@ struct BitsPlan {
   bool sweeps_apart(int64_t n, int32_t mh) const {
     return (mh > 0 ? mh_res.threads > 0 : resident()) && n > kResidentSweeps / (mh > 1 ? mh : 1);
   }
+  BytesCosts cost;  // plan on bytes only
+  // Whether k intervals of n sweeps, each with an exchange step or without, are faster in a launch per
+  // half-sweep and step than in one resident launch: short calls of large lattices, whose way into shared
+  // memory and out again is not paid back, and lattices that few CTAs hold.
+  bool faster_apart(int64_t n, int64_t k, bool exchange) const {
+    if (cost.half <= 0.0) return false;
+    const double one = cost.launch + k * (2.0 * n * cost.half + (exchange ? cost.tail : 0.0));
+    // (estimates: where they are close the resident launch stands, of runs, whose tails the estimate puts too
+    // high, more so)
+    const double close = n > 0 && exchange ? 0.88 : n > 0 ? 0.92 : 0.95;
+    return k * (2.0 * n * cost.half_apart + (exchange ? cost.step_apart : 0.0)) < close * one;
+  }
   // exchange intervals one launch takes at most (mh passes per visit; 0: plain sweeps)
   int64_t max_intervals(int32_t mh) const {
     if (mh > 0) return mh_res.threads > 0 && mh < kResidentIntervals ? kResidentIntervals / mh : 1;
