@@ -125,23 +125,24 @@ __device__ __forceinline__ void halo_drain(const HaloBars *hb, uint32_t mine, ui
   }
 }
 
-// End of a launch of slabs: all threads of all CTAs of the cluster call it, after a barrier that follows their
-// last wait.  `stop`: a wait of this CTA has been given up.  No CTA exits while a push to it is on its way.
-// (What only this path needs is in shared memory or read from the hardware again: kept in registers through the
-// sweeps it cost 2 % at L = 40 on bytes.)
-__device__ __forceinline__ void halo_leave(HaloBars *hb, bool stop) {
-  const uint32_t S = cluster_ctas();
-  if (stop && threadIdx.x < S)
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
-                     mapa_shared((uint32_t)__cvta_generic_to_shared(&hb->stopped), threadIdx.x)),
-                 "r"(1u)
-                 : "memory");
-  __syncwarp();
+// A wait was given up (any thread, any number of them): every CTA of the cluster will know in halo_leave.
+__device__ __forceinline__ void halo_give_up(HaloBars *hb) {
+  const uint32_t flag = (uint32_t)__cvta_generic_to_shared(&hb->stopped);
+  for (uint32_t q = 0; q < cluster_ctas(); ++q)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa_shared(flag, q)), "r"(1u) : "memory");
+}
+
+// End of a launch of slabs: all threads of all CTAs of the cluster call it after their last wait.  No CTA exits
+// while a push to it is on its way.  What only the path after a given-up wait needs is in shared memory or read
+// from the hardware again (kept in registers through the sweeps it cost 2 % at L = 40 on bytes), and the path
+// of every other launch is the barrier and one load: a CTA barrier to gather the threads' flags took a call of
+// two sweeps at L = 20, R = 5 on bytes from 9.4 to 10.3 us.
+__device__ __forceinline__ void halo_leave(HaloBars *hb) {
   sync_slabs<2>();
   volatile HaloBars *own = hb;
   if (own->stopped == 0u) return;  // every wait of the cluster was served
   if (threadIdx.x == 0) {
-    const uint32_t rank = cluster_rank();
+    const uint32_t rank = cluster_rank(), S = cluster_ctas();
     halo_drain(hb, own->pushed, dsmem_load(&hb->pushed, (rank + S - 1) % S), dsmem_load(&hb->pushed, (rank + 1) % S), own->bytes);
   }
   __syncwarp();

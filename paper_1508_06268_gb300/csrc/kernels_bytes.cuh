@@ -203,7 +203,10 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     }
   };
   auto wait_halos = [&](uint32_t h, int c) {
-    if (!halo_wait(&hb, h, xa.err)) gave_up.sweep[c] = 1u;
+    if (!halo_wait(&hb, h, xa.err)) {
+      gave_up.sweep[c] = 1u;
+      halo_give_up(&hb);
+    }
   };
 
   auto update = [&](int g, int c, const RowWord (&rw)[NR], const Words4 &w, const float4 &h4, uint32_t hb, bool valid) {
@@ -238,9 +241,10 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
 
   const int n_iv = xa.enabled ? ba.n_iv : 1;
   uint32_t h = 0, sweep = sweep0;
+  bool gone = false;  // (all threads) this launch's results are not to be had
   for (int iv = 0; iv < n_iv; ++iv) {
     if (!ok || (kDebugBuild && stops_here(ba.stop, iv, xa.err))) {
-      gave_up.exchange = 1u;
+      gone = true;
       break;
     }
 #pragma unroll 1
@@ -282,7 +286,10 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
         }
       }
     }
-    if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) gave_up.exchange = 1u;
+    if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) {
+      gave_up.exchange = 1u;
+      halo_give_up(&hb);
+    }
     if (!xa.enabled) break;
 
     // ---- energies (Eq. 1): small replicas by one warp each, others by the whole CTA ---------------
@@ -351,13 +358,17 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     auto energy_of = [&](int B, long long F) {
       return -xa.J * (double)B - (BIM ? xa.h * (double)F : __longlong_as_double(F));
     };
-    if (!exchange_from_records<!BIM, false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, &gave_up.exchange, energy_of)) break;
+    if (!exchange_from_records<!BIM, false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, &gave_up.exchange, energy_of)) {
+      gone = true;
+      break;
+    }
     if (iv + 1 < n_iv) tab_fill_temps<BIM, false>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
-  __syncthreads();
-  const bool gone = gave_up.exchange != 0u;  // this launch's results are not to be had
-  if (S > 1) halo_leave(&hb, gone);
+  if (S > 1) {
+    if (gone) halo_give_up(&hb);
+    halo_leave(&hb);
+  }
   copy_planes(1, PZ, false);
   if (xa.enabled && !gone && blockIdx.x == 0)
     for (int r = tid; r < R; r += nt) {

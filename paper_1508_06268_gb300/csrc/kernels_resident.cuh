@@ -277,7 +277,10 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     }
   };
   auto wait_halos = [&](uint32_t h, int flag) {
-    if (!halo_wait(&hb, h, xa.err)) gave_up.sweep[flag] = 1u;
+    if (!halo_wait(&hb, h, xa.err)) {
+      gave_up.sweep[flag] = 1u;
+      halo_give_up(&hb);
+    }
   };
 
   bool valid;
@@ -302,9 +305,10 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
 
   const int n_iv = xa.enabled ? ra.n_iv : 1;
   uint32_t h = 0, sweep = sweep0;  // half-sweeps done in this launch; current sweep
+  bool gone = false;  // (all threads) this launch's results are not to be had
   for (int iv = 0; iv < n_iv; ++iv) {
     if (!ok || (kDebugBuild && stops_here(ra.stop, iv, xa.err))) {
-      gave_up.exchange = 1u;
+      gone = true;
       break;
     }
 #pragma unroll 1
@@ -389,7 +393,10 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
         ++h;
       }
     }
-    if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) gave_up.exchange = 1u;
+    if (S > 1 && (gave_up.sweep[0] || gave_up.sweep[1] || (h > 0 && !halo_wait(&hb, h - 1, xa.err)))) {
+      gave_up.exchange = 1u;
+      halo_give_up(&hb);
+    }
     if (!xa.enabled) break;
     const bool xi = XI && iv >= ra.xi_first;
     if (xi)
@@ -491,15 +498,19 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
       const double Fd = BIM ? xa.h * (double)F : (double)(2 * F - Htot) * fscale;
       return -xa.J * (double)B - Fd;
     };
-    if (!exchange_from_records<false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, &gave_up.exchange, energy_of)) break;
+    if (!exchange_from_records<false>(v, xa, xs, rec, S, epoch, xa.j + (uint32_t)iv, &gave_up.exchange, energy_of)) {
+      gone = true;
+      break;
+    }
     if (xi && blockIdx.x == 0)
       for (int k = tid; k < R; k += nt) ra.xi_t2r[(int64_t)iv * R + k] = xs.t2r[k];
     if (iv + 1 < n_iv) tab_fill_temps<BIM>(v, tab, slot0, gact, [&](int g) { return xs.r2t[r0 + g]; });
     __syncthreads();
   }
-  __syncthreads();
-  const bool gone = gave_up.exchange != 0u;  // this launch's results are not to be had
-  if (S > 1) halo_leave(&hb, gone);
+  if (S > 1) {
+    if (gone) halo_give_up(&hb);
+    halo_leave(&hb);
+  }
 
   for (int t = tid; ok && t < gact * 2 * WC; t += nt) {
     const int g = t / (2 * WC), rem = t % (2 * WC), c = rem / WC, wl = rem % WC;
