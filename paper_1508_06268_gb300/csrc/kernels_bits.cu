@@ -391,7 +391,9 @@ int make_bits_plan(int32_t L, int32_t Rcap, bool bimodal, BitsPlan *plan, std::s
   bool resident = false;
   double cycles = 0.0;
   if (L < 64) {
-    resident = resident_shape(L, Rcap, bimodal, &rs, &cycles);
+    // (int8 at L = 32: above 800 replicas the staged cluster kernel, us per 100 sweeps resident / staged: R = 800
+    // 2910 / 3053, 1000 3876 / 3786, 1500 5667 / 5337)
+    resident = !(i8 && L == 32 && Rcap > 800) && resident_shape(L, Rcap, bimodal, &rs, &cycles);
   } else if (!i8 && sms_dev > 0 && Rcap <= kResidentMaxR64) {
     const int units = ((Rcap + 3) / 4 * L + sms_dev - 1) / sms_dev;
     resident = resident_shape(L, Rcap, bimodal, &rs, &cycles) && cycles < 2070.0 * (5.2 + 0.76 * std::max(units, 3));
