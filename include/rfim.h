@@ -158,10 +158,11 @@ int rfim_set_measure_xi(rfim_ctx *ctx, int32_t on);
    (q >> 2, r, s mh + h mod 2^32, c3(METRO, stage, fine colour)), so counters repeat after
    2^32 / mh sweeps.  The paper keeps mh = 0 for its physics results; the multi-hit chain has the
    same Boltzmann law but other dynamics.  Bit layout only; tile in {8, 16, 32}, L in {16, 32, 64}
-   divisible by 2 tile.  When the current launch shape has no multi-hit kernel the context gets a
+   divisible by 2 tile, R_capacity >= 4 at L = 64.  When the current launch shape has no multi-hit kernel the context gets a
    resident shape for multi-hit sweeps beside it, or, where there is none or it would be slower (many
-   replicas at L = 64), switches to the default cluster shape of its L (synchronous in both cases).  Errors: RFIM_EINVAL (mh < 0, int8 layout, unsupported tile), RFIM_ENOMEM / RFIM_ECUDA
-   from the plan switch. */
+   replicas at L = 64), switches to the default cluster shape of its L (synchronous in both cases).  Errors: RFIM_EINVAL (mh < 0, int8
+   layout, unsupported tile), RFIM_ENOMEM / RFIM_ECUDA from the plan switch (RFIM_ECUDA also for fewer than four
+   replicas at L = 64). */
 int rfim_set_multihit(rfim_ctx *ctx, int32_t mh, int32_t tile);
 
 /* Thermal averages of one realization (Sec. 7) from its accumulators (obs as filled by

@@ -382,7 +382,9 @@ class Realization:
         self._check(self._lib.rfim_selftest_resident(self._h, stop_cta, stop_interval, number))
 
     def plan(self) -> str:
-        """Launch shape of the sweep kernel ("S,G,GT,threads[,4][,int8]"; "" for the int8 kernels)."""
+        """Launch shape of the sweep kernel: "S,G,GT,threads[,4][,int8]" for the cluster (S = 0: grid-wide)
+        kernels, "S,G,NB,threads,r[,int8]" (m: several items per thread) for the resident kernel, "S,G,4,threads,b"
+        for the resident kernel on bytes, "" for one int8 launch per half-sweep (rfim_get_plan)."""
         buf = C.create_string_buffer(64)
         self._check(self._lib.rfim_get_plan(self._h, buf, 64))
         return buf.value.decode()

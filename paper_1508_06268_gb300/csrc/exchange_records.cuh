@@ -137,7 +137,7 @@ __device__ __forceinline__ bool exchange_from_records(const RealView &v, const E
   // REAL: the 64-bit field sums are doubles.  Every CTA polls every record, so the lines they lie in
   // are what the step waits for: a warp's load takes each line once (a lane per replica that read
   // its S records one after another took it S times; L = 24, R = 40, eight slabs: 8.7 us for the
-  // whole tail of an interval, now 6.4).
+  // whole tail of an interval, 6.4 so, and 6.0 with the energies on bytes from registers as well).
   if (S == 1 || (S & (S - 1)) != 0) {  // one slab, or a number of slabs that no default shape has
     for (int r = tid; r < R; r += nt) {
       int B = 0, M = 0;

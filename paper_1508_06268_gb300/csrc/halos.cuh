@@ -25,8 +25,8 @@ constexpr unsigned kMbarSpinLimit = 1u << 20;
 
 // Waits of a CTA that were given up.  Half-sweeps (or tile visits) alternate between two flags: a thread that
 // reads one late, just before the next barrier, must not see what others set in the half-sweep after.
-// (L = 32, R = 70: 1.22 us per half-sweep, 1.20 with waits whose end nobody looks at; the flag read by every
-// thread instead took 1.27, __syncthreads_or instead of the flags 1.29.)
+// (L = 32, R = 70: 1.20 us per half-sweep, 1.18 with waits whose end nobody looks at; the flag read by every
+// thread instead took 1.25, __syncthreads_or instead of the flags 1.28.)
 struct GaveUp {
   uint32_t sweep[2], exchange;
 };
