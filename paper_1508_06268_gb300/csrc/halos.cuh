@@ -125,7 +125,8 @@ __device__ __forceinline__ void halo_drain(const HaloBars *hb, uint32_t mine, ui
   }
 }
 
-// A wait was given up (any thread, any number of them): every CTA of the cluster will know in halo_leave.
+// A wait of this CTA was given up (any thread, any number of them, before it leaves): every CTA of the cluster
+// will know in halo_leave.
 __device__ __forceinline__ void halo_give_up(HaloBars *hb) {
   const uint32_t flag = (uint32_t)__cvta_generic_to_shared(&hb->stopped);
   for (uint32_t q = 0; q < cluster_ctas(); ++q)

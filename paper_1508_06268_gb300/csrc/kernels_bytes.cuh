@@ -203,10 +203,7 @@ __global__ void __launch_bounds__(512, ONE && VW < 4 ? 1 : 2) k_resident_bytes(c
     }
   };
   auto wait_halos = [&](uint32_t h, int c) {
-    if (!halo_wait(&hb, h, xa.err)) {
-      gave_up.sweep[c] = 1u;
-      halo_give_up(&hb);
-    }
+    if (!halo_wait(&hb, h, xa.err)) gave_up.sweep[c] = 1u;  // (the cluster hears of it at the end of the interval)
   };
 
   auto update = [&](int g, int c, const RowWord (&rw)[NR], const Words4 &w, const float4 &h4, uint32_t hb, bool valid) {

@@ -277,10 +277,7 @@ __global__ void __launch_bounds__(NT) k_resident(const RealView v, const __grid_
     }
   };
   auto wait_halos = [&](uint32_t h, int flag) {
-    if (!halo_wait(&hb, h, xa.err)) {
-      gave_up.sweep[flag] = 1u;
-      halo_give_up(&hb);
-    }
+    if (!halo_wait(&hb, h, xa.err)) gave_up.sweep[flag] = 1u;  // (the cluster hears of it at the end of the interval)
   };
 
   bool valid;
